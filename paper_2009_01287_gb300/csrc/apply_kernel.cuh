@@ -170,14 +170,18 @@ struct ApplyArgs {
   const int64_t* off;
   const double* ih;           // 1 / h per element
   const double* aih;          // a / h per element (a: the diffusion coefficient)
-  const double* ahk;          // a h per element (cube meshes)
   const double* ak;           // a per element
   const int64_t* toff;        // offset of the element's side traces in tr
   double* tr;                 // side traces: [side][node][u, dn]
   const int32_t* sf_ptr;
   const SubFaceRec* sf;
   const SubFaceBr2* sfb;      // square meshes, BR2: the multiplied-out liftings
-  const SubFaceRec3* sf3;     // cube meshes
+  const SubFaceModal3* sfm3;  // cube meshes
+  const ElemRec3* erec3;
+  const int2* hang3;
+  const int4* side3;
+  double* xm;
+  int moff3[kMaxP + 1];
   const double* tab;          // basis + face tables
   const int32_t* order;       // degree-sorted element order
   const ApplyTile* tiles;

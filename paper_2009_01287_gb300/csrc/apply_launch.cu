@@ -29,6 +29,7 @@ __global__ void __launch_bounds__(kThreads) trace_kernel(const ApplyArgs A) {
 // (pcg_sc set, x = p, y = q) it also forms the step alpha = (r.z) / (p.q) once
 // for the kernels that apply the update r -= alpha q, x += alpha p (alpha = 0
 // once the solve has stopped: iterations queued after the stop change nothing).
+template <int NT>
 __device__ __forceinline__ void apply_exit(const ApplyArgs& A, double* red) {
   __shared__ unsigned s_last;
   pdl_trigger();   // this CTA's tiles are done: the next kernel may start launching
@@ -48,8 +49,8 @@ __device__ __forceinline__ void apply_exit(const ApplyArgs& A, double* red) {
     __threadfence();
     if (A.dot_partial) {
       double v = 0.0;
-      for (int i = threadIdx.x; i < A.n_tiles; i += kThreads) v += __ldcg(A.dot_partial + i);
-      v = block_sum<kThreads>(v, red);
+      for (int i = threadIdx.x; i < A.n_tiles; i += NT) v += __ldcg(A.dot_partial + i);
+      v = block_sum<NT>(v, red);
       if (threadIdx.x == 0) {
         *A.dot_out = v;
         if (A.pcg_sc) A.pcg_sc[SC_ALPHA] = status == 0.0 ? rz / v : 0.0;
@@ -93,7 +94,7 @@ __global__ void __launch_bounds__(kThreads) apply_kernel(const ApplyArgs A) {
     }
     __syncthreads();
   }
-  apply_exit(A, red);
+  apply_exit<kThreads>(A, red);
 }
 
 // Persistent operator kernel of mapped squares (same scheduling as on boxes).
@@ -123,31 +124,41 @@ __global__ void __launch_bounds__(kThreads) apply_map_kernel(const ApplyArgs A) 
     }
     __syncthreads();
   }
-  apply_exit(A, red);
+  apply_exit<kThreads>(A, red);
 }
 
-__global__ void __launch_bounds__(kThreads) trace3_kernel(const ApplyArgs A) {
+// Modes and side traces of x on cube meshes.  UPDATE (inside PCG): p = z +
+// beta p (first: p = z, and the initial scalars and loop condition) takes the
+// place of x.
+template <bool UPDATE>
+__global__ void __launch_bounds__(kThreads3)
+modal3_kernel(const ApplyArgs A, double* p, const double* z, double* sc, cudaGraphConditionalHandle h,
+              int use_cond, int first) {
   pdl_entry();
+  extern __shared__ __align__(16) double smem[];
+  double beta = 0.0;
+  if (UPDATE) {
+    if (!first && sc[SC_STATUS] != 0.0) return;   // stopped: the loop condition is already clear
+    if (!first) beta = sc[SC_BETA];
+  }
   const ApplyTile T = A.tiles[blockIdx.x];
   switch (T.p) {
-    case 1: trace3_tile<1>(A, T); break;
-    case 2: trace3_tile<2>(A, T); break;
-    case 3: trace3_tile<3>(A, T); break;
-    case 4: trace3_tile<4>(A, T); break;
-    case 5: trace3_tile<5>(A, T); break;
-    case 6: trace3_tile<6>(A, T); break;
-    case 7: trace3_tile<7>(A, T); break;
-    case 8: trace3_tile<8>(A, T); break;
+#define DG_MODAL_CASE(PP) \
+    case PP: modal3_tile<PP, UPDATE>(A, T, smem, p, z, beta, first != 0); break;
+    DG_MODAL_CASE(1) DG_MODAL_CASE(2) DG_MODAL_CASE(3) DG_MODAL_CASE(4)
+    DG_MODAL_CASE(5) DG_MODAL_CASE(6) DG_MODAL_CASE(7) DG_MODAL_CASE(8)
+#undef DG_MODAL_CASE
     default: break;
   }
+  if (UPDATE && first) pcg_first_scalars(sc, h, use_cond);
 }
 
 // Persistent operator kernel of cube meshes (same scheduling as on squares).
 template <bool BR2>
-__global__ void __launch_bounds__(kThreads) apply3_kernel(const ApplyArgs A) {
+__global__ void __launch_bounds__(kThreads3) apply3_kernel(const ApplyArgs A) {
   pdl_entry();
   extern __shared__ __align__(16) double smem[];
-  __shared__ double red[kThreads];
+  __shared__ double red[kThreads3];
   __shared__ int s_tile;
   while (true) {
     if (threadIdx.x == 0) s_tile = (int)atomicAdd(A.sched, 1u);
@@ -169,7 +180,7 @@ __global__ void __launch_bounds__(kThreads) apply3_kernel(const ApplyArgs A) {
     }
     __syncthreads();
   }
-  apply_exit(A, red);
+  apply_exit<kThreads3>(A, red);
 }
 
 // static shared-memory layout of a degree-p tile up to the item partials (doubles)
@@ -228,14 +239,18 @@ ApplyArgs make_apply_args(const dg_mesh& M, const double* x, double* y, Reduce r
   A.off = M.d_off;
   A.ih = M.d_ih;
   A.aih = M.d_aih;
-  A.ahk = M.d_ahk;
   A.ak = M.d_ak;
   A.toff = M.d_toff;
   A.tr = M.d_tr;
   A.sf_ptr = M.d_sf_ptr;
   A.sf = M.d_sf;
   A.sfb = M.d_sfb;
-  A.sf3 = M.d_sf3;
+  A.sfm3 = M.d_sfm3;
+  A.erec3 = M.d_erec3;
+  A.hang3 = reinterpret_cast<const int2*>(M.d_hang3);
+  A.side3 = reinterpret_cast<const int4*>(M.d_side3);
+  A.xm = M.d_xm;
+  for (int p = 0; p <= kMaxP; ++p) A.moff3[p] = M.moff3[p];
   A.tab = M.d_tables;
   A.order = M.d_order;
   A.tiles = M.d_tiles;
@@ -275,11 +290,13 @@ int apply_kernel_setup(const dg_mesh& M) {
   const bool br2 = M.opts.form == DG_FORM_BR2;
   if (M.host.dim == 3) {
     const int smem = (int)M.apply3_smem;
-    DG_REQUIRE(smem <= optin, "operator tile needs too much shared memory");
+    DG_REQUIRE(smem <= optin && M.modal3_smem <= optin, "operator tile needs too much shared memory");
+    DG_CUDA(cudaFuncSetAttribute(modal3_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
+    DG_CUDA(cudaFuncSetAttribute(modal3_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
     DG_CUDA(cudaFuncSetAttribute(apply3_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
     DG_CUDA(cudaFuncSetAttribute(apply3_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    if (br2) DG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, apply3_kernel<true>, kThreads, smem));
-    else DG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, apply3_kernel<false>, kThreads, smem));
+    if (br2) DG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, apply3_kernel<true>, kThreads3, smem));
+    else DG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, apply3_kernel<false>, kThreads3, smem));
     return sms * (per > 0 ? per : 1);
   }
   const int smem = (int)M.apply_smem;
@@ -300,10 +317,15 @@ int apply_kernel_setup(const dg_mesh& M) {
   return sms * (per > 0 ? per : 1);
 }
 
+static void launch_modal3(const dg_mesh& M, const ApplyArgs& A, cudaStream_t s) {
+  launch_k(modal3_kernel<false>, M.n_tiles, kThreads3, (size_t)M.modal3_smem, s, A, (double*)nullptr,
+           (const double*)nullptr, (double*)nullptr, (cudaGraphConditionalHandle)0, 0, 0);
+}
+
 void launch_trace(const dg_mesh& M, const double* x, cudaStream_t s) {
   if (M.n_tiles == 0) return;
   const ApplyArgs A = make_apply_args(M, x, nullptr, Reduce{});
-  if (M.host.dim == 3) launch_k(trace3_kernel, M.n_tiles, kThreads, 0, s, A);
+  if (M.host.dim == 3) launch_modal3(M, A, s);
   else launch_k(trace_kernel, M.n_tiles, kThreads, 0, s, A);
   DG_CUDA(cudaGetLastError());
 }
@@ -316,10 +338,10 @@ void launch_apply(const dg_mesh& M, const double* x, double* y, Reduce red, cuda
   A.pcg_sc = pcg_sc;
   const int grid = M.n_tiles < M.apply_grid ? M.n_tiles : M.apply_grid;
   if (M.host.dim == 3) {
-    if (with_trace) launch_k(trace3_kernel, M.n_tiles, kThreads, 0, s, A);
+    if (with_trace) launch_modal3(M, A, s);
     const int smem3 = (int)M.apply3_smem;
-    if (M.opts.form == DG_FORM_BR2) launch_k(apply3_kernel<true>, grid, kThreads, smem3, s, A);
-    else launch_k(apply3_kernel<false>, grid, kThreads, smem3, s, A);
+    if (M.opts.form == DG_FORM_BR2) launch_k(apply3_kernel<true>, grid, kThreads3, smem3, s, A);
+    else launch_k(apply3_kernel<false>, grid, kThreads3, smem3, s, A);
     DG_CUDA(cudaGetLastError());
     return;
   }
@@ -331,6 +353,14 @@ void launch_apply(const dg_mesh& M, const double* x, double* y, Reduce red, cuda
   }
   else if (M.opts.form == DG_FORM_BR2) launch_k(apply_kernel<true>, grid, kThreads, smem, s, A);
   else launch_k(apply_kernel<false>, grid, kThreads, smem, s, A);
+  DG_CUDA(cudaGetLastError());
+}
+
+void launch_modal3_update(const dg_mesh& M, double* p, const double* z, double* sc,
+                          unsigned long long cond_handle, int use_cond, int first, cudaStream_t s) {
+  const ApplyArgs A = make_apply_args(M, p, nullptr, Reduce{});
+  launch_k(modal3_kernel<true>, M.n_tiles, kThreads3, (size_t)M.modal3_smem, s, A, p, z, sc,
+           (cudaGraphConditionalHandle)cond_handle, use_cond, first);
   DG_CUDA(cudaGetLastError());
 }
 

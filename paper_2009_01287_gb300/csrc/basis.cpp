@@ -1,5 +1,6 @@
 // Host 1D polynomial machinery: Gauss-Lobatto nodes (Section 2.2), Gauss
 // rules and Lagrange values for the setup of the device tables.
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 
@@ -182,6 +183,55 @@ Basis1D make_basis(int p) {
 }
 
 }  // namespace
+
+// phi_k(t), k = 0..n-1
+static void legendre_modes(int n, double t, double* out) {
+  for (int k = 0; k < n; ++k) {
+    double pk, pk1;
+    legendre(k, 2.0 * t - 1.0, pk, pk1);
+    out[k] = std::sqrt(2.0 * k + 1.0) * (k == 0 ? 1.0 : pk);
+  }
+}
+
+void modal_tables(int p, std::vector<double>& out) {
+  const int n = p + 1, H = n / 2, HC = (n + 1) / 2;
+  // mode k of the nodal basis function i: int phi_k l_i, exact with n Gauss points
+  const Basis1D& b = basis1d(p);
+  std::vector<double> gx, gw, l(n), f(n), W((size_t)n * n, 0.0);
+  gauss_rule(n, gx, gw);
+  for (int g = 0; g < n; ++g) {
+    lagrange_eval(b.nodes, gx[g], l.data());
+    legendre_modes(n, gx[g], f.data());
+    for (int k = 0; k < n; ++k)
+      for (int i = 0; i < n; ++i) W[k * n + i] += gw[g] * f[k] * l[i];
+  }
+  for (int a = 0; a < HC; ++a)
+    for (int i = 0; i < HC; ++i) out.push_back(0.5 * (W[2 * a * n + i] + W[2 * a * n + p - i]));
+  for (int a = 0; a < H; ++a)
+    for (int i = 0; i < H; ++i) out.push_back(0.5 * (W[(2 * a + 1) * n + i] - W[(2 * a + 1) * n + p - i]));
+  auto s = [](int k) { return std::sqrt(2.0 * k + 1.0); };
+  for (int k = 0; k < n; ++k)
+    for (int m = 0; m < n; ++m) {
+      const int lo = std::min(k, m);
+      out.push_back((k + m) % 2 == 0 ? 2.0 * s(k) * s(m) * lo * (lo + 1.0) : 0.0);
+    }
+  for (int k = 0; k < n; ++k) out.push_back(s(k));
+  for (int k = 0; k < n; ++k) out.push_back(s(k) * k * (k + 1.0));
+}
+
+void modal_restriction(int L, int o, double* R) {
+  std::vector<double> gx, gw;
+  gauss_rule(kMaxN, gx, gw);
+  std::fill(R, R + kMaxN * kMaxN, 0.0);
+  double fine[kMaxN], coarse[kMaxN];
+  const double scale = 1.0 / (double)(1LL << L);
+  for (int g = 0; g < kMaxN; ++g) {
+    legendre_modes(kMaxN, gx[g], fine);
+    legendre_modes(kMaxN, (o + gx[g]) * scale, coarse);
+    for (int k = 0; k < kMaxN; ++k)
+      for (int m = k; m < kMaxN; ++m) R[k * kMaxN + m] += gw[g] * fine[k] * coarse[m];
+  }
+}
 
 const Basis1D& basis1d(int p) {
   static std::once_flag once;

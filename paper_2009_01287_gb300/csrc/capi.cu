@@ -53,6 +53,12 @@ void upload_tiles(dg_mesh* M, cudaStream_t s) {
   M->d_items = a.upload(M->h_items, s);
   M->d_item_ptr = a.upload(M->h_item_ptr, s);
   M->d_side_items = a.upload(M->h_side_items, s);
+  if (M->host.dim == 3) {
+    M->d_sfm3 = a.upload(M->h_sfm3, s);
+    M->d_erec3 = a.upload(M->h_erec3, s);
+    M->d_hang3 = a.upload(M->h_hang3, s);
+    M->d_side3 = a.upload(M->h_side3, s);
+  }
   DG_CUDA(cudaStreamSynchronize(s));
 }
 
@@ -63,26 +69,28 @@ void upload_mesh(dg_mesh* M, cudaStream_t s) {
   M->d_p = a.upload(m.p, s);
   M->d_off = a.upload(m.off, s);
   {
-    std::vector<double> ih(m.n), aih(m.n), ahk(m.n);
+    std::vector<double> ih(m.n), aih(m.n);
     std::vector<int64_t> toff(m.n + 1, 0);
     for (int64_t k = 0; k < m.n; ++k) {
       ih[k] = 1.0 / M->h_h[k];
       aih[k] = m.coef[k] / M->h_h[k];
-      ahk[k] = m.coef[k] * M->h_h[k];
       const int64_t np = m.p[k] + 1;
-      toff[k + 1] = toff[k] + (m.dim == 3 ? 12 * np * np : 8 * np);
+      toff[k + 1] = toff[k] + 8 * np;
     }
     M->d_ih = a.upload(ih, s);
     M->d_aih = a.upload(aih, s);
-    M->d_ahk = a.upload(ahk, s);
     M->d_ak = a.upload(m.coef, s);
-    M->d_toff = a.upload(toff, s);
-    M->d_tr = a.alloc<double>(toff[m.n]);
+    if (m.dim == 3) {
+      M->d_tr = a.alloc<double>(2 * M->n_trace3);
+      M->d_xm = a.alloc<double>(M->n_dofs);
+    } else {
+      M->d_toff = a.upload(toff, s);
+      M->d_tr = a.alloc<double>(toff[m.n]);
+    }
   }
   M->d_sf_ptr = a.upload(m.sf_ptr, s);
   M->d_sf = a.upload(M->h_sf, s);
   M->d_sfb = M->h_sfb.empty() ? nullptr : a.upload(M->h_sfb, s);
-  M->d_sf3 = a.upload(M->h_sf3, s);
   if (m.mapped) {
     M->d_sfm = a.upload(M->h_sfm, s);
     M->d_gvol = a.upload(M->h_gvol, s);

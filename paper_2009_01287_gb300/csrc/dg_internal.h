@@ -17,7 +17,8 @@ namespace dg {
 
 constexpr int kMaxP = 8;
 constexpr int kMaxN = kMaxP + 1;
-constexpr int kThreads = 256;   // threads per CTA of the operator kernel
+constexpr int kThreads = 256;   // threads per CTA of the operator kernel on squares
+constexpr int kThreads3 = 128;  // and of its two kernels on cubes
 // elements of degree p per operator CTA (one thread per node, at most 16)
 constexpr int apply_epb(int p) {
   return (kThreads / ((p + 1) * (p + 1))) > 16 ? 16 : (kThreads / ((p + 1) * (p + 1)));
@@ -98,31 +99,57 @@ struct SubFaceRec3 {
   int32_t tab_oo[2]; // own-own 1D face mass per tangential axis ((p+1)^2)
   int32_t tab_on[2]; // own-neighbour ((p+1) x (pn+1))
   int32_t tab_nn[2]; // neighbour-neighbour ((pn+1)^2)
-  // BR2 lifting products per tangential axis (Minv: 1D mass inverse):
-  //   Z = M_oo Minv M_oo, V = M_oo Minv M_on, X = M_on Minv_n M_no, Y = M_on Minv_n M_nn
-  // (on a whole own face M_oo is the 1D mass matrix, so Z = M_oo and V = M_on;
-  // on a whole neighbour face likewise Y = M_on)
-  int32_t tab_z[2], tab_v[2], tab_x[2], tab_y[2];
   double sigma;      // SIPG penalty
   double area;       // physical area of the sub-face
-  double cz, cx;     // BR2: a eta coef area^2 Minv_00 / h^3 of the own / neighbour element,
-                     // a the larger coefficient of the sub-face's two sides
+};
+
+// The same sub-face as the kernels read it, in the Legendre modes of its two
+// sides (records in tile order: by element of the tile, side and sub-face).
+// In the orthonormal modes of the sub-face itself, with J = u- - u+ and
+// F = dn- - dn+ (both sides' outward derivatives), the residual over a h is
+//   r = cz J + cf F + (BR2) the two liftings,  c2 = cc J,
+// both returned to the own side's modes through R^T when it is larger.
+struct SubFaceModal3 {
+  int32_t nb;        // neighbour element, -1 on the boundary
+  int32_t pn;        // neighbour degree
+  int32_t nbr_off;   // the other side's trace on the sub-face (double2 units in the trace buffer)
+  int32_t own_off;   // the own trace on the sub-face
+  int32_t tab_ra, tab_rb;   // larger own side: R per tangential axis (rows of kMaxN)
+  int32_t tab_sa, tab_sb;   // BR2, hanging: S = R R^T of the larger side's degree
+  double cz;         // SIPG: sigma area; BR2: the own lifting's factor
+  double cx;         // BR2: the neighbour lifting's factor
+  double czx;        // factor of J on modes both sides have (whole faces of both: cz + cx, else cz)
+  double cf, cc;
+};
+// per element in tile order
+struct ElemRec3 {
+  int64_t off;       // first DOF
+  int32_t toff;      // its six side traces (double2 units)
+  int32_t pad;
+  double ah, aih;    // a h, a / h
 };
 
 // Shared-memory budget (doubles) of one 3D operator tile; the host sizes the
-// tiles and their sub-face item chunks so that every one fits.
+// tiles and their rounds of hanging sub-faces so that every one fits.
 constexpr int kApply3Budget = 9 * 1024;
-constexpr int kApply3MinChunk = 12;   // sub-face items a tile keeps room for
-// doubles of shared memory one element of degree p needs in a 3D tile (volume
-// passes and the per-side residual and normal-derivative coefficients)
+// elements of degree p a tile takes at most: about one line of nodes (or
+// modes) per thread of the CTA in every volume pass, whole warps of them
+constexpr int apply3_epb(int p) {
+  return p == 1 ? 16 : p == 2 ? 14 : p == 3 ? 8 : p == 4 ? 5 : p == 5 ? 3 : p == 6 ? 2 : p == 7 ? 2 : 1;
+}
+// doubles of a degree's modal tables (Modal3)
+constexpr int modal3_doubles(int p) {
+  return ((p + 2) / 2) * ((p + 2) / 2) + ((p + 1) / 2) * ((p + 1) / 2) + (p + 1) * (p + 1) + 2 * (p + 1);
+}
+// doubles of shared memory one element of degree p needs in a 3D tile (its
+// modes, its residual and the residuals of its sides)
 constexpr int apply3_elem_doubles(int p) {
-  return 5 * (p + 1) * (p + 1) * (p + 1) + 12 * (p + 1) * (p + 1);
+  return 2 * (p + 1) * (p + 1) * (p + 1) + 12 * (p + 1) * (p + 1);
 }
-// doubles one sub-face item needs: first-pass scratch ((p+1) x nq per product,
-// nq = max(p, pn) + 1) and its two partial side arrays
-constexpr int apply3_item_doubles(int p, int nq, bool br2) {
-  return (br2 ? 8 : 4) * (p + 1) * nq + 2 * (p + 1) * (p + 1);
-}
+// doubles per sub-face smaller than the own side, and per sub-face of a larger
+// neighbour (BR2; nq = the tile's largest neighbour degree or its own, plus 1)
+constexpr int apply3_own_doubles(int p) { return 4 * (p + 1) * (p + 1); }
+constexpr int apply3_nbr_doubles(int p, int nq) { return nq * nq + (p + 1) * nq; }
 
 // Offsets of the degree-p 1D matrices inside the device table buffer.
 struct BasisOff {
@@ -136,7 +163,10 @@ struct ApplyTile {
   int32_t count;
   int32_t inst;      // batch instance of the tile's elements (0 for a single mesh)
   int32_t nq;        // 3D: max(p, neighbour degrees) + 1 over the tile
-  int32_t chunk;     // 3D: sub-face items processed at a time
+  int32_t chunk;     // 3D: sub-face items sorted together (the whole tile)
+  int32_t hang;      // 3D: first entry of the tile's hanging sub-faces
+  int32_t n_c, n_b;  // 3D: sub-faces smaller than the own side; then, BR2, of larger neighbours
+  int32_t cap_c, cap_b;   // 3D: how many of each a round takes
 };
 
 // ------------------------------------------------------------------ mapped squares
@@ -260,6 +290,14 @@ inline void side_axes3(int s, int& ax, int& t0, int& t1) {
   t0 = (ax == 0) ? 1 : 0;
   t1 = (ax == 2) ? 1 : 2;
 }
+
+// Orthonormal Legendre modes phi_k = sqrt(2k+1) P_k(2t-1) on [0, 1] (3D
+// operator).  modal_tables appends a degree's tables: node -> mode, even modes
+// by sums of mirrored nodes and odd modes by differences; the 1D stiffness;
+// phi_k(1) and phi_k'(1).  modal_restriction: R_km (kMaxN x kMaxN, zero for
+// k > m) with phi_m((o + s) / 2^L) = sum_k R_km phi_k(s).
+void modal_tables(int p, std::vector<double>& out);
+void modal_restriction(int L, int o, double* R);
 
 // Face-mass tables (Section 2: exact face integrals on sub-faces).
 struct FaceTables {

@@ -114,6 +114,20 @@ struct dg_mesh {
   std::vector<dg::SubFaceRec> h_sf;
   std::vector<dg::SubFaceBr2> h_sfb;    // square meshes, BR2: one per h_sf record
   std::vector<dg::SubFaceRec3> h_sf3;   // cube meshes
+  // cube meshes, for the kernels: the sub-face records in tile order, element
+  // records in tile order, per tile its hanging sub-faces (record, local
+  // element * 6 + side), per (order position, side) {first record, first
+  // hanging entry of the tile, their count or 0, 0}
+  std::vector<dg::SubFaceModal3> h_sfm3;
+  std::vector<dg::ElemRec3> h_erec3;
+  std::vector<int32_t> h_hang3;
+  std::vector<int32_t> h_side3;
+  int moff3[dg::kMaxP + 1] = {0};       // modal tables of each degree in h_tables
+  std::vector<int32_t> h_toff3;         // cube meshes: trace offset of every element (double2 units)
+  std::vector<int32_t> h_suboff3;       // trace offset per record on a larger own side, else -1
+  std::vector<int32_t> h_rtab3;         // per record {R_a, R_b, S_a, S_b} table offsets of the larger side
+  int64_t n_trace3 = 0;                 // length of the trace buffer (double2)
+  int64_t modal3_smem = 0;              // dynamic shared memory of the modes / traces kernel
   // mapped squares: one record per h_sf record, the volume tables of each
   // degree, the map; the geometric factors at the Gauss points - per element
   // (offset h_goff[k]) the volume factors a w_g w_h G of its (p+2)^2 points as
@@ -165,14 +179,17 @@ struct dg_mesh {
   int64_t* d_off = nullptr;
   double* d_ih = nullptr;       // 1 / h
   double* d_aih = nullptr;      // a / h (normal derivatives of traces and test functions)
-  double* d_ahk = nullptr;      // a h (volume term on cubes)
   double* d_ak = nullptr;       // a
   int64_t* d_toff = nullptr;    // side-trace offsets (8 (p+1) doubles per element)
   double* d_tr = nullptr;       // side traces written by each apply
   int32_t* d_sf_ptr = nullptr;
   dg::SubFaceRec* d_sf = nullptr;
   dg::SubFaceBr2* d_sfb = nullptr;
-  dg::SubFaceRec3* d_sf3 = nullptr;
+  dg::SubFaceModal3* d_sfm3 = nullptr;   // cube meshes
+  dg::ElemRec3* d_erec3 = nullptr;
+  int32_t* d_hang3 = nullptr;
+  int32_t* d_side3 = nullptr;
+  double* d_xm = nullptr;       // cube meshes: modes of the operator's argument
   dg::SubFaceMap* d_sfm = nullptr;   // mapped squares
   double* d_gvol = nullptr;          // mapped squares: geometric factors (h_gvol, h_goff, h_gface)
   int64_t* d_goff = nullptr;

@@ -641,11 +641,10 @@ void launch_pcg_init(const double* b, double* x, double* r, int64_t n, Reduce bb
 }
 
 // p = z + beta p (first: p = z) tile by tile, and the side traces of the new p
-// for the next operator apply, so the apply needs no trace launch of its own.
-// The last CTA to finish advances the iteration count and the scalars, tests
-// convergence and sets the graph's while condition (first: the initial
-// scalars, from the preconditioner's r . z and b . b).
-template <bool CUBE>
+// for the next operator apply, so the apply needs no trace launch of its own
+// (squares; modal3_kernel does the same on cubes).  The last CTA of the
+// preconditioner's final kernel has advanced the scalars and tested
+// convergence (first: the initial scalars are set here).
 __global__ void __launch_bounds__(kThreads)
 pcg_p_trace_kernel(const ApplyArgs A, double* __restrict__ p, const double* __restrict__ z, double* sc,
                    cudaGraphConditionalHandle h, int use_cond, int first) {
@@ -654,7 +653,7 @@ pcg_p_trace_kernel(const ApplyArgs A, double* __restrict__ p, const double* __re
   const double beta = first ? 0.0 : sc[SC_BETA];
   const ApplyTile T = A.tiles[blockIdx.x];
   const int np = T.p + 1;
-  const int nn = CUBE ? np * np * np : np * np;
+  const int nn = np * np;
   for (int t = threadIdx.x; t < T.count * nn; t += blockDim.x) {
     const int e = t / nn;
     const int64_t i = A.off[A.order[T.first + e]] + (t - e * nn);
@@ -663,32 +662,25 @@ pcg_p_trace_kernel(const ApplyArgs A, double* __restrict__ p, const double* __re
   __syncthreads();
   switch (T.p) {
 #define DG_TRACE_CASE(PP) \
-    case PP: if (CUBE) trace3_tile<PP, false>(A, T); else trace_tile<PP, false>(A, T); break;
+    case PP: trace_tile<PP, false>(A, T); break;
     DG_TRACE_CASE(1) DG_TRACE_CASE(2) DG_TRACE_CASE(3) DG_TRACE_CASE(4)
     DG_TRACE_CASE(5) DG_TRACE_CASE(6) DG_TRACE_CASE(7) DG_TRACE_CASE(8)
 #undef DG_TRACE_CASE
     default: break;
   }
-  if (first && blockIdx.x == 0 && threadIdx.x == 0) {
-    sc[SC_RZ] = sc[SC_RZNEW];
-    sc[SC_RR] = sc[SC_BB];
-    sc[SC_IT] = 0.0;
-    sc[SC_STATUS] = 0.0;
-    // a zero right-hand side needs no iteration (x = 0 is exact)
-    if (use_cond) cudaGraphSetConditional(h, sc[SC_BB] > 0.0 ? 1u : 0u);
-  }
+  if (first) pcg_first_scalars(sc, h, use_cond);
 }
 
 void launch_pcg_p_trace(const dg_mesh& M, double* p, const double* z, double* sc,
                         unsigned long long cond_handle, int use_cond, int first, cudaStream_t s) {
   if (M.n_tiles == 0) return;
+  if (M.host.dim == 3) {
+    launch_modal3_update(M, p, z, sc, cond_handle, use_cond, first, s);
+    return;
+  }
   const ApplyArgs A = make_apply_args(M, p, nullptr, Reduce{});
-  if (M.host.dim == 3)
-    launch_k(pcg_p_trace_kernel<true>, M.n_tiles, kThreads, 0, s, A, p, z, sc,
-             (cudaGraphConditionalHandle)cond_handle, use_cond, first);
-  else
-    launch_k(pcg_p_trace_kernel<false>, M.n_tiles, kThreads, 0, s, A, p, z, sc,
-             (cudaGraphConditionalHandle)cond_handle, use_cond, first);
+  launch_k(pcg_p_trace_kernel, M.n_tiles, kThreads, 0, s, A, p, z, sc,
+           (cudaGraphConditionalHandle)cond_handle, use_cond, first);
   DG_CUDA(cudaGetLastError());
 }
 

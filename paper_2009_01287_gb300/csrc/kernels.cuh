@@ -46,6 +46,18 @@ struct PcgCtl {
   unsigned long long cond = 0;      // cudaGraphConditionalHandle
   int use_cond = 0;
 };
+// the scalars a PCG solve starts from and, with use_cond, the loop condition
+// (by one thread of the kernel that forms the first p)
+__device__ __forceinline__ void pcg_first_scalars(double* sc, cudaGraphConditionalHandle h, int use_cond) {
+  if (blockIdx.x != 0 || threadIdx.x != 0) return;
+  sc[SC_RZ] = sc[SC_RZNEW];
+  sc[SC_RR] = sc[SC_BB];
+  sc[SC_IT] = 0.0;
+  sc[SC_STATUS] = 0.0;
+  // a zero right-hand side needs no iteration (x = 0 is exact)
+  if (use_cond) cudaGraphSetConditional(h, sc[SC_BB] > 0.0 ? 1u : 0u);
+}
+
 // Events recorded between the parts of a preconditioner apply: ev[0] start,
 // ev[1] after the block solves, ev[2] after the restriction, ev[3] after the
 // LOR solve, ev[4] after the final combination.  With marks the block solves
@@ -81,6 +93,10 @@ int precond_final_blocks(const dg_precond& pc);
 int precond_kernel_count(const dg_precond& pc);
 
 enum { TK_PQ = 0, TK_RR = 1, TK_RZ = 2, TK_P = 3, TK_BB = 4, TK_COUNT = 8 };
+
+// its form on cube meshes (modes and traces of the new p)
+void launch_modal3_update(const dg_mesh& M, double* p, const double* z, double* sc,
+                          unsigned long long cond_handle, int use_cond, int first, cudaStream_t s);
 
 void launch_pcg_init(const double* b, double* x, double* r, int64_t n, Reduce bb, cudaStream_t s);
 // p = z + beta p (first: p = z and the initial scalars) tile by tile, writing

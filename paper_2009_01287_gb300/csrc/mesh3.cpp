@@ -112,24 +112,24 @@ void build_topology3(HostMesh& m) {
   }
 }
 
-// degree-sorted element order and tiles of the 3D operator kernel.  Elements
+// degree-sorted element order and tiles of the 3D operator kernels.  Elements
 // are sorted by (p, nq), descending, nq = max(p, neighbour degrees) + 1; a tile
-// is a run of equal (p, nq) with as many elements as fill 256 threads while the
-// volume and side arrays leave room for a chunk of at least kApply3MinChunk
-// sub-face items.  The tile's sub-faces are a flat list of (record, side)
-// items, processed in chunks that fit the shared-memory budget; per element
-// side the first item and the count.
+// is a run of equal (p, nq) with at most apply3_epb(p) elements (fewer on small
+// meshes, so that two tiles fall to every SM) while its arrays leave room for a
+// round of at least one hanging sub-face of each kind.  The tile's sub-faces
+// are a flat list of (record, side) items; those whose larger side is the
+// element's own or (BR2) the neighbour's make the tile's hanging lists, which
+// the operator kernel takes in rounds that fit the shared-memory budget.
 void build_tiles3(dg_mesh* M) {
   const HostMesh& m = M->host;
   const bool br2 = M->opts.form == DG_FORM_BR2;
-  std::vector<int32_t> nq(m.n), nitem(m.n);
+  std::vector<int32_t> nq(m.n);
   for (int64_t k = 0; k < m.n; ++k) {
     int q = m.p[k] + 1;
     const int b = m.sf_ptr[6 * k], e = m.sf_ptr[6 * k + 6];
     for (int j = b; j < e; ++j)
       if (m.sf3[j].nb >= 0) q = std::max(q, m.p[m.sf3[j].nb] + 1);
     nq[k] = q;
-    nitem[k] = e - b;
   }
   std::vector<int32_t> order(m.n);
   for (int64_t k = 0; k < m.n; ++k) order[k] = (int32_t)k;
@@ -137,86 +137,232 @@ void build_tiles3(dg_mesh* M) {
     if (m.p[a] != m.p[b]) return m.p[a] > m.p[b];
     return nq[a] > nq[b];
   });
+  // elements per tile: halved while the mesh gives fewer tiles than two per SM
+  int epb[kMaxP + 1], div = 1;
+  for (;; div *= 2) {
+    int64_t cnt[kMaxP + 1] = {0}, tiles = 0;
+    for (int64_t k = 0; k < m.n; ++k) ++cnt[m.p[k]];
+    bool more = false;
+    for (int p = 1; p <= kMaxP; ++p) {
+      epb[p] = std::max(1, apply3_epb(p) / div);
+      more = more || (cnt[p] > 0 && epb[p] > 1);
+      tiles += (cnt[p] + epb[p] - 1) / epb[p];
+    }
+    if (tiles >= 304 || !more) break;
+  }
   M->h_tiles.clear();
   M->h_items.clear();
   M->h_item_ptr.assign(1, 0);
   M->h_side_items.assign(12 * (size_t)m.n, 0);
+  M->h_sfm3.clear();
+  M->h_erec3.clear();
+  M->h_hang3.clear();
+  M->h_side3.assign(24 * (size_t)m.n, 0);
   M->apply3_smem = 0;
+  M->modal3_smem = 0;
   for (int64_t i = 0; i < m.n;) {
-    const int P = m.p[order[i]], Q = nq[order[i]], NP = P + 1;
+    const int P = m.p[order[i]], Q = nq[order[i]], N2 = (P + 1) * (P + 1);
     const int fixed_per = apply3_elem_doubles(P);
-    const int item_per = apply3_item_doubles(P, Q, br2);
-    const int by_threads = std::max(1, kThreads / (NP * NP * NP));
-    int64_t j = i, items = 0;
-    while (j < m.n && m.p[order[j]] == P && nq[order[j]] == Q && j - i < by_threads) {
-      const int64_t cnt = j - i + 1, it = items + nitem[order[j]];
-      const int64_t need = 2 * NP * NP + cnt * fixed_per + std::min<int64_t>(it, kApply3MinChunk) * item_per;
+    const int own_per = apply3_own_doubles(P), nbr_per = apply3_nbr_doubles(P, Q);
+    int64_t j = i;
+    while (j < m.n && m.p[order[j]] == P && nq[order[j]] == Q && j - i < epb[P]) {
+      const int64_t need = modal3_doubles(P) + (j - i + 1) * fixed_per + own_per + nbr_per;
       if (need > M->apply3_budget && j > i) break;
-      items = it;
       ++j;
     }
-    const int64_t fixed = 2 * NP * NP + (j - i) * fixed_per;
-    const int64_t room = (M->apply3_budget - fixed) / item_per;
-    DG_REQUIRE(room >= 1, "3D operator tile does not fit in shared memory");
     ApplyTile T{};
     T.p = P;
     T.first = (int32_t)i;
     T.count = (int32_t)(j - i);
     T.nq = Q;
-    T.chunk = (int32_t)std::min<int64_t>(items, room);
+    T.hang = (int32_t)(M->h_hang3.size() / 2);
+    std::vector<std::pair<int32_t, int32_t>> own, nbr;   // (record, side) of the hanging lists
     for (int64_t e = 0; e < T.count; ++e) {
       const int64_t pos = i + e;
       const int32_t k = order[pos];
+      const double a = m.coef[k], h = M->h_h[k];
+      M->h_erec3.push_back({m.off[k], M->h_toff3[k], 0, a * h, a / h});
       for (int s = 0; s < 6; ++s) {
         const int b = m.sf_ptr[6 * (int64_t)k + s], c = m.sf_ptr[6 * (int64_t)k + s + 1] - b;
         M->h_side_items[12 * pos + 2 * s] = (int32_t)(M->h_items.size() / 2);
         M->h_side_items[12 * pos + 2 * s + 1] = c;
+        int32_t* sd = &M->h_side3[24 * pos + 4 * s];
+        sd[0] = (int32_t)M->h_sfm3.size();
+        sd[1] = (int32_t)own.size();
+        sd[2] = 0;
         for (int q = 0; q < c; ++q) {
           M->h_items.push_back(b + q);
           M->h_items.push_back((int32_t)(6 * e + s));
+          const SubFaceRec3& f = M->h_sf3[b + q];
+          const int32_t es = (int32_t)(6 * e + s), rec = (int32_t)M->h_sfm3.size();
+          const bool in = f.nb >= 0, mine = !(f.full & 1), his = in && !(f.full & 2);
+          if (mine) {
+            own.push_back({rec, es});
+            ++sd[2];
+          }
+          if (his && br2) nbr.push_back({rec, es});
+          // the record in modes, scaled by 1 / (a h)
+          SubFaceModal3 r{};
+          r.nb = f.nb;
+          r.pn = f.pn;
+          r.own_off = mine ? M->h_suboff3[b + q] : M->h_toff3[k] + s * N2;
+          const double ia = 1.0 / (a * h), half = in ? 0.5 : 1.0;
+          r.cf = -half * f.area * ia;
+          r.cc = -half * f.area / (h * h);
+          if (in) {
+            int back = -1;   // the same sub-face seen from the neighbour
+            for (int g = m.sf_ptr[6 * (int64_t)f.nb + f.nb_side]; g < m.sf_ptr[6 * (int64_t)f.nb + f.nb_side + 1]; ++g)
+              if (m.sf3[g].nb == k) back = g;
+            r.nbr_off = his ? M->h_suboff3[back] : M->h_toff3[f.nb] + f.nb_side * (f.pn + 1) * (f.pn + 1);
+            const int32_t* tb = mine ? &M->h_rtab3[4 * (size_t)(b + q)] : his ? &M->h_rtab3[4 * (size_t)back] : nullptr;
+            if (tb) {
+              r.tab_ra = tb[0];
+              r.tab_rb = tb[1];
+              r.tab_sa = tb[2];
+              r.tab_sb = tb[3];
+            }
+          }
+          if (br2) {
+            // both sides' lifting energies carry the larger coefficient of the sub-face
+            const double w = in ? std::max(a, m.coef[f.nb]) : a;
+            const double c0 = w * M->eta * (in ? 0.25 : 1.0) * f.area * f.area * ia;
+            r.cz = c0 * (basis1d(P).Minv[0] / (h * h * h));
+            r.czx = r.cz;
+            if (in) {
+              const double hn = M->h_h[f.nb];
+              r.cx = c0 * (basis1d(f.pn).Minv[0] / (hn * hn * hn));
+              if (!mine && !his) r.czx = r.cz + r.cx;
+            }
+          } else {
+            r.cz = f.sigma * f.area * ia;
+          }
+          M->h_sfm3.push_back(r);
         }
       }
     }
-    // Within each chunk the items go in the order of the branches their
-    // threads take - interior first, then the BR2 whole-face flags, then the
-    // neighbour degree (the loop bound) - so that a warp of the two
-    // contraction passes spans fewer kinds of item.  The high half of the
-    // side field keeps the item's position in sub-face order: the second pass
-    // writes the item's partials there, and the third adds them in that order.
+    // the neighbours' liftings by descending neighbour degree, so that a warp
+    // spans few loop bounds
+    std::stable_sort(nbr.begin(), nbr.end(), [&](const std::pair<int32_t, int32_t>& x, const std::pair<int32_t, int32_t>& y) {
+      return M->h_sfm3[x.first].pn > M->h_sfm3[y.first].pn;
+    });
+    for (const auto* l : {&own, &nbr})
+      for (const auto& v : *l) {
+        M->h_hang3.push_back(v.first);
+        M->h_hang3.push_back(v.second);
+      }
+    T.n_c = (int32_t)own.size();
+    T.n_b = (int32_t)nbr.size();
+    const int64_t fixed = modal3_doubles(P) + (j - i) * (int64_t)fixed_per;
+    // rounds: all at once if they fit, else the same number of rounds for both
+    const int64_t room = M->apply3_budget - fixed;
+    int64_t rounds = 1, need = 0;
+    auto per = [&](int64_t n) { return (n + rounds - 1) / rounds; };
+    for (;; ++rounds) {
+      need = per(T.n_c) * own_per + per(T.n_b) * nbr_per;
+      if (need <= room || (per(T.n_c) <= 1 && per(T.n_b) <= 1)) break;
+    }
+    T.cap_c = (int32_t)std::max<int64_t>(1, per(T.n_c));
+    T.cap_b = (int32_t)std::max<int64_t>(1, per(T.n_b));
+    // Host order of the items: by the branches their threads take - interior
+    // first, then the BR2 whole-face flags, then the neighbour degree; the high
+    // half of the side field keeps the item's position in sub-face order.
     {
       const int64_t t0 = M->h_item_ptr.back(), t1 = (int64_t)M->h_items.size() / 2;
-      DG_REQUIRE(T.chunk < 65536, "3D operator: sub-face chunk too long");
-      std::vector<std::pair<int32_t, int32_t>> key;   // (branch key, position in the chunk)
-      std::vector<int32_t> rec, side;
-      for (int64_t c0 = t0; c0 < t1; c0 += T.chunk) {
-        const int64_t c1 = std::min<int64_t>(c0 + T.chunk, t1);
-        key.clear();
-        rec.assign(M->h_items.begin() + 2 * c0, M->h_items.begin() + 2 * c1);
-        for (int64_t g = c0; g < c1; ++g) {
-          const SubFaceRec3& f = M->h_sf3[M->h_items[2 * g]];
-          const bool in = f.nb >= 0;
-          const int zv = (br2 && !(f.full & 1)) ? 1 : 0, yy = (br2 && in && !(f.full & 2)) ? 1 : 0;
-          key.push_back({((in ? 0 : 1) << 12) | (zv << 11) | (yy << 10) | (in ? 16 - f.pn : 0),
-                         (int32_t)(g - c0)});
-        }
-        std::stable_sort(key.begin(), key.end(),
-                         [](const std::pair<int32_t, int32_t>& a, const std::pair<int32_t, int32_t>& b) {
-                           return a.first < b.first;
-                         });
-        for (int64_t g = c0; g < c1; ++g) {
-          const int32_t pos = key[g - c0].second;
-          M->h_items[2 * g] = rec[2 * pos];
-          M->h_items[2 * g + 1] = rec[2 * pos + 1] | (pos << 16);
-        }
+      DG_REQUIRE(t1 - t0 < 65536, "3D operator: too many sub-faces in a tile");
+      T.chunk = (int32_t)(t1 - t0);
+      std::vector<std::pair<int32_t, int32_t>> key;   // (branch key, position in the tile)
+      const std::vector<int32_t> rec(M->h_items.begin() + 2 * t0, M->h_items.end());
+      for (int64_t g = t0; g < t1; ++g) {
+        const SubFaceRec3& f = M->h_sf3[M->h_items[2 * g]];
+        const bool in = f.nb >= 0;
+        const int zv = (br2 && !(f.full & 1)) ? 1 : 0, yy = (br2 && in && !(f.full & 2)) ? 1 : 0;
+        key.push_back({((in ? 0 : 1) << 12) | (zv << 11) | (yy << 10) | (in ? 16 - f.pn : 0), (int32_t)(g - t0)});
+      }
+      std::stable_sort(key.begin(), key.end(),
+                       [](const std::pair<int32_t, int32_t>& x, const std::pair<int32_t, int32_t>& y) {
+                         return x.first < y.first;
+                       });
+      for (int64_t g = t0; g < t1; ++g) {
+        const int32_t pos = key[g - t0].second;
+        M->h_items[2 * g] = rec[2 * pos];
+        M->h_items[2 * g + 1] = rec[2 * pos + 1] | (pos << 16);
       }
     }
     M->h_item_ptr.push_back((int32_t)(M->h_items.size() / 2));
+    M->apply3_smem = std::max<int64_t>(M->apply3_smem, 8 * (fixed + T.cap_c * (int64_t)own_per + T.cap_b * (int64_t)nbr_per));
+    M->modal3_smem = std::max<int64_t>(
+        M->modal3_smem, 8 * (modal3_doubles(P) + T.count * (int64_t)N2 * (P + 1) + T.cap_c * 2 * (int64_t)N2));
     M->h_tiles.push_back(T);
-    M->apply3_smem = std::max<int64_t>(M->apply3_smem, 8LL * (fixed + T.chunk * item_per));
     i = j;
   }
   M->n_tiles = (int)M->h_tiles.size();
   M->h_order = order;
+}
+
+// Trace offsets of every element's sides and, on sides with smaller
+// neighbours, of every sub-face; and the restriction tables of those (after
+// the records).
+static void build_modal3(dg_mesh* M) {
+  const HostMesh& m = M->host;
+  const bool br2 = M->opts.form == DG_FORM_BR2;
+  for (int p = 1; p <= kMaxP; ++p) {
+    M->moff3[p] = (int)M->h_tables.size();
+    modal_tables(p, M->h_tables);
+  }
+  M->moff3[0] = M->moff3[1];
+  int64_t at = 0;
+  M->h_toff3.resize(m.n);
+  for (int64_t k = 0; k < m.n; ++k) {
+    M->h_toff3[k] = (int32_t)at;
+    at += 6 * (m.p[k] + 1) * (m.p[k] + 1);
+    DG_REQUIRE(at < (1LL << 31), "too many side traces");
+  }
+  M->h_suboff3.assign(m.sf3.size(), -1);
+  M->h_rtab3.assign(4 * m.sf3.size(), 0);
+  std::map<std::tuple<int, int, int>, int> index;   // (0 or degree + 1, level, position)
+  auto table = [&](int p, int L, int o) {
+    const auto key = std::make_tuple(p, L, o);
+    const auto it = index.find(key);
+    if (it != index.end()) return it->second;
+    double R[kMaxN * kMaxN];
+    modal_restriction(L, o, R);
+    const int n = p, at0 = (int)M->h_tables.size();
+    if (p == 0) {
+      M->h_tables.insert(M->h_tables.end(), R, R + kMaxN * kMaxN);
+    } else {   // S = R R^T on the first p modes
+      for (int i = 0; i < n; ++i)
+        for (int j = 0; j < n; ++j) {
+          double v = 0.0;
+          for (int q = std::max(i, j); q < n; ++q) v += R[i * kMaxN + q] * R[j * kMaxN + q];
+          M->h_tables.push_back(v);
+        }
+    }
+    index.emplace(key, at0);
+    return at0;
+  };
+  for (int64_t k = 0; k < m.n; ++k)
+    for (int s = 0; s < 6; ++s) {
+      int ax, ta, tb;
+      side_axes3(s, ax, ta, tb);
+      for (int j = m.sf_ptr[6 * k + s]; j < m.sf_ptr[6 * k + s + 1]; ++j) {
+        const auto& f = m.sf3[j];
+        if (f.len == m.size[k]) continue;
+        const int L = ilog2(m.size[k] / f.len), n = m.p[k] + 1;
+        const int oa = (f.a0 - m.lo[3 * k + ta]) / f.len, ob = (f.b0 - m.lo[3 * k + tb]) / f.len;
+        M->h_suboff3[j] = (int32_t)at;
+        at += n * n;
+        DG_REQUIRE(at < (1LL << 31), "too many side traces");
+        int32_t* t = &M->h_rtab3[4 * (size_t)j];
+        t[0] = table(0, L, oa);
+        t[1] = table(0, L, ob);
+        if (br2) {
+          t[2] = table(n, L, oa);
+          t[3] = table(n, L, ob);
+        }
+      }
+    }
+  DG_REQUIRE(M->h_tables.size() < (1ULL << 31), "face tables too large");
+  M->n_trace3 = at;
 }
 
 void build_mesh_host3(dg_mesh* M, const dg_mesh_desc* desc, const dg_options& o) {
@@ -294,86 +440,15 @@ void build_mesh_host3(dg_mesh* M, const dg_mesh_desc* desc, const dg_options& o)
         M->h_sf3[j] = r;
       }
     }
-  // BR2 lifting products of the face tables (the lifting of a sub-face jump,
-  // its element mass inverse and the face mass back onto the side nodes, per
-  // tangential axis), appended after the face tables
-  std::vector<double> prod;
-  std::map<std::tuple<int, int, int, int>, int> pindex;
-  const int pbase = (int)ft.data.size();
-  auto product = [&](int kind, int p, int pn, int oo, int on, int nn) {
-    const auto key = std::make_tuple(kind, kind == 0 ? oo : on, kind == 3 ? nn : (kind == 1 ? oo : -1), p * 16 + pn);
-    auto it = pindex.find(key);
-    if (it != pindex.end()) return it->second;
-    const int a = p + 1, b = pn + 1;
-    const double* Moo = ft.data.data() + oo;
-    const double* Mon = ft.data.data() + on;
-    const double* Mnn = ft.data.data() + nn;
-    const std::vector<double>& Mi = basis1d(p).Minv;
-    const std::vector<double>& Min = basis1d(pn).Minv;
-    const int cols = (kind == 0 || kind == 2) ? a : b;
-    const int o = (int)prod.size();
-    prod.resize(o + (size_t)a * cols, 0.0);
-    for (int i = 0; i < a; ++i)
-      for (int j = 0; j < cols; ++j) {
-        double v = 0.0;
-        if (kind == 0) {          // Z = M_oo Minv M_oo
-          for (int u = 0; u < a; ++u)
-            for (int w = 0; w < a; ++w) v += Moo[i * a + u] * Mi[u * a + w] * Moo[w * a + j];
-        } else if (kind == 1) {   // V = M_oo Minv M_on
-          for (int u = 0; u < a; ++u)
-            for (int w = 0; w < a; ++w) v += Moo[i * a + u] * Mi[u * a + w] * Mon[w * b + j];
-        } else if (kind == 2) {   // X = M_on Minv_n M_no
-          for (int u = 0; u < b; ++u)
-            for (int w = 0; w < b; ++w) v += Mon[i * b + u] * Min[u * b + w] * Mon[j * b + w];
-        } else {                  // Y = M_on Minv_n M_nn
-          for (int u = 0; u < b; ++u)
-            for (int w = 0; w < b; ++w) v += Mon[i * b + u] * Min[u * b + w] * Mnn[w * b + j];
-        }
-        prod[o + (size_t)i * cols + j] = v;
-      }
-    pindex.emplace(key, pbase + o);
-    return pbase + o;
-  };
-  for (int64_t k = 0; k < m.n; ++k)
-    for (int s = 0; s < 6; ++s)
-      for (int j = m.sf_ptr[6 * k + s]; j < m.sf_ptr[6 * k + s + 1]; ++j) {
-        SubFaceRec3& r = M->h_sf3[j];
-        const int P = m.p[k];
-        const bool in = r.nb >= 0;
-        const double coef = in ? 0.25 : 1.0;
-        const double hk = M->h_h[k];
-        // both sides' lifting energies carry the larger coefficient of the sub-face
-        const double w = in ? std::max(m.coef[k], m.coef[r.nb]) : m.coef[k];
-        r.cz = w * (M->eta * coef * r.area * r.area * basis1d(P).Minv[0] / (hk * hk * hk));
-        for (int d = 0; d < 2; ++d) {
-          r.tab_z[d] = product(0, P, P, r.tab_oo[d], r.tab_oo[d], r.tab_oo[d]);
-          if (in) {
-            r.tab_v[d] = product(1, P, r.pn, r.tab_oo[d], r.tab_on[d], r.tab_nn[d]);
-            r.tab_x[d] = product(2, P, r.pn, r.tab_oo[d], r.tab_on[d], r.tab_nn[d]);
-            r.tab_y[d] = product(3, P, r.pn, r.tab_oo[d], r.tab_on[d], r.tab_nn[d]);
-          } else {
-            r.tab_v[d] = r.tab_x[d] = r.tab_y[d] = r.tab_z[d];
-          }
-        }
-        if (in) {
-          const double hn = M->h_h[r.nb];
-          r.cx = w * (M->eta * coef * r.area * r.area * basis1d(r.pn).Minv[0] / (hn * hn * hn));
-        }
-      }
   const int base = (int)M->h_tables.size();
   M->h_tables.insert(M->h_tables.end(), ft.data.begin(), ft.data.end());
-  M->h_tables.insert(M->h_tables.end(), prod.begin(), prod.end());
-  DG_REQUIRE(M->h_tables.size() < (1ULL << 31), "face tables too large");
   for (auto& r : M->h_sf3)
     for (int d = 0; d < 2; ++d) {
       r.tab_oo[d] += base;
       r.tab_on[d] += base;
       r.tab_nn[d] += base;
-      r.tab_z[d] += base;
-      r.tab_v[d] += base;
-      r.tab_x[d] += base;
-      r.tab_y[d] += base;
     }
+  build_modal3(M);
   build_tiles3(M);
   // operation and byte counts of one operator apply, as the kernels do it
   dg_mesh_stats& S = M->stats;
@@ -381,33 +456,31 @@ void build_mesh_host3(dg_mesh* M, const dg_mesh_desc* desc, const dg_options& o)
   S.n_elems = m.n;
   S.n_dofs = M->n_dofs;
   S.n_subfaces = (int64_t)m.sf3.size();
+  // FP64 operations of both kernels, a multiply-add, a product and a sum each
+  // counted as one
   const bool br2 = o.form == DG_FORM_BR2;
   double fma = 0.0;
   for (int64_t k = 0; k < m.n; ++k) {
     const double a = m.p[k] + 1.0, a2 = a * a, a3 = a2 * a;
-    fma += 7.0 * a3 * a + 6.0 * a3 + 6.0 * a3;   // volume, traces' dn, gather
+    const double H = std::floor(a / 2), C = a - H;
+    const double line = C * C + H * H + 2.0 * H;                       // one line between nodes and modes
+    const double stiff = H * H + (C - 1.0) * (C - 1.0);                // one line's stiffness
+    fma += 3.0 * a2 * (2.0 * line + stiff + 2.0 * (2.0 * a + 4.0));    // + traces, lift
     for (int j = m.sf_ptr[6 * k]; j < m.sf_ptr[6 * k + 6]; ++j) {
       const auto& f = m.sf3[j];
-      const bool own_full = f.len == m.size[k];
-      if (f.nb < 0) {
-        fma += 4.0 * a3 + ((br2 && !own_full) ? 2.0 * a3 : 0.0);   // M_oo on u, dn; BR2: Z on u
-        continue;
-      }
-      const double b = m.p[f.nb] + 1.0, b2 = b * b;
-      const bool nb_full = f.len == m.size[f.nb];
-      fma += 4.0 * a3 + 2.0 * a * b2 + 2.0 * a2 * b;   // M_oo on u-, dn-; M_on on u+, dn+
-      if (br2) {
-        fma += 2.0 * a3;                                          // X on u-
-        if (!own_full) fma += 2.0 * a3 + a * b2 + a2 * b;         // Z on u-, V on u+
-        if (!nb_full) fma += a * b2 + a2 * b;                     // Y on u+
-      }
+      fma += 5.0 * a2;
+      if (f.nb < 0) continue;
+      const double b = m.p[f.nb] + 1.0;
+      const double tri = a2 * (a + 1.0);                               // R or R^T in both directions
+      if (f.len != m.size[k]) fma += 4.0 * tri + (br2 ? 2.0 * a3 : 0.0);
+      else if (f.len != m.size[f.nb] && br2) fma += std::min(a, b) * b * (b + std::min(a, b));
       const int lg = std::abs(ilog2(m.size[k]) - ilog2(m.size[f.nb]));
       S.max_level_gap = std::max<int64_t>(S.max_level_gap, lg);
     }
   }
   S.apply_flops = 2.0 * fma;
   S.apply_bytes = 16.0 * (double)M->n_dofs + (double)m.n * (4 + 8 + 8 + 4 + 16) +
-                  (double)m.sf3.size() * sizeof(SubFaceRec3);
+                  (double)m.sf3.size() * sizeof(SubFaceModal3);
 }
 
 // Rows of element k of y = A x on a cube mesh, with the records and tables the
