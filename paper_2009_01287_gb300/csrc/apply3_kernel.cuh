@@ -16,22 +16,27 @@
 //     per position whatever the degree;
 //   - the nodes' mirror symmetry and the modes' parity halve the transforms
 //     and the traces of opposite faces (sums and differences of node pairs).
-// Two kernels per apply:
-//  modal3  x^ of every element, the traces u and a grad u . n of its six sides
-//          in modes and, on the sides with smaller neighbours, their
-//          restriction to every sub-face (formed once for both sides' use);
-//  apply3  one CTA per tile of elements of one degree P:
-//    faces   whole sides point by point in modes; a side with smaller
-//            neighbours per sub-face (J = jump, F = flux in the sub-face's
-//            modes, back through R^T; BR2's own lifting through S = R R^T);
-//            BR2's neighbour lifting on sub-faces of a larger neighbour
-//            through its S;
-//    volume  per line of modes K x^ plus the lift of the two side residuals,
-//            along z, y, x; then the transposed transform along x, y, z.
-// On the 16^3 hp-random workload (1.7M unknowns, BR2) FP64 operations per
-// apply fell from 219 M to 128 M FMA-sized ones against the nodal form
-// with its face-mass products.
-// Each sub-face is evaluated from both of its sides (no atomics): applies are
+// Three kernels per apply:
+//  modal3  x^ of every element and the traces u and a grad u . n of its six
+//          sides in modes;
+//  hang3   per sub-face between a larger and a smaller side (a pair): the
+//          larger side's traces restricted by R, J = jump and F = flux, and
+//          the residuals of both sides, the larger side's back through R^T.
+//          BR2's lifting on the larger side, R R^T J, serves both sides.  Its
+//          own kernel, because an element can have anything from none to
+//          dozens of them: taken inside the element's tile they made the
+//          heaviest tile four times the mean and the SMs 54% busy on average;
+//  apply3  one CTA per tile of elements of one degree P: side residuals point
+//          by point in modes (same-size neighbours and the boundary) or summed
+//          from the pairs' in order; then per line of modes K x^ plus the lift
+//          of the two side residuals, along z, y, x, and the transposed
+//          transform along x, y, z.
+// Measured (GB300), apply of the 16^3 hp-random workload (1.7M unknowns, BR2):
+// 689 us in nodal form with face-mass products, 350 in modes with the hanging
+// sub-faces inside the tiles, 272 with their own kernel; 79k unknowns, SIPG,
+// 62.8 / 48.6 / 33.0 us.  The FP64 operations alone are 0.218 ms on the large
+// one at the measured 1.06 TFLOP/s.
+// Every sum has a fixed order and there are no atomics on data: applies are
 // bit-reproducible.
 #pragma once
 
@@ -149,7 +154,6 @@ __device__ __forceinline__ void modal3_tile(const ApplyArgs& A, const ApplyTile&
   constexpr int NP = P + 1, N2 = NP * NP, N3 = N2 * NP;
   double* tb = sm;
   double* sx = tb + B::SIZE;
-  double* sy = sx + T.count * N3;   // [cap_c][2][N2]: half-restricted traces
   const double *E = tb, *O = tb + B::oO, *S = tb + B::oS, *Q = tb + B::oQ;
   const int tid = threadIdx.x, nl = T.count * N2;
   for (int i = tid; i < B::SIZE; i += kThreads3) tb[i] = __ldg(A.tab + A.moff3[P] + i);
@@ -212,49 +216,145 @@ __device__ __forceinline__ void modal3_tile(const ApplyArgs& A, const ApplyTile&
     const int e = t / N3;
     A.xm[er[e].off + (t - e * N3)] = sx[t];
   }
-  // sides with smaller neighbours: u and dn restricted to each sub-face,
-  // R_a (x) R_b, one thread per line of one of the two quantities
-  const int2* hang = A.hang3 + T.hang;
-  for (int c0 = 0; c0 < T.n_c; c0 += T.cap_c) {
-    const int nc = min(T.cap_c, T.n_c - c0);
-    __syncthreads();   // the traces above (and the last round's scratch)
-    for (int t = tid; t < nc * 2 * NP; t += kThreads3) {
-      const int it = t / (2 * NP), rem = t - it * 2 * NP;
-      const int w = rem / NP, n = rem - w * NP;
-      const int2 hg = hang[c0 + it];
-      const SubFaceModal3& f = A.sfm3[hg.x];
-      const int e = hg.y / 6, s = hg.y - e * 6;
-      const double* src = reinterpret_cast<const double*>(tr + er[e].toff + s * N2 + n * NP) + w;
+}
+
+// one line times R, upper triangular, or R^T
+template <int NP>
+__device__ __forceinline__ void line_restrict(const double (&v)[NP], double (&o)[NP], const double* R) {
 #pragma unroll
-      for (int q = 0; q < NP; ++q) v[q] = src[2 * q];
-      const double* R = A.tab + f.tab_ra;
-      double* dst = sy + (it * 2 + w) * N2 + n * NP;
+  for (int k = 0; k < NP; ++k) {
+    double a = __ldg(R + k * kMaxN + k) * v[k];
 #pragma unroll
-      for (int k = 0; k < NP; ++k) {
-        double a = __ldg(R + k * kMaxN + k) * v[k];
+    for (int m = k + 1; m < NP; ++m) a = fma(__ldg(R + k * kMaxN + m), v[m], a);
+    o[k] = a;
+  }
+}
+template <int NP>
+__device__ __forceinline__ void line_restrict_t(const double (&v)[NP], double (&o)[NP], const double* R) {
 #pragma unroll
-        for (int m = k + 1; m < NP; ++m) a = fma(__ldg(R + k * kMaxN + m), v[m], a);
-        dst[k] = a;
+  for (int m = 0; m < NP; ++m) {
+    double a = __ldg(R + m) * v[0];
+#pragma unroll
+    for (int k = 1; k <= m; ++k) a = fma(__ldg(R + k * kMaxN + m), v[k], a);
+    o[m] = a;
+  }
+}
+
+// The hanging pairs of one tile (one degree P of the larger side).  Residuals
+// over a h and normal-derivative coefficients over a h of either side go to
+// the results part of the trace buffer.
+template <int P, bool BR2>
+__device__ __forceinline__ void hang3_tile(const ApplyArgs& A, const HangTile& T, double* sm) {
+  constexpr int NP = P + 1, N2 = NP * NP;
+  const int cnt = T.count, NS = T.ns, NM = NP > NS ? NP : NS;
+  double* sX = sm;                    // [cnt][2][N2]: restricted u, dn; then J, residual
+  double* sY = sX + cnt * 2 * N2;     // [cnt][2][N2]: half-way products
+  const int tid = threadIdx.x;
+  const HangPair* hp = A.hang3 + T.first;
+  double2* tr = reinterpret_cast<double2*>(A.tr);
+  const double* trd = A.tr;
+  double v[NP], o[NP];
+  auto load = [&](const double* p, int st) {
+#pragma unroll
+    for (int q = 0; q < NP; ++q) v[q] = p[q * st];
+  };
+  auto store = [&](double* p, int st) {
+#pragma unroll
+    for (int q = 0; q < NP; ++q) p[q * st] = o[q];
+  };
+  for (int t = tid; t < cnt * 2 * NP; t += kThreads3) {   // R along the first axis
+    const int it = t / (2 * NP), rem = t - it * 2 * NP, w = rem / NP, n = rem - w * NP;
+    load(trd + 2 * ((int64_t)hp[it].src_b + n * NP) + w, 2);
+    line_restrict<NP>(v, o, A.tab + hp[it].tab_ra);
+    store(sY + (it * 2 + w) * N2 + n * NP, 1);
+  }
+  __syncthreads();
+  for (int t = tid; t < cnt * 2 * NP; t += kThreads3) {   // and the second
+    const int it = t / (2 * NP), rem = t - it * 2 * NP, w = rem / NP, i = rem - w * NP;
+    load(sY + (it * 2 + w) * N2 + i, NP);
+    line_restrict<NP>(v, o, A.tab + hp[it].tab_rb);
+    store(sX + (it * 2 + w) * N2 + i, NP);
+  }
+  __syncthreads();
+  // J and F of the larger side; the smaller side's are their negatives
+  for (int t = tid; t < cnt * NM * NM; t += kThreads3) {
+    const int it = t / (NM * NM), q = t - it * NM * NM, i = q % NM, j = q / NM;
+    const HangPair& h = hp[it];
+    const int ns = h.ns;
+    const bool big = i < NP && j < NP, small = i < ns && j < ns;
+    if (!big && !small) continue;
+    double* X = sX + it * 2 * N2 + j * NP + i;
+    double J = big ? X[0] : 0.0, F = big ? X[N2] : 0.0;
+    if (small) {
+      const double2 s = tr[h.src_s + j * ns + i];
+      J -= s.x;
+      F -= s.y;
+      // (BR2: the larger side's lifting is added to the residual below)
+      tr[h.dst_s + j * ns + i] = make_double2(-fma(h.cz_s, J, h.cf_s * F), -h.cc_s * J);
+    }
+    if (big) {
+      X[0] = J;
+      X[N2] = BR2 ? (small ? fma(h.cx_b, J, h.cf_b * F) : h.cf_b * F) : fma(h.cz_b, J, h.cf_b * F);
+    }
+  }
+  __syncthreads();
+  constexpr int W = BR2 ? 1 : 2;   // SIPG: J and the residual go back together
+  for (int t = tid; t < cnt * W * NP; t += kThreads3) {
+    const int it = t / (W * NP), rem = t - it * W * NP, w = rem / NP, n = rem - w * NP;
+    load(sX + (it * 2 + w) * N2 + n * NP, 1);
+    line_restrict_t<NP>(v, o, A.tab + hp[it].tab_ra);
+    store(sY + (it * 2 + w) * N2 + n * NP, 1);
+  }
+  __syncthreads();
+  for (int t = tid; t < cnt * W * NP; t += kThreads3) {
+    const int it = t / (W * NP), rem = t - it * W * NP, w = rem / NP, i = rem - w * NP;
+    const HangPair& h = hp[it];
+    load(sY + (it * 2 + w) * N2 + i, NP);
+    line_restrict_t<NP>(v, o, A.tab + h.tab_rb);
+    if (BR2) store(sX + it * 2 * N2 + i, NP);   // R^T J: the lifting, and c2
+    double* dst = A.tr + 2 * ((int64_t)h.dst_b + i) + (w == 0 ? 1 : 0);
+    const double c = w == 0 ? h.cc_b : 1.0;
+#pragma unroll
+    for (int q = 0; q < NP; ++q) dst[2 * q * NP] = w == 0 ? c * o[q] : o[q];
+  }
+  if (!BR2) return;
+  __syncthreads();
+  for (int t = tid; t < cnt * NP; t += kThreads3) {   // R R^T J
+    const int it = t / NP, n = t - it * NP;
+    load(sX + it * 2 * N2 + n * NP, 1);
+    line_restrict<NP>(v, o, A.tab + hp[it].tab_ra);
+    store(sY + it * 2 * N2 + n * NP, 1);
+  }
+  __syncthreads();
+  for (int t = tid; t < cnt * NP; t += kThreads3) {
+    const int it = t / NP, i = t - it * NP;
+    const HangPair& h = hp[it];
+    load(sY + it * 2 * N2 + i, NP);
+    line_restrict<NP>(v, o, A.tab + h.tab_rb);
+    const int ns = h.ns;
+    double* X = sX + it * 2 * N2 + N2 + i;
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+      X[q * NP] = fma(h.cz_b, o[q], X[q * NP]);
+      if (i < ns && q < ns) {
+        double2* d = tr + h.dst_s + q * ns + i;
+        d->x = fma(-h.cx_s, o[q], d->x);
       }
     }
-    __syncthreads();
-    for (int t = tid; t < nc * 2 * NP; t += kThreads3) {
-      const int it = t / (2 * NP), rem = t - it * 2 * NP;
-      const int w = rem / NP, i = rem - w * NP;
-      const SubFaceModal3& f = A.sfm3[hang[c0 + it].x];
-      const double* src = sy + (it * 2 + w) * N2 + i;
-#pragma unroll
-      for (int q = 0; q < NP; ++q) v[q] = src[q * NP];
-      const double* R = A.tab + f.tab_rb;
-      double* dst = reinterpret_cast<double*>(tr + f.own_off + i) + w;
-#pragma unroll
-      for (int k = 0; k < NP; ++k) {
-        double a = __ldg(R + k * kMaxN + k) * v[k];
-#pragma unroll
-        for (int m = k + 1; m < NP; ++m) a = fma(__ldg(R + k * kMaxN + m), v[m], a);
-        dst[2 * k * NP] = a;
-      }
-    }
+  }
+  __syncthreads();
+  for (int t = tid; t < cnt * NP; t += kThreads3) {   // the larger side's residual back
+    const int it = t / NP, n = t - it * NP;
+    load(sX + it * 2 * N2 + N2 + n * NP, 1);
+    line_restrict_t<NP>(v, o, A.tab + hp[it].tab_ra);
+    store(sY + it * 2 * N2 + n * NP, 1);
+  }
+  __syncthreads();
+  for (int t = tid; t < cnt * NP; t += kThreads3) {
+    const int it = t / NP, i = t - it * NP;
+    load(sY + it * 2 * N2 + i, NP);
+    line_restrict_t<NP>(v, o, A.tab + hp[it].tab_rb);
+    store(A.tr + 2 * ((int64_t)hp[it].dst_b + i), 2 * NP);
   }
 }
 
@@ -263,14 +363,12 @@ __device__ __forceinline__ void apply3_tile(const ApplyArgs& A, const ApplyTile&
                                             double* red) {
   using B = Modal3<P>;
   constexpr int NP = P + 1, N2 = NP * NP, N3 = N2 * NP;
-  const int cnt = T.count, nl = cnt * N2, NQ = T.nq;
+  const int cnt = T.count, nl = cnt * N2;
   double* tb = sm;
   double* sx = tb + B::SIZE;
   double* sg = sx + cnt * N3;
   double* sr = sg + cnt * N3;              // [cnt][6][N2] side residuals over a h
   double* sc = sr + cnt * 6 * N2;          // [cnt][6][N2] normal-derivative coefficients over a h
-  double* sw = sc + cnt * 6 * N2;          // larger sides' sub-faces: [cap_c][4][N2]
-  double* sb = sw + T.cap_c * 4 * N2;      // BR2, larger neighbours: [cap_b][NQ * NQ + NP * NQ]
   const double *E = tb, *O = tb + B::oO, *K = tb + B::oK, *S = tb + B::oS, *Q = tb + B::oQ;
   const int tid = threadIdx.x;
   const double2* tr = reinterpret_cast<const double2*>(A.tr);
@@ -280,194 +378,38 @@ __device__ __forceinline__ void apply3_tile(const ApplyArgs& A, const ApplyTile&
     const int e = t / N3;
     sx[t] = __ldg(A.xm + er[e].off + (t - e * N3));
   }
-  // ---- whole sides (same-size neighbour, boundary, or a sub-face of a larger
-  // neighbour, whose restricted trace is in place): diagonal in modes
+  // ---- side residuals: same-size neighbours and the boundary point by point
+  // (diagonal in modes), hanging sides from their pairs' results, in order
   for (int t = tid; t < cnt * 6 * N2; t += kThreads3) {
     const int es = t / N2, q = t - es * N2;
-    const int4 sd = __ldg(A.side3 + (int64_t)T.first * 6 + es);   // {record, first sub-face, sub-faces}
-    double r = 0.0, c = 0.0;
-    if (sd.z == 0) {
+    const int2 sd = __ldg(A.side3 + (int64_t)T.first * 6 + es);   // {record, 0} or {first result, pairs}
+    double r, c;
+    if (sd.y == 0) {
       const SubFaceModal3& f = A.sfm3[sd.x];
-      const int i = q % NP, j = q / NP, npn = f.pn + 1;
+      const int i = q % NP, j = q / NP, nn = f.nn;
       const double2 o = __ldg(tr + f.own_off + q);
       double J = o.x, F = o.y;
-      const bool in = f.nb >= 0 && i < npn && j < npn;
+      const bool in = i < nn && j < nn;   // boundary: nn = 0
       if (in) {
-        const double2 n = __ldg(tr + f.nbr_off + j * npn + i);
+        const double2 n = __ldg(tr + f.nbr_off + j * nn + i);
         J -= n.x;
         F -= n.y;   // the neighbour's outward dn
       }
       r = fma(BR2 && in ? f.czx : f.cz, J, f.cf * F);
       c = f.cc * J;
+    } else {
+      const double2* src = tr + sd.x + q;
+      const double2 f = __ldg(src);
+      r = f.x;
+      c = f.y;
+      for (int g = 1; g < sd.y; ++g) {
+        const double2 n = __ldg(src + g * N2);
+        r += n.x;
+        c += n.y;
+      }
     }
     sr[t] = r;
     sc[t] = c;
-  }
-  // ---- sub-faces smaller than the own side (C) and, for BR2, sub-faces of a
-  // larger neighbour (its lifting), in rounds that fit the scratch
-  const int2* hang = A.hang3 + T.hang;
-  const int n_b = BR2 ? T.n_b : 0;
-  for (int c0 = 0, b0 = 0; c0 < T.n_c || b0 < n_b; c0 += T.cap_c, b0 += T.cap_b) {
-    const int nc = max(0, min(T.cap_c, T.n_c - c0)), nb = max(0, min(T.cap_b, n_b - b0));
-    for (int t = tid; t < nc * N2; t += kThreads3) {   // J and the point-by-point residual
-      const int it = t / N2, q = t - it * N2;
-      const SubFaceModal3& f = A.sfm3[hang[c0 + it].x];
-      const int i = q % NP, j = q / NP, npn = f.pn + 1;
-      const double2 o = __ldg(tr + f.own_off + q);
-      double J = o.x, F = o.y;
-      const bool in = i < npn && j < npn;
-      if (in) {
-        const double2 n = __ldg(tr + f.nbr_off + j * npn + i);
-        J -= n.x;
-        F -= n.y;
-      }
-      double* X = sw + it * 4 * N2;
-      X[q] = J;
-      X[N2 + q] = BR2 ? (in ? fma(f.cx, J, f.cf * F) : f.cf * F) : fma(f.cz, J, f.cf * F);
-    }
-    for (int t = tid; t < nb * NQ * NQ; t += kThreads3) {   // J in the larger neighbour's modes
-      const int it = t / (NQ * NQ), q = t - it * NQ * NQ;
-      const SubFaceModal3& f = A.sfm3[hang[T.n_c + b0 + it].x];
-      const int i = q % NQ, j = q / NQ, npn = f.pn + 1;
-      if (i < npn && j < npn) {
-        double J = -__ldg(tr + f.nbr_off + j * npn + i).x;
-        if (i < NP && j < NP) J += __ldg(tr + f.own_off + j * NP + i).x;
-        sb[it * (NQ * NQ + NP * NQ) + j * NQ + i] = J;
-      }
-    }
-    __syncthreads();
-    // first tangential axis: R^T J, and S J (BR2) or R^T of the residual
-    for (int t = tid; t < nc * 2 * NP; t += kThreads3) {
-      const int it = t / (2 * NP), rem = t - it * 2 * NP;
-      const int w = rem / NP, n = rem - w * NP;
-      const SubFaceModal3& f = A.sfm3[hang[c0 + it].x];
-      const double* X = sw + it * 4 * N2 + (BR2 ? 0 : w) * N2 + n * NP;
-      double* Y = sw + it * 4 * N2 + (2 + w) * N2 + n * NP;
-      double v[NP];
-#pragma unroll
-      for (int q = 0; q < NP; ++q) v[q] = X[q];
-      if (BR2 && w == 1) {
-        const double* Sa = A.tab + f.tab_sa;
-#pragma unroll
-        for (int m = 0; m < NP; ++m) {
-          double a = __ldg(Sa + m * NP) * v[0];
-#pragma unroll
-          for (int k = 1; k < NP; ++k) a = fma(__ldg(Sa + m * NP + k), v[k], a);
-          Y[m] = a;
-        }
-      } else {
-        const double* R = A.tab + f.tab_ra;
-#pragma unroll
-        for (int m = 0; m < NP; ++m) {
-          double a = __ldg(R + m) * v[0];
-#pragma unroll
-          for (int k = 1; k <= m; ++k) a = fma(__ldg(R + k * kMaxN + m), v[k], a);
-          Y[m] = a;
-        }
-      }
-    }
-    for (int t = tid; t < nb * NP * NQ; t += kThreads3) {
-      const int it = t / (NP * NQ), rem = t - it * NP * NQ;
-      const int i = rem % NP, n = rem / NP;
-      const SubFaceModal3& f = A.sfm3[hang[T.n_c + b0 + it].x];
-      const int npn = f.pn + 1;
-      double* X = sb + it * (NQ * NQ + NP * NQ);
-      if (i < npn && n < npn) {
-        const double* Sa = A.tab + f.tab_sa + i * npn;
-        double a = 0.0;
-        for (int m = 0; m < npn; ++m) a = fma(__ldg(Sa + m), X[n * NQ + m], a);
-        X[NQ * NQ + n * NP + i] = a;
-      }
-    }
-    __syncthreads();
-    // second tangential axis
-    for (int t = tid; t < nc * 2 * NP; t += kThreads3) {
-      const int it = t / (2 * NP), rem = t - it * 2 * NP;
-      const int w = rem / NP, i = rem - w * NP;
-      const SubFaceModal3& f = A.sfm3[hang[c0 + it].x];
-      const double* Y = sw + it * 4 * N2 + (2 + w) * N2 + i;
-      double* X = sw + it * 4 * N2 + w * N2 + i;
-      double v[NP];
-#pragma unroll
-      for (int q = 0; q < NP; ++q) v[q] = Y[q * NP];
-      if (BR2 && w == 1) {
-        const double* Sb = A.tab + f.tab_sb;
-#pragma unroll
-        for (int m = 0; m < NP; ++m) {
-          double a = __ldg(Sb + m * NP) * v[0];
-#pragma unroll
-          for (int k = 1; k < NP; ++k) a = fma(__ldg(Sb + m * NP + k), v[k], a);
-          X[m * NP] = fma(f.cz, a, X[m * NP]);
-        }
-      } else {
-        const double* R = A.tab + f.tab_rb;
-#pragma unroll
-        for (int m = 0; m < NP; ++m) {
-          double a = __ldg(R + m) * v[0];
-#pragma unroll
-          for (int k = 1; k <= m; ++k) a = fma(__ldg(R + k * kMaxN + m), v[k], a);
-          X[m * NP] = w == 0 ? f.cc * a : a;
-        }
-      }
-    }
-    for (int t = tid; t < nb * N2; t += kThreads3) {
-      const int it = t / N2, q = t - it * N2;
-      const int i = q % NP, j = q / NP;
-      const int2 hg = hang[T.n_c + b0 + it];
-      const SubFaceModal3& f = A.sfm3[hg.x];
-      const int npn = f.pn + 1;
-      if (i < npn && j < npn) {
-        const double* Sb = A.tab + f.tab_sb + j * npn;
-        const double* Y = sb + it * (NQ * NQ + NP * NQ) + NQ * NQ + i;
-        double a = 0.0;
-        for (int n = 0; n < npn; ++n) a = fma(__ldg(Sb + n), Y[n * NP], a);
-        sr[hg.y * N2 + q] = fma(f.cx, a, sr[hg.y * N2 + q]);
-      }
-    }
-    if (BR2) {   // back through R^T, after the own lifting joined the residual
-#pragma unroll
-      for (int ax = 0; ax < 2; ++ax) {
-        __syncthreads();
-        for (int t = tid; t < nc * NP; t += kThreads3) {
-          const int it = t / NP, n = t - it * NP;
-          const SubFaceModal3& f = A.sfm3[hang[c0 + it].x];
-          double* X = sw + it * 4 * N2 + N2;
-          const double* src = ax == 0 ? X + n * NP : X + N2 + n;
-          double* dst = ax == 0 ? X + N2 + n * NP : X + n;
-          const int st = ax == 0 ? 1 : NP;
-          double v[NP];
-#pragma unroll
-          for (int q = 0; q < NP; ++q) v[q] = src[q * st];
-          const double* R = A.tab + (ax == 0 ? f.tab_ra : f.tab_rb);
-#pragma unroll
-          for (int m = 0; m < NP; ++m) {
-            double a = __ldg(R + m) * v[0];
-#pragma unroll
-            for (int k = 1; k <= m; ++k) a = fma(__ldg(R + k * kMaxN + m), v[k], a);
-            dst[m * st] = a;
-          }
-        }
-      }
-    }
-    __syncthreads();
-    // every mode of a side adds its sub-faces of this round, in order
-    if (nc > 0)
-      for (int t = tid; t < cnt * 6 * N2; t += kThreads3) {
-        const int es = t / N2, q = t - es * N2;
-        const int4 sd = __ldg(A.side3 + (int64_t)T.first * 6 + es);
-        const int lo = max(sd.y, c0), hi = min(sd.y + sd.z, c0 + nc);
-        if (lo < hi) {
-          double r = sr[t], c = sc[t];
-          for (int g = lo; g < hi; ++g) {
-            const double* X = sw + (g - c0) * 4 * N2 + q;
-            c += X[0];
-            r += X[N2];
-          }
-          sr[t] = r;
-          sc[t] = c;
-        }
-      }
-    __syncthreads();
   }
   __syncthreads();
   // ---- volume and lift, one thread per line of modes

@@ -178,8 +178,9 @@ struct ApplyArgs {
   const SubFaceBr2* sfb;      // square meshes, BR2: the multiplied-out liftings
   const SubFaceModal3* sfm3;  // cube meshes
   const ElemRec3* erec3;
-  const int2* hang3;
-  const int4* side3;
+  const HangPair* hang3;
+  const HangTile* hang_tiles;
+  const int2* side3;
   double* xm;
   int moff3[kMaxP + 1];
   const double* tab;          // basis + face tables

@@ -63,9 +63,12 @@ __device__ __forceinline__ void apply_exit(const ApplyArgs& A, double* red) {
   }
 }
 
-// Persistent operator kernel: a grid sized to the resident capacity takes
+// Persistent operator kernel: a grid sized to the resident capacity, CTA b
+// starting on tile b (consecutive CTAs land on different SMs) and then taking
 // tiles from an atomic counter, heaviest first (tiles are degree-sorted), so
-// the uneven tiles balance across SMs.  The last CTA to leave resets the
+// the uneven tiles balance across SMs.  The next tile's number is fetched
+// while a tile runs (two slots, so that a fast warp's fetch cannot overwrite
+// the number a slow one has yet to read).  The last CTA to leave resets the
 // counter and, when a dot product is requested, sums the tile partials in
 // tile order (deterministic whichever CTA ran which tile).
 template <bool BR2>
@@ -73,13 +76,9 @@ __global__ void __launch_bounds__(kThreads) apply_kernel(const ApplyArgs A) {
   pdl_entry();
   extern __shared__ __align__(16) double smem[];
   __shared__ double red[kThreads];
-  __shared__ int s_tile;
-  while (true) {
-    if (threadIdx.x == 0) s_tile = (int)atomicAdd(A.sched, 1u);
-    __syncthreads();
-    const int t = s_tile;
-    __syncthreads();
-    if (t >= A.n_tiles) break;
+  __shared__ int s_next[2];
+  for (int t = blockIdx.x, par = 0; t < A.n_tiles; par ^= 1) {
+    if (threadIdx.x == 0) s_next[par] = (int)(gridDim.x + atomicAdd(A.sched, 1u));
     const ApplyTile T = A.tiles[t];
     switch (T.p) {
       case 1: apply_tile<1, BR2>(A, T, t, smem, red); break;
@@ -93,6 +92,7 @@ __global__ void __launch_bounds__(kThreads) apply_kernel(const ApplyArgs A) {
       default: break;
     }
     __syncthreads();
+    t = s_next[par];
   }
   apply_exit<kThreads>(A, red);
 }
@@ -103,13 +103,9 @@ __global__ void __launch_bounds__(kThreads) apply_map_kernel(const ApplyArgs A) 
   pdl_entry();
   extern __shared__ __align__(16) double smem[];
   __shared__ double red[kThreads];
-  __shared__ int s_tile;
-  while (true) {
-    if (threadIdx.x == 0) s_tile = (int)atomicAdd(A.sched, 1u);
-    __syncthreads();
-    const int t = s_tile;
-    __syncthreads();
-    if (t >= A.n_tiles) break;
+  __shared__ int s_next[2];
+  for (int t = blockIdx.x, par = 0; t < A.n_tiles; par ^= 1) {
+    if (threadIdx.x == 0) s_next[par] = (int)(gridDim.x + atomicAdd(A.sched, 1u));
     const ApplyTile T = A.tiles[t];
     switch (T.p) {
       case 1: apply_map_tile<1, BR2>(A, T, t, smem, red); break;
@@ -123,6 +119,7 @@ __global__ void __launch_bounds__(kThreads) apply_map_kernel(const ApplyArgs A) 
       default: break;
     }
     __syncthreads();
+    t = s_next[par];
   }
   apply_exit<kThreads>(A, red);
 }
@@ -153,19 +150,31 @@ modal3_kernel(const ApplyArgs A, double* p, const double* z, double* sc, cudaGra
   if (UPDATE && first) pcg_first_scalars(sc, h, use_cond);
 }
 
+// Residuals of both sides of every hanging sub-face of a cube mesh.
+template <bool BR2>
+__global__ void __launch_bounds__(kThreads3) hang3_kernel(const ApplyArgs A) {
+  pdl_entry();
+  extern __shared__ __align__(16) double smem[];
+  const HangTile T = A.hang_tiles[blockIdx.x];
+  switch (T.p) {
+#define DG_HANG_CASE(PP) \
+    case PP: hang3_tile<PP, BR2>(A, T, smem); break;
+    DG_HANG_CASE(1) DG_HANG_CASE(2) DG_HANG_CASE(3) DG_HANG_CASE(4)
+    DG_HANG_CASE(5) DG_HANG_CASE(6) DG_HANG_CASE(7) DG_HANG_CASE(8)
+#undef DG_HANG_CASE
+    default: break;
+  }
+}
+
 // Persistent operator kernel of cube meshes (same scheduling as on squares).
 template <bool BR2>
 __global__ void __launch_bounds__(kThreads3) apply3_kernel(const ApplyArgs A) {
   pdl_entry();
   extern __shared__ __align__(16) double smem[];
   __shared__ double red[kThreads3];
-  __shared__ int s_tile;
-  while (true) {
-    if (threadIdx.x == 0) s_tile = (int)atomicAdd(A.sched, 1u);
-    __syncthreads();
-    const int t = s_tile;
-    __syncthreads();
-    if (t >= A.n_tiles) break;
+  __shared__ int s_next[2];
+  for (int t = blockIdx.x, par = 0; t < A.n_tiles; par ^= 1) {
+    if (threadIdx.x == 0) s_next[par] = (int)(gridDim.x + atomicAdd(A.sched, 1u));
     const ApplyTile T = A.tiles[t];
     switch (T.p) {
       case 1: apply3_tile<1, BR2>(A, T, t, smem, red); break;
@@ -179,6 +188,7 @@ __global__ void __launch_bounds__(kThreads3) apply3_kernel(const ApplyArgs A) {
       default: break;
     }
     __syncthreads();
+    t = s_next[par];
   }
   apply_exit<kThreads3>(A, red);
 }
@@ -247,8 +257,9 @@ ApplyArgs make_apply_args(const dg_mesh& M, const double* x, double* y, Reduce r
   A.sfb = M.d_sfb;
   A.sfm3 = M.d_sfm3;
   A.erec3 = M.d_erec3;
-  A.hang3 = reinterpret_cast<const int2*>(M.d_hang3);
-  A.side3 = reinterpret_cast<const int4*>(M.d_side3);
+  A.hang3 = M.d_hang3;
+  A.hang_tiles = M.d_hang_tiles;
+  A.side3 = reinterpret_cast<const int2*>(M.d_side3);
   A.xm = M.d_xm;
   for (int p = 0; p <= kMaxP; ++p) A.moff3[p] = M.moff3[p];
   A.tab = M.d_tables;
@@ -317,9 +328,18 @@ int apply_kernel_setup(const dg_mesh& M) {
   return sms * (per > 0 ? per : 1);
 }
 
+static void launch_hang3(const dg_mesh& M, const ApplyArgs& A, cudaStream_t s) {
+  const int g = (int)M.h_hang_tiles.size();
+  if (g == 0) return;
+  const size_t smem = (size_t)M.hang3_smem;
+  if (M.opts.form == DG_FORM_BR2) launch_k(hang3_kernel<true>, g, kThreads3, smem, s, A);
+  else launch_k(hang3_kernel<false>, g, kThreads3, smem, s, A);
+}
+
 static void launch_modal3(const dg_mesh& M, const ApplyArgs& A, cudaStream_t s) {
   launch_k(modal3_kernel<false>, M.n_tiles, kThreads3, (size_t)M.modal3_smem, s, A, (double*)nullptr,
            (const double*)nullptr, (double*)nullptr, (cudaGraphConditionalHandle)0, 0, 0);
+  launch_hang3(M, A, s);
 }
 
 void launch_trace(const dg_mesh& M, const double* x, cudaStream_t s) {
@@ -361,6 +381,7 @@ void launch_modal3_update(const dg_mesh& M, double* p, const double* z, double* 
   const ApplyArgs A = make_apply_args(M, p, nullptr, Reduce{});
   launch_k(modal3_kernel<true>, M.n_tiles, kThreads3, (size_t)M.modal3_smem, s, A, p, z, sc,
            (cudaGraphConditionalHandle)cond_handle, use_cond, first);
+  launch_hang3(M, A, s);
   DG_CUDA(cudaGetLastError());
 }
 

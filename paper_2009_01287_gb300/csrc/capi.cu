@@ -56,7 +56,6 @@ void upload_tiles(dg_mesh* M, cudaStream_t s) {
   if (M->host.dim == 3) {
     M->d_sfm3 = a.upload(M->h_sfm3, s);
     M->d_erec3 = a.upload(M->h_erec3, s);
-    M->d_hang3 = a.upload(M->h_hang3, s);
     M->d_side3 = a.upload(M->h_side3, s);
   }
   DG_CUDA(cudaStreamSynchronize(s));
@@ -83,6 +82,8 @@ void upload_mesh(dg_mesh* M, cudaStream_t s) {
     if (m.dim == 3) {
       M->d_tr = a.alloc<double>(2 * M->n_trace3);
       M->d_xm = a.alloc<double>(M->n_dofs);
+      M->d_hang3 = a.upload(M->h_hang3, s);
+      M->d_hang_tiles = a.upload(M->h_hang_tiles, s);
     } else {
       M->d_toff = a.upload(toff, s);
       M->d_tr = a.alloc<double>(toff[m.n]);

@@ -103,24 +103,38 @@ struct SubFaceRec3 {
   double area;       // physical area of the sub-face
 };
 
-// The same sub-face as the kernels read it, in the Legendre modes of its two
-// sides (records in tile order: by element of the tile, side and sub-face).
-// In the orthonormal modes of the sub-face itself, with J = u- - u+ and
-// F = dn- - dn+ (both sides' outward derivatives), the residual over a h is
-//   r = cz J + cf F + (BR2) the two liftings,  c2 = cc J,
-// both returned to the own side's modes through R^T when it is larger.
+// A same-size or boundary sub-face as the kernels read it, in the Legendre
+// modes of its side (in tile order, by element of the tile and side).  With
+// J = u- - u+ and F = dn- - dn+ (both sides' outward derivatives) the residual
+// over a h is r = cz J + cf F and the normal-derivative coefficient c2 = cc J,
+// mode by mode.
 struct SubFaceModal3 {
-  int32_t nb;        // neighbour element, -1 on the boundary
-  int32_t pn;        // neighbour degree
-  int32_t nbr_off;   // the other side's trace on the sub-face (double2 units in the trace buffer)
-  int32_t own_off;   // the own trace on the sub-face
-  int32_t tab_ra, tab_rb;   // larger own side: R per tangential axis (rows of kMaxN)
-  int32_t tab_sa, tab_sb;   // BR2, hanging: S = R R^T of the larger side's degree
+  int32_t nn;        // neighbour degree + 1, 0 on the boundary
+  int32_t nbr_off;   // the neighbour's trace (double2 units in the trace buffer)
+  int32_t own_off;   // the own trace
+  int32_t pad;
   double cz;         // SIPG: sigma area; BR2: the own lifting's factor
-  double cx;         // BR2: the neighbour lifting's factor
-  double czx;        // factor of J on modes both sides have (whole faces of both: cz + cx, else cz)
+  double czx;        // BR2, modes both sides have: plus the neighbour lifting's
   double cf, cc;
 };
+// A sub-face between a larger and a smaller side (J, F seen from the larger).
+struct HangPair {
+  int32_t src_b, src_s;     // traces of the larger and the smaller side
+  int32_t dst_b, dst_s;     // results (r, c2) of either
+  int32_t tab_ra, tab_rb;   // R per tangential axis (rows of kMaxN)
+  int32_t ns;               // the smaller element's degree + 1
+  int32_t pad;
+  double cz_b, cx_b, cf_b, cc_b;   // larger side: own and neighbour lifting (SIPG: cz = sigma area), F, c2
+  double cz_s, cx_s, cf_s, cc_s;   // smaller side
+};
+// a CTA's share of the pairs: one degree p of the larger side
+struct HangTile {
+  int32_t p, first, count;
+  int32_t ns;               // largest ns of the tile
+};
+// pairs per tile: one line of u or dn per thread
+constexpr int hang3_pairs(int p) { return kThreads3 / (2 * (p + 1)); }
+constexpr int hang3_doubles(int p) { return 4 * (p + 1) * (p + 1); }   // per pair
 // per element in tile order
 struct ElemRec3 {
   int64_t off;       // first DOF
@@ -129,8 +143,8 @@ struct ElemRec3 {
   double ah, aih;    // a h, a / h
 };
 
-// Shared-memory budget (doubles) of one 3D operator tile; the host sizes the
-// tiles and their rounds of hanging sub-faces so that every one fits.
+// Shared-memory budget (doubles) of one 3D operator tile; the tiles' element
+// counts grow and shrink with it.
 constexpr int kApply3Budget = 9 * 1024;
 // elements of degree p a tile takes at most: about one line of nodes (or
 // modes) per thread of the CTA in every volume pass, whole warps of them
@@ -146,10 +160,6 @@ constexpr int modal3_doubles(int p) {
 constexpr int apply3_elem_doubles(int p) {
   return 2 * (p + 1) * (p + 1) * (p + 1) + 12 * (p + 1) * (p + 1);
 }
-// doubles per sub-face smaller than the own side, and per sub-face of a larger
-// neighbour (BR2; nq = the tile's largest neighbour degree or its own, plus 1)
-constexpr int apply3_own_doubles(int p) { return 4 * (p + 1) * (p + 1); }
-constexpr int apply3_nbr_doubles(int p, int nq) { return nq * nq + (p + 1) * nq; }
 
 // Offsets of the degree-p 1D matrices inside the device table buffer.
 struct BasisOff {
@@ -162,11 +172,7 @@ struct ApplyTile {
   int32_t first;     // index into the degree-sorted element order
   int32_t count;
   int32_t inst;      // batch instance of the tile's elements (0 for a single mesh)
-  int32_t nq;        // 3D: max(p, neighbour degrees) + 1 over the tile
   int32_t chunk;     // 3D: sub-face items sorted together (the whole tile)
-  int32_t hang;      // 3D: first entry of the tile's hanging sub-faces
-  int32_t n_c, n_b;  // 3D: sub-faces smaller than the own side; then, BR2, of larger neighbours
-  int32_t cap_c, cap_b;   // 3D: how many of each a round takes
 };
 
 // ------------------------------------------------------------------ mapped squares

@@ -114,19 +114,19 @@ struct dg_mesh {
   std::vector<dg::SubFaceRec> h_sf;
   std::vector<dg::SubFaceBr2> h_sfb;    // square meshes, BR2: one per h_sf record
   std::vector<dg::SubFaceRec3> h_sf3;   // cube meshes
-  // cube meshes, for the kernels: the sub-face records in tile order, element
-  // records in tile order, per tile its hanging sub-faces (record, local
-  // element * 6 + side), per (order position, side) {first record, first
-  // hanging entry of the tile, their count or 0, 0}
+  // cube meshes, for the kernels: same-size and boundary sub-face records and
+  // element records in tile order, the hanging pairs and their tiles, and per
+  // (order position, side) {record, 0} or {first result, number of pairs}
   std::vector<dg::SubFaceModal3> h_sfm3;
   std::vector<dg::ElemRec3> h_erec3;
-  std::vector<int32_t> h_hang3;
+  std::vector<dg::HangPair> h_hang3;
+  std::vector<dg::HangTile> h_hang_tiles;
   std::vector<int32_t> h_side3;
   int moff3[dg::kMaxP + 1] = {0};       // modal tables of each degree in h_tables
   std::vector<int32_t> h_toff3;         // cube meshes: trace offset of every element (double2 units)
-  std::vector<int32_t> h_suboff3;       // trace offset per record on a larger own side, else -1
-  std::vector<int32_t> h_rtab3;         // per record {R_a, R_b, S_a, S_b} table offsets of the larger side
-  int64_t n_trace3 = 0;                 // length of the trace buffer (double2)
+  std::vector<int32_t> h_resoff3;       // per record of a hanging sub-face, the offset of its results, else -1
+  int64_t n_trace3 = 0;                 // length of the trace buffer, results included (double2)
+  int64_t hang3_smem = 0;               // dynamic shared memory of the hanging pairs' kernel
   int64_t modal3_smem = 0;              // dynamic shared memory of the modes / traces kernel
   // mapped squares: one record per h_sf record, the volume tables of each
   // degree, the map; the geometric factors at the Gauss points - per element
@@ -187,7 +187,8 @@ struct dg_mesh {
   dg::SubFaceBr2* d_sfb = nullptr;
   dg::SubFaceModal3* d_sfm3 = nullptr;   // cube meshes
   dg::ElemRec3* d_erec3 = nullptr;
-  int32_t* d_hang3 = nullptr;
+  dg::HangPair* d_hang3 = nullptr;
+  dg::HangTile* d_hang_tiles = nullptr;
   int32_t* d_side3 = nullptr;
   double* d_xm = nullptr;       // cube meshes: modes of the operator's argument
   dg::SubFaceMap* d_sfm = nullptr;   // mapped squares

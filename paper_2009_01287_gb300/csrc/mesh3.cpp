@@ -112,14 +112,45 @@ void build_topology3(HostMesh& m) {
   }
 }
 
-// degree-sorted element order and tiles of the 3D operator kernels.  Elements
-// are sorted by (p, nq), descending, nq = max(p, neighbour degrees) + 1; a tile
-// is a run of equal (p, nq) with at most apply3_epb(p) elements (fewer on small
-// meshes, so that two tiles fall to every SM) while its arrays leave room for a
-// round of at least one hanging sub-face of each kind.  The tile's sub-faces
-// are a flat list of (record, side) items; those whose larger side is the
-// element's own or (BR2) the neighbour's make the tile's hanging lists, which
-// the operator kernel takes in rounds that fit the shared-memory budget.
+// factors of a sub-face's terms seen from element k, over a h: own lifting (or
+// the SIPG penalty), the neighbour's lifting, the flux, and c2
+struct FaceScale {
+  double cz, cx, cf, cc;
+};
+static FaceScale face_scale(const dg_mesh& M, int64_t k, const SubFaceRec3& f) {
+  const HostMesh& m = M.host;
+  const double a = m.coef[k], h = M.h_h[k], ia = 1.0 / (a * h);
+  const bool in = f.nb >= 0;
+  const double half = in ? 0.5 : 1.0;
+  FaceScale s{};
+  s.cf = -half * f.area * ia;
+  s.cc = -half * f.area / (h * h);
+  if (M.opts.form != DG_FORM_BR2) {
+    s.cz = f.sigma * f.area * ia;
+    return s;
+  }
+  // both sides' lifting energies carry the larger coefficient of the sub-face
+  const double w = in ? std::max(a, m.coef[f.nb]) : a;
+  const double c = w * M.eta * (in ? 0.25 : 1.0) * f.area * f.area * ia;
+  s.cz = c * (basis1d(m.p[k]).Minv[0] / (h * h * h));
+  if (in) {
+    const double hn = M.h_h[f.nb];
+    s.cx = c * (basis1d(f.pn).Minv[0] / (hn * hn * hn));
+  }
+  return s;
+}
+
+// Tiles per SM below which a mesh's tiles are halved: 430k unknowns (779 tiles
+// unhalved) took 90.6 us per apply with at least 2 or 4, 96.9 with 6 and 112
+// with 16 (half-empty warps); 147k unknowns 50.4 / 51.0 / 49.2 / 53.5.
+constexpr int kTilesPerSm = 3;
+
+// degree-sorted element order and tiles of the 3D operator kernels.  A tile is
+// a run of elements of equal (p, nq), nq = max(p, neighbour degrees) + 1, both
+// descending, of at most apply3_epb(p) elements (scaled with the tile's
+// shared-memory budget, and halved on small meshes until there are kTilesPerSm
+// tiles per SM).  The tile's sub-faces are
+// also listed flat as (record, side) items in host order.
 void build_tiles3(dg_mesh* M) {
   const HostMesh& m = M->host;
   const bool br2 = M->opts.form == DG_FORM_BR2;
@@ -137,18 +168,18 @@ void build_tiles3(dg_mesh* M) {
     if (m.p[a] != m.p[b]) return m.p[a] > m.p[b];
     return nq[a] > nq[b];
   });
-  // elements per tile: halved while the mesh gives fewer tiles than two per SM
-  int epb[kMaxP + 1], div = 1;
-  for (;; div *= 2) {
+  // elements per tile: halved while the mesh gives fewer tiles than kTilesPerSm per SM
+  int epb[kMaxP + 1];
+  for (int div = 1;; div *= 2) {
     int64_t cnt[kMaxP + 1] = {0}, tiles = 0;
     for (int64_t k = 0; k < m.n; ++k) ++cnt[m.p[k]];
     bool more = false;
     for (int p = 1; p <= kMaxP; ++p) {
-      epb[p] = std::max(1, apply3_epb(p) / div);
+      epb[p] = std::max(1, (int)(apply3_epb(p) * M->apply3_budget / (kApply3Budget * div)));
       more = more || (cnt[p] > 0 && epb[p] > 1);
       tiles += (cnt[p] + epb[p] - 1) / epb[p];
     }
-    if (tiles >= 304 || !more) break;
+    if (tiles >= kTilesPerSm * 152 || !more) break;
   }
   M->h_tiles.clear();
   M->h_items.clear();
@@ -156,27 +187,17 @@ void build_tiles3(dg_mesh* M) {
   M->h_side_items.assign(12 * (size_t)m.n, 0);
   M->h_sfm3.clear();
   M->h_erec3.clear();
-  M->h_hang3.clear();
-  M->h_side3.assign(24 * (size_t)m.n, 0);
+  M->h_side3.assign(12 * (size_t)m.n, 0);
   M->apply3_smem = 0;
   M->modal3_smem = 0;
   for (int64_t i = 0; i < m.n;) {
     const int P = m.p[order[i]], Q = nq[order[i]], N2 = (P + 1) * (P + 1);
-    const int fixed_per = apply3_elem_doubles(P);
-    const int own_per = apply3_own_doubles(P), nbr_per = apply3_nbr_doubles(P, Q);
     int64_t j = i;
-    while (j < m.n && m.p[order[j]] == P && nq[order[j]] == Q && j - i < epb[P]) {
-      const int64_t need = modal3_doubles(P) + (j - i + 1) * fixed_per + own_per + nbr_per;
-      if (need > M->apply3_budget && j > i) break;
-      ++j;
-    }
+    while (j < m.n && m.p[order[j]] == P && nq[order[j]] == Q && j - i < epb[P]) ++j;
     ApplyTile T{};
     T.p = P;
     T.first = (int32_t)i;
     T.count = (int32_t)(j - i);
-    T.nq = Q;
-    T.hang = (int32_t)(M->h_hang3.size() / 2);
-    std::vector<std::pair<int32_t, int32_t>> own, nbr;   // (record, side) of the hanging lists
     for (int64_t e = 0; e < T.count; ++e) {
       const int64_t pos = i + e;
       const int32_t k = order[pos];
@@ -186,83 +207,32 @@ void build_tiles3(dg_mesh* M) {
         const int b = m.sf_ptr[6 * (int64_t)k + s], c = m.sf_ptr[6 * (int64_t)k + s + 1] - b;
         M->h_side_items[12 * pos + 2 * s] = (int32_t)(M->h_items.size() / 2);
         M->h_side_items[12 * pos + 2 * s + 1] = c;
-        int32_t* sd = &M->h_side3[24 * pos + 4 * s];
-        sd[0] = (int32_t)M->h_sfm3.size();
-        sd[1] = (int32_t)own.size();
-        sd[2] = 0;
         for (int q = 0; q < c; ++q) {
           M->h_items.push_back(b + q);
           M->h_items.push_back((int32_t)(6 * e + s));
-          const SubFaceRec3& f = M->h_sf3[b + q];
-          const int32_t es = (int32_t)(6 * e + s), rec = (int32_t)M->h_sfm3.size();
-          const bool in = f.nb >= 0, mine = !(f.full & 1), his = in && !(f.full & 2);
-          if (mine) {
-            own.push_back({rec, es});
-            ++sd[2];
-          }
-          if (his && br2) nbr.push_back({rec, es});
-          // the record in modes, scaled by 1 / (a h)
-          SubFaceModal3 r{};
-          r.nb = f.nb;
-          r.pn = f.pn;
-          r.own_off = mine ? M->h_suboff3[b + q] : M->h_toff3[k] + s * N2;
-          const double ia = 1.0 / (a * h), half = in ? 0.5 : 1.0;
-          r.cf = -half * f.area * ia;
-          r.cc = -half * f.area / (h * h);
-          if (in) {
-            int back = -1;   // the same sub-face seen from the neighbour
-            for (int g = m.sf_ptr[6 * (int64_t)f.nb + f.nb_side]; g < m.sf_ptr[6 * (int64_t)f.nb + f.nb_side + 1]; ++g)
-              if (m.sf3[g].nb == k) back = g;
-            r.nbr_off = his ? M->h_suboff3[back] : M->h_toff3[f.nb] + f.nb_side * (f.pn + 1) * (f.pn + 1);
-            const int32_t* tb = mine ? &M->h_rtab3[4 * (size_t)(b + q)] : his ? &M->h_rtab3[4 * (size_t)back] : nullptr;
-            if (tb) {
-              r.tab_ra = tb[0];
-              r.tab_rb = tb[1];
-              r.tab_sa = tb[2];
-              r.tab_sb = tb[3];
-            }
-          }
-          if (br2) {
-            // both sides' lifting energies carry the larger coefficient of the sub-face
-            const double w = in ? std::max(a, m.coef[f.nb]) : a;
-            const double c0 = w * M->eta * (in ? 0.25 : 1.0) * f.area * f.area * ia;
-            r.cz = c0 * (basis1d(P).Minv[0] / (h * h * h));
-            r.czx = r.cz;
-            if (in) {
-              const double hn = M->h_h[f.nb];
-              r.cx = c0 * (basis1d(f.pn).Minv[0] / (hn * hn * hn));
-              if (!mine && !his) r.czx = r.cz + r.cx;
-            }
-          } else {
-            r.cz = f.sigma * f.area * ia;
-          }
-          M->h_sfm3.push_back(r);
         }
+        int32_t* sd = &M->h_side3[12 * pos + 2 * s];
+        if (M->h_resoff3[b] >= 0) {   // hanging: its results, one after another
+          sd[0] = M->h_resoff3[b];
+          sd[1] = c;
+          continue;
+        }
+        const SubFaceRec3& f = M->h_sf3[b];
+        SubFaceModal3 r{};
+        r.own_off = M->h_toff3[k] + s * N2;
+        if (f.nb >= 0) {
+          r.nn = f.pn + 1;
+          r.nbr_off = M->h_toff3[f.nb] + f.nb_side * r.nn * r.nn;
+        }
+        const FaceScale fs = face_scale(*M, k, f);
+        r.cz = fs.cz;
+        r.czx = fs.cz + fs.cx;
+        r.cf = fs.cf;
+        r.cc = fs.cc;
+        sd[0] = (int32_t)M->h_sfm3.size();
+        M->h_sfm3.push_back(r);
       }
     }
-    // the neighbours' liftings by descending neighbour degree, so that a warp
-    // spans few loop bounds
-    std::stable_sort(nbr.begin(), nbr.end(), [&](const std::pair<int32_t, int32_t>& x, const std::pair<int32_t, int32_t>& y) {
-      return M->h_sfm3[x.first].pn > M->h_sfm3[y.first].pn;
-    });
-    for (const auto* l : {&own, &nbr})
-      for (const auto& v : *l) {
-        M->h_hang3.push_back(v.first);
-        M->h_hang3.push_back(v.second);
-      }
-    T.n_c = (int32_t)own.size();
-    T.n_b = (int32_t)nbr.size();
-    const int64_t fixed = modal3_doubles(P) + (j - i) * (int64_t)fixed_per;
-    // rounds: all at once if they fit, else the same number of rounds for both
-    const int64_t room = M->apply3_budget - fixed;
-    int64_t rounds = 1, need = 0;
-    auto per = [&](int64_t n) { return (n + rounds - 1) / rounds; };
-    for (;; ++rounds) {
-      need = per(T.n_c) * own_per + per(T.n_b) * nbr_per;
-      if (need <= room || (per(T.n_c) <= 1 && per(T.n_b) <= 1)) break;
-    }
-    T.cap_c = (int32_t)std::max<int64_t>(1, per(T.n_c));
-    T.cap_b = (int32_t)std::max<int64_t>(1, per(T.n_b));
     // Host order of the items: by the branches their threads take - interior
     // first, then the BR2 whole-face flags, then the neighbour degree; the high
     // half of the side field keeps the item's position in sub-face order.
@@ -289,9 +259,8 @@ void build_tiles3(dg_mesh* M) {
       }
     }
     M->h_item_ptr.push_back((int32_t)(M->h_items.size() / 2));
-    M->apply3_smem = std::max<int64_t>(M->apply3_smem, 8 * (fixed + T.cap_c * (int64_t)own_per + T.cap_b * (int64_t)nbr_per));
-    M->modal3_smem = std::max<int64_t>(
-        M->modal3_smem, 8 * (modal3_doubles(P) + T.count * (int64_t)N2 * (P + 1) + T.cap_c * 2 * (int64_t)N2));
+    M->apply3_smem = std::max<int64_t>(M->apply3_smem, 8 * (modal3_doubles(P) + T.count * (int64_t)apply3_elem_doubles(P)));
+    M->modal3_smem = std::max<int64_t>(M->modal3_smem, 8 * (modal3_doubles(P) + T.count * (int64_t)N2 * (P + 1)));
     M->h_tiles.push_back(T);
     i = j;
   }
@@ -299,12 +268,11 @@ void build_tiles3(dg_mesh* M) {
   M->h_order = order;
 }
 
-// Trace offsets of every element's sides and, on sides with smaller
-// neighbours, of every sub-face; and the restriction tables of those (after
-// the records).
+// Trace offsets of every element's sides, result offsets of both sides of
+// every hanging sub-face, and the hanging pairs with their restriction tables
+// and tiles (after the records).
 static void build_modal3(dg_mesh* M) {
   const HostMesh& m = M->host;
-  const bool br2 = M->opts.form == DG_FORM_BR2;
   for (int p = 1; p <= kMaxP; ++p) {
     M->moff3[p] = (int)M->h_tables.size();
     modal_tables(p, M->h_tables);
@@ -317,52 +285,80 @@ static void build_modal3(dg_mesh* M) {
     at += 6 * (m.p[k] + 1) * (m.p[k] + 1);
     DG_REQUIRE(at < (1LL << 31), "too many side traces");
   }
-  M->h_suboff3.assign(m.sf3.size(), -1);
-  M->h_rtab3.assign(4 * m.sf3.size(), 0);
-  std::map<std::tuple<int, int, int>, int> index;   // (0 or degree + 1, level, position)
-  auto table = [&](int p, int L, int o) {
-    const auto key = std::make_tuple(p, L, o);
-    const auto it = index.find(key);
-    if (it != index.end()) return it->second;
-    double R[kMaxN * kMaxN];
-    modal_restriction(L, o, R);
-    const int n = p, at0 = (int)M->h_tables.size();
-    if (p == 0) {
-      M->h_tables.insert(M->h_tables.end(), R, R + kMaxN * kMaxN);
-    } else {   // S = R R^T on the first p modes
-      for (int i = 0; i < n; ++i)
-        for (int j = 0; j < n; ++j) {
-          double v = 0.0;
-          for (int q = std::max(i, j); q < n; ++q) v += R[i * kMaxN + q] * R[j * kMaxN + q];
-          M->h_tables.push_back(v);
-        }
+  M->h_resoff3.assign(m.sf3.size(), -1);
+  for (int64_t k = 0; k < m.n; ++k)
+    for (int j = m.sf_ptr[6 * k]; j < m.sf_ptr[6 * k + 6]; ++j) {
+      const auto& f = m.sf3[j];
+      if (f.nb < 0 || m.size[f.nb] == m.size[k]) continue;
+      M->h_resoff3[j] = (int32_t)at;
+      at += (m.p[k] + 1) * (m.p[k] + 1);
+      DG_REQUIRE(at < (1LL << 31), "too many side traces");
     }
-    index.emplace(key, at0);
+  M->n_trace3 = at;
+  std::map<std::pair<int, int>, int> index;   // (level, position) -> R
+  auto table = [&](int L, int o) {
+    const auto it = index.find({L, o});
+    if (it != index.end()) return it->second;
+    const int at0 = (int)M->h_tables.size();
+    M->h_tables.resize(at0 + kMaxN * kMaxN);
+    modal_restriction(L, o, M->h_tables.data() + at0);
+    index[{L, o}] = at0;
     return at0;
   };
+  std::vector<std::pair<int, HangPair>> pairs;   // by the larger side's degree
   for (int64_t k = 0; k < m.n; ++k)
     for (int s = 0; s < 6; ++s) {
       int ax, ta, tb;
       side_axes3(s, ax, ta, tb);
       for (int j = m.sf_ptr[6 * k + s]; j < m.sf_ptr[6 * k + s + 1]; ++j) {
         const auto& f = m.sf3[j];
-        if (f.len == m.size[k]) continue;
-        const int L = ilog2(m.size[k] / f.len), n = m.p[k] + 1;
-        const int oa = (f.a0 - m.lo[3 * k + ta]) / f.len, ob = (f.b0 - m.lo[3 * k + tb]) / f.len;
-        M->h_suboff3[j] = (int32_t)at;
-        at += n * n;
-        DG_REQUIRE(at < (1LL << 31), "too many side traces");
-        int32_t* t = &M->h_rtab3[4 * (size_t)j];
-        t[0] = table(0, L, oa);
-        t[1] = table(0, L, ob);
-        if (br2) {
-          t[2] = table(n, L, oa);
-          t[3] = table(n, L, ob);
-        }
+        if (f.len == m.size[k]) continue;   // seen from the larger side
+        const int L = ilog2(m.size[k] / f.len), N2 = (m.p[k] + 1) * (m.p[k] + 1);
+        int back = -1;   // the same sub-face seen from the smaller side
+        for (int g = m.sf_ptr[6 * (int64_t)f.nb + f.nb_side]; g < m.sf_ptr[6 * (int64_t)f.nb + f.nb_side + 1]; ++g)
+          if (m.sf3[g].nb == k) back = g;
+        DG_REQUIRE(back >= 0 && M->h_resoff3[back] >= 0, "hanging sub-face without a smaller side");
+        HangPair h{};
+        h.ns = m.p[f.nb] + 1;
+        h.src_b = M->h_toff3[k] + s * N2;
+        h.src_s = M->h_toff3[f.nb] + f.nb_side * h.ns * h.ns;
+        h.dst_b = M->h_resoff3[j];
+        h.dst_s = M->h_resoff3[back];
+        h.tab_ra = table(L, (f.a0 - m.lo[3 * k + ta]) / f.len);
+        h.tab_rb = table(L, (f.b0 - m.lo[3 * k + tb]) / f.len);
+        const FaceScale b = face_scale(*M, k, M->h_sf3[j]), t = face_scale(*M, f.nb, M->h_sf3[back]);
+        h.cz_b = b.cz;
+        h.cx_b = b.cx;
+        h.cf_b = b.cf;
+        h.cc_b = b.cc;
+        h.cz_s = t.cz;
+        h.cx_s = t.cx;
+        h.cf_s = t.cf;
+        h.cc_s = t.cc;
+        pairs.push_back({m.p[k], h});
       }
     }
   DG_REQUIRE(M->h_tables.size() < (1ULL << 31), "face tables too large");
-  M->n_trace3 = at;
+  std::stable_sort(pairs.begin(), pairs.end(), [](const std::pair<int, HangPair>& a, const std::pair<int, HangPair>& b) {
+    return a.first != b.first ? a.first > b.first : a.second.ns > b.second.ns;
+  });
+  M->h_hang3.clear();
+  M->h_hang_tiles.clear();
+  M->hang3_smem = 0;
+  // fewer pairs per tile on small meshes (whole warps of them)
+  int div = 1;
+  while (div < 4 && (int64_t)pairs.size() < kTilesPerSm * 152 * 12 / div) div *= 2;
+  for (size_t i = 0; i < pairs.size();) {
+    const int P = pairs[i].first;
+    HangTile T{P, (int32_t)i, 0, pairs[i].second.ns};
+    while (i < pairs.size() && pairs[i].first == P && T.count < std::max(1, hang3_pairs(P) / div)) {
+      M->h_hang3.push_back(pairs[i].second);
+      ++T.count;
+      ++i;
+    }
+    M->h_hang_tiles.push_back(T);
+    M->hang3_smem = std::max<int64_t>(M->hang3_smem, 8LL * T.count * hang3_doubles(P));
+  }
 }
 
 void build_mesh_host3(dg_mesh* M, const dg_mesh_desc* desc, const dg_options& o) {
@@ -461,7 +457,7 @@ void build_mesh_host3(dg_mesh* M, const dg_mesh_desc* desc, const dg_options& o)
   const bool br2 = o.form == DG_FORM_BR2;
   double fma = 0.0;
   for (int64_t k = 0; k < m.n; ++k) {
-    const double a = m.p[k] + 1.0, a2 = a * a, a3 = a2 * a;
+    const double a = m.p[k] + 1.0, a2 = a * a;
     const double H = std::floor(a / 2), C = a - H;
     const double line = C * C + H * H + 2.0 * H;                       // one line between nodes and modes
     const double stiff = H * H + (C - 1.0) * (C - 1.0);                // one line's stiffness
@@ -470,10 +466,8 @@ void build_mesh_host3(dg_mesh* M, const dg_mesh_desc* desc, const dg_options& o)
       const auto& f = m.sf3[j];
       fma += 5.0 * a2;
       if (f.nb < 0) continue;
-      const double b = m.p[f.nb] + 1.0;
       const double tri = a2 * (a + 1.0);                               // R or R^T in both directions
-      if (f.len != m.size[k]) fma += 4.0 * tri + (br2 ? 2.0 * a3 : 0.0);
-      else if (f.len != m.size[f.nb] && br2) fma += std::min(a, b) * b * (b + std::min(a, b));
+      if (f.len != m.size[k]) fma += (br2 ? 5.0 : 4.0) * tri;
       const int lg = std::abs(ilog2(m.size[k]) - ilog2(m.size[f.nb]));
       S.max_level_gap = std::max<int64_t>(S.max_level_gap, lg);
     }
