@@ -35,20 +35,24 @@ struct DevArena {
   }
 };
 
-// CSR on the device: int32 indices, values of the preconditioner precision
+// A sparse matrix on the device in slices (SlicePlan): int32 columns, values of
+// the preconditioner precision.
+struct DevSlices {
+  int64_t rows = 0, nnz = 0;
+  int32_t* hdr = nullptr;    // 4 per slice: first entry / 32, rounds, lanes per row, first slot of `row`
+  int32_t* row = nullptr;    // matrix row of every slot, -1: none
+  int32_t* idx = nullptr;    // column of every lane's entry, round by round, -1: none
+  void* val = nullptr;
+  int n_cta = 0;             // the first n_cta slices take a whole CTA (one row each)
+  int n_warp = 0;            // slices after them, one warp each
+};
+
+// CSR on the device (the prolongation P)
 struct DevCsr {
   int64_t rows = 0, nnz = 0;
   int32_t* ptr = nullptr;
   int32_t* idx = nullptr;
   void* val = nullptr;
-  int group = 1;       // lanes per row in the group tier (power of two <= 32)
-  int group_all = 1;   // lanes per row of the fused AMG up-sweep (set per level from the mean row length)
-  // rows read by a whole CTA (more than kCsrCtaRow entries) and by a whole
-  // warp (more than long_min entries); the group tier skips both
-  int32_t* cta_rows = nullptr;
-  int32_t* warp_rows = nullptr;
-  int n_cta = 0, n_warp = 0;
-  int long_min = 0x7fffffff;
 };
 
 // lanes per row for a CSR with the given average row length
@@ -63,25 +67,19 @@ constexpr int kCsrCtaRow = 1024;
 // threads resident on the whole GPU at full occupancy (152 SMs x 2048)
 constexpr int64_t kResidentThreads = 152 * 2048;
 
-// the CTA and warp tiers of a CSR row kernel launch (see DevCsr)
-struct CsrTiers {
-  const int32_t* cta_rows;
-  const int32_t* warp_rows;
-  int n_cta, n_warp;
-  int long_min;
-};
-
 struct DevLevel {
   int64_t n = 0;
   int64_t n_cont = 0;  // rows [0, n_cont) continue to the next level (smoothed,
                        // restricted); rows [n_cont, n) are coarsest levels of
                        // their problem and are solved densely (blocks below)
-  DevCsr Rpre, Sb, Sp;  // composite V-cycle operators on the continuing rows (see AmgLevel)
+  // composite V-cycle operators on the continuing rows (see AmgLevel): Rpre, and
+  // [Sb | Sp] as one matrix (columns from n_cont on are the next level's)
+  DevSlices Rpre, S;
   // large levels take the plain form instead (fewer matrix bytes, two more
   // launches): A on the continuing rows, R = P^T, P, the l1 diagonal inverse
   // and two work vectors
   bool plain = false;
-  DevCsr A, R, P;
+  DevSlices A, R, P;
   void* dinv = nullptr;
   void* t1 = nullptr;
   void* t2 = nullptr;
@@ -225,7 +223,8 @@ struct dg_precond {
   int64_t n_dofs = 0, n_c = 0;
   dg_precond_stats stats{};
   dg::DevArena arena;
-  dg::DevCsr P, PT;          // P: n_dofs x n_c (rows = DG nodes), PT = P^T
+  dg::DevCsr P;           // n_dofs x n_c (rows = DG nodes)
+  dg::DevSlices PT;          // P^T
   void* dinv = nullptr;      // n_dofs, 1/A_jj on V_J and 0 elsewhere
   int32_t* e_pos = nullptr;     // n_dofs, slot of the node's result in zE, or -1 outside the V_e
   // block-solve work units, largest blocks first: one per 32-row panel of a

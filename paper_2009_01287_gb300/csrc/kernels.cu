@@ -10,65 +10,76 @@ namespace dg {
 
 // ============================================================== preconditioner
 
-// ---- CSR row kernels in three tiers (the rows of P^T and of the AMG levels
-// are very uneven): rows longer than kCsrCtaRow entries take one CTA each
-// (entries strided over the CTA, fixed block tree), rows longer than
-// long_min take one warp each (fixed shuffle tree), and the rest are read by
-// G lanes per row (fixed shuffle tree over G).  The grid holds the CTA-tier
-// CTAs first, then the warp tier (8 rows per CTA), then the group tier, whose
-// row loop advances by whole warps so that every lane reaches the shuffles.
-// Every sum has a fixed order, so the results are deterministic.
-template <typename T, int G, class Op>
+// ---- Sparse rows in slices (DevSlices).  One warp per slice: every round is
+// one coalesced load of 32 columns and 32 values, four rounds in flight, then
+// the gathers; a row's lanes are added by a fixed shuffle tree.  Slices come
+// longest first and a row has at most 16 rounds (32 lanes and up to 32 rounds
+// for the longest, a whole CTA above kCsrCtaRow entries), so no row sets the
+// length of the launch: with CSR rows of a fixed number of lanes the up-sweep
+// of a 45k-row cube level (42 entries per row on average, 2,000 at most) took
+// 81 us for 41 MB.  The first slice's columns and values are loaded before the
+// wait for the preceding kernel: no kernel writes them.  Every sum has a fixed
+// order, so the results are deterministic.
+constexpr int kRoundsInFlight = 4;
+template <typename T, class Op>
 __global__ void __launch_bounds__(kVecThreads)
-csr_rows_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ idx,
-                const T* __restrict__ val, int64_t rows, CsrTiers tiers, const Op op_arg) {
-  pdl_entry();
-  const Op op = op_arg.bind();   // per-thread values an operation loads once (after the wait)
-  int bid = blockIdx.x;
-  if (bid < tiers.n_cta) {
-    __shared__ double sred[kVecThreads];
-    const int row = __ldg(tiers.cta_rows + bid);
-    const int e = ptr[row + 1];
-    T s = 0;
-    for (int t = ptr[row] + threadIdx.x; t < e; t += kVecThreads) s += __ldg(val + t) * op.x(__ldg(idx + t));
-    pdl_trigger();
-    const double tot = block_sum<kVecThreads>((double)s, sred);
-    if (threadIdx.x == 0) op.store(row, (T)tot);
-    return;
-  }
-  bid -= tiers.n_cta;
-  const int warp_ctas = (tiers.n_warp + 7) >> 3;
-  if (bid < warp_ctas) {
-    const int w = bid * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (w >= tiers.n_warp) return;   // whole warps leave together
-    const int row = __ldg(tiers.warp_rows + w);
-    const int e = ptr[row + 1];
-    T s = 0;
-    for (int t = ptr[row] + lane; t < e; t += 32) s += __ldg(val + t) * op.x(__ldg(idx + t));
+slice_rows_kernel(const int4* __restrict__ hdr, const int32_t* __restrict__ rows, const int32_t* __restrict__ idx,
+                  const T* __restrict__ val, int n_cta, int n_warp, const Op op_arg) {
+  constexpr int U = kRoundsInFlight;
+  __shared__ double sred[kVecThreads];
+  const bool wide = (int)blockIdx.x < n_cta;   // one row per CTA
+  const int width = wide ? kVecThreads : 32, lane = threadIdx.x % width;
+  const int step = wide ? n_cta + n_warp : (gridDim.x - n_cta) * (kVecThreads / 32);
+  int s = wide ? blockIdx.x : n_cta + (blockIdx.x - n_cta) * (kVecThreads / 32) + threadIdx.x / 32;
+  int j[U];
+  T a[U];
+  int4 h = make_int4(0, 0, 1, 0);
+  const int32_t* ip = idx;
+  const T* vp = val;
+  auto load = [&](int k) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) op.store(row, s);
-    return;
-  }
-  bid -= warp_ctas;
-  const int nb = gridDim.x - tiers.n_cta - warp_ctas;
-  const int lane = threadIdx.x % G;
-  const int64_t groups_per_grid = ((int64_t)nb * blockDim.x) / G;
-  const int64_t g0 = (bid * (int64_t)blockDim.x + threadIdx.x) / G;
-  const int64_t rounds = (rows + groups_per_grid - 1) / groups_per_grid;
-  for (int64_t rd = 0; rd < rounds; ++rd) {
-    const int64_t row = g0 + rd * groups_per_grid;
-    T s = 0;
-    bool mine = false;
-    if (row < rows) {
-      const int b = ptr[row], e = ptr[row + 1];
-      mine = e - b <= tiers.long_min;
-      if (mine)
-        for (int t = b + lane; t < e; t += G) s += __ldg(val + t) * op.x(__ldg(idx + t));
+    for (int u = 0; u < U; ++u) {
+      const bool in = k + u < h.y;
+      j[u] = in ? __ldg(ip + (int64_t)(k + u) * width) : -1;
+      a[u] = in ? __ldg(vp + (int64_t)(k + u) * width) : (T)0;
     }
+  };
+  auto open = [&]() {
+    h = __ldg(hdr + s);
+    ip = idx + 32 * (int64_t)h.x + lane;
+    vp = val + 32 * (int64_t)h.x + lane;
+    load(0);
+  };
+  const bool any = s < n_cta + n_warp;
+  if (any) open();
+  pdl_entry();
+  if (!any) return;   // whole warps
+  const Op op = op_arg.bind();   // per-thread values an operation loads once (after the wait)
+  while (true) {
+    T sum = 0;
+    for (int k = 0; k < h.y;) {
+      T x[U];
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, G);
-    if (mine && lane == 0) op.store(row, s);
+      for (int u = 0; u < U; ++u) x[u] = j[u] >= 0 ? op.x(j[u]) : (T)0;
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (j[u] >= 0) sum = fma(a[u], x[u], sum);
+      k += U;
+      if (k < h.y) load(k);
+    }
+    if (wide) {
+      const double tot = block_sum<kVecThreads>((double)sum, sred);
+      if (threadIdx.x == 0) op.store(__ldg(rows + h.w), (T)tot);
+      return;
+    }
+    for (int o = h.z >> 1; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+    if ((lane & (h.z - 1)) == 0) {
+      const int row = __ldg(rows + h.w + lane / h.z);
+      if (row >= 0) op.store(row, sum);
+    }
+    s += step;
+    if (s >= n_cta + n_warp) break;
+    open();
   }
 }
 
@@ -135,27 +146,24 @@ struct OpPost {  // out = xp + D^-1 (b - A xp) (post-smoothing)
   __device__ void store(int64_t i, T s) const { out[i] = fma(dinv[i], b[i] - s, xp[i]); }
 };
 
+template <typename T>
+struct OpUp {  // out = Sb b + Sp xc: columns from n on are the next level's
+  const T* b;
+  const T* xc;
+  T* out;
+  int n;
+  __device__ OpUp bind() const { return *this; }
+  __device__ T x(int j) const { return j < n ? __ldg(b + j) : __ldg(xc + (j - n)); }
+  __device__ void store(int64_t i, T s) const { out[i] = s; }
+};
+
 template <typename T, class Op>
-static void launch_rows(const DevCsr& A, const Op& op, cudaStream_t s) {
+static void launch_rows(const DevSlices& A, const Op& op, cudaStream_t s) {
   if (A.rows == 0) return;
-  int64_t threads = A.rows * (int64_t)A.group;
-  int64_t blocks = (threads + kVecThreads - 1) / kVecThreads;
+  int blocks = (A.n_warp + 7) / 8;
   if (blocks > 8 * 152) blocks = 8 * 152;
-  const int32_t* p = A.ptr;
-  const int32_t* ix = A.idx;
-  const T* v = (const T*)A.val;
-  const CsrTiers tr{A.cta_rows, A.warp_rows, A.n_cta, A.n_warp, A.long_min};
-  const int g = (int)blocks + A.n_cta + (A.n_warp + 7) / 8;
-#define DG_ROWS(G) launch_k(csr_rows_kernel<T, G, Op>, g, kVecThreads, 0, s, p, ix, v, A.rows, tr, op)
-  switch (A.group) {
-    case 1: DG_ROWS(1); break;
-    case 2: DG_ROWS(2); break;
-    case 4: DG_ROWS(4); break;
-    case 8: DG_ROWS(8); break;
-    case 16: DG_ROWS(16); break;
-    default: DG_ROWS(32); break;
-  }
-#undef DG_ROWS
+  launch_k(slice_rows_kernel<T, Op>, A.n_cta + blocks, kVecThreads, 0, s, (const int4*)A.hdr, A.row, A.idx,
+           (const T*)A.val, A.n_cta, A.n_warp, op);
 }
 
 // dense y = Ainv x, one warp per row
@@ -262,10 +270,12 @@ constexpr int kFinalCtasPerSm = 5;
 // when rr is given, the r . r reduction beside it (the PCG residual norm).
 // With a deferred PCG update (xr.q) r is r - alpha q, stored here with
 // x += alpha p: every other reader of r has finished when this kernel runs.
-// G lanes per DG row share its P entries; the row's own terms (r, D_J^-1, the
-// block result) are loaded before the P entries so that both chains of loads
-// are in flight together.
-template <typename T, int G>
+// One lane per DG row, rows in order (P has two to five entries per row; more
+// lanes per row measured slower, and so did rows sorted by length within
+// chunks of 256 and handed over through shared memory: 22 against 16 us on 430k
+// unknowns).  The row's own terms (r, D_J^-1, the block result) are loaded
+// before the P entries so that both chains of loads are in flight together.
+template <typename T>
 __global__ void __launch_bounds__(kVecThreads, kFinalCtasPerSm)
 precond_final_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ idx,
                      const T* __restrict__ val, const T* __restrict__ ec,
@@ -274,43 +284,29 @@ precond_final_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict_
                      double* __restrict__ z, int64_t n, Reduce red, Reduce rr, PcgCtl ctl, XrDefer xr) {
   pdl_entry();
   __shared__ double sred[kVecThreads];
-  const int lane = threadIdx.x % G;
-  const int64_t groups_per_grid = ((int64_t)gridDim.x * blockDim.x) / G;
-  const int64_t g0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G;
-  const int64_t rounds = (n + groups_per_grid - 1) / groups_per_grid;
   double dot = 0.0, dot_rr = 0.0;
-  for (int64_t rd = 0; rd < rounds; ++rd) {
-    const int64_t i = g0 + rd * groups_per_grid;
-    T s = 0, tj = 0, te = 0;
-    double ri = 0.0;
-    bool has_e = false;
-    if (i < n) {
-      if (lane == 0) {
-        if (xr.q) {   // r is rewritten below: plain loads
-          const double a = *xr.alpha;
-          ri = fma(-a, xr.q[i], r[i]);
-          xr.r_out[i] = ri;
-          xr.x[i] = fma(a, xr.p[i], xr.x[i]);
-        } else {
-          ri = __ldg(r + i);
-        }
-        tj = __ldg(dinv + i) * (T)ri;
-        const int ep = __ldg(e_pos + i);
-        has_e = ep >= 0;
-        if (has_e) te = __ldg(zE + ep);
-      }
-      for (int t = ptr[i] + lane; t < ptr[i + 1]; t += G) s += __ldg(val + t) * __ldg(ec + __ldg(idx + t));
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    double ri;
+    if (xr.q) {   // r is rewritten below: plain loads
+      const double a = *xr.alpha;
+      ri = fma(-a, xr.q[i], r[i]);
+      xr.r_out[i] = ri;
+      xr.x[i] = fma(a, xr.p[i], xr.x[i]);
+    } else {
+      ri = __ldg(r + i);
     }
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, G);
-    if (i < n && lane == 0) {
-      s += tj;
-      if (has_e) s += te;
-      const double zi = (double)s;
-      z[i] = zi;
-      dot += zi * ri;
-      dot_rr += ri * ri;
-    }
+    const T tj = __ldg(dinv + i) * (T)ri;
+    const int ep = __ldg(e_pos + i);
+    T te = 0;
+    if (ep >= 0) te = __ldg(zE + ep);
+    T s = 0;
+    for (int t = ptr[i]; t < ptr[i + 1]; ++t) s += __ldg(val + t) * __ldg(ec + __ldg(idx + t));
+    s += tj;
+    if (ep >= 0) s += te;
+    const double zi = (double)s;
+    z[i] = zi;
+    dot += zi * ri;
+    dot_rr += ri * ri;
   }
   pdl_trigger();   // rows done: the next kernel launches during the reductions
   if (rr.partial) {
@@ -362,50 +358,6 @@ int precond_final_blocks(const dg_precond& pc) {
   int64_t b = (pc.n_dofs + kVecThreads - 1) / kVecThreads;   // one lane per row
   if (b > kFinalCtasPerSm * 152) b = kFinalCtasPerSm * 152;   // one resident wave
   return (int)(b < 1 ? 1 : b);
-}
-
-// fused up-sweep of one AMG level: xo = Sb b + Sp xc (G lanes per row share
-// both rows; fixed shuffle tree)
-template <typename T, int G>
-__global__ void __launch_bounds__(kVecThreads)
-amg_up_kernel(const int32_t* __restrict__ bp, const int32_t* __restrict__ bi, const T* __restrict__ bv,
-              const int32_t* __restrict__ pp, const int32_t* __restrict__ pi, const T* __restrict__ pv,
-              const T* __restrict__ b, const T* __restrict__ xc, T* __restrict__ xo, int64_t rows) {
-  pdl_entry();
-  const int lane = threadIdx.x % G;
-  const int64_t groups_per_grid = ((int64_t)gridDim.x * blockDim.x) / G;
-  const int64_t g0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G;
-  const int64_t rounds = (rows + groups_per_grid - 1) / groups_per_grid;
-  for (int64_t rd = 0; rd < rounds; ++rd) {
-    const int64_t row = g0 + rd * groups_per_grid;
-    T s = 0;
-    if (row < rows) {
-      for (int t = bp[row] + lane; t < bp[row + 1]; t += G) s += __ldg(bv + t) * __ldg(b + __ldg(bi + t));
-      for (int t = pp[row] + lane; t < pp[row + 1]; t += G) s += __ldg(pv + t) * __ldg(xc + __ldg(pi + t));
-    }
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, G);
-    if (row < rows && lane == 0) xo[row] = s;
-  }
-}
-
-template <typename T>
-static void launch_up(const DevLevel& L, const T* b, const T* xc, T* xo, cudaStream_t s) {
-  if (L.n_cont == 0) return;
-  int64_t blocks = (L.n_cont * (int64_t)L.Sb.group_all + kVecThreads - 1) / kVecThreads;
-  if (blocks > 8 * 152) blocks = 8 * 152;
-#define DG_UP(G)                                                                                  \
-  launch_k(amg_up_kernel<T, G>, (int)blocks, kVecThreads, 0, s, L.Sb.ptr, L.Sb.idx,              \
-           (const T*)L.Sb.val, L.Sp.ptr, L.Sp.idx, (const T*)L.Sp.val, b, xc, xo, L.n_cont)
-  switch (L.Sb.group_all) {
-    case 1: DG_UP(1); break;
-    case 2: DG_UP(2); break;
-    case 4: DG_UP(4); break;
-    case 8: DG_UP(8); break;
-    case 16: DG_UP(16); break;
-    default: DG_UP(32); break;
-  }
-#undef DG_UP
 }
 
 // y = W x for a dense row-major m x n matrix, one CTA per row (fixed block
@@ -482,12 +434,12 @@ static void vcycle(const dg_precond& pc, size_t l, cudaStream_t s) {
     const int g = (int)std::min<int64_t>(L.coarse_w_rows, 8 * 152);
     launch_k(dense_rect_kernel<T>, g, kVecThreads, 0, s, (const T*)L.coarse_w, (const T*)L.b, (T*)C.xo,
              L.coarse_w_rows, L.n);
-    launch_up<T>(L, (const T*)L.b, (const T*)C.xo, (T*)L.xo, s);    // correction + smoothing
+    launch_rows<T>(L.S, OpUp<T>{(const T*)L.b, (const T*)C.xo, (T*)L.xo, (int)L.n_cont}, s);   // correction + smoothing
   } else if (L.n_cont > 0) {
     const DevLevel& C = pc.levels[l + 1];
     launch_rows<T>(L.Rpre, OpSpmv<T>{(const T*)L.b, (T*)C.b}, s);   // restrict b - A D^-1 b
     vcycle<T>(pc, l + 1, s);
-    launch_up<T>(L, (const T*)L.b, (const T*)C.xo, (T*)L.xo, s);    // correction + smoothing
+    launch_rows<T>(L.S, OpUp<T>{(const T*)L.b, (const T*)C.xo, (T*)L.xo, (int)L.n_cont}, s);   // correction + smoothing
   }
   if (L.n_end > 0 && L.max_end > 0) {
     const int gx = L.n_end < 8 * 152 ? L.n_end : 8 * 152;
@@ -537,20 +489,15 @@ static void precond_impl(const dg_precond& pc, const double* r, double* z, Reduc
   if (mk) DG_CUDA(cudaEventRecord(mk->ev[3], s));
   if (pc.n_blocks > 0 && !mk) DG_CUDA(cudaStreamWaitEvent(s, pc.ev_join, 0));
   const int nb = precond_final_blocks(pc);
-#define DG_FINAL(G)                                                                          \
-  launch_k(precond_final_kernel<T, G>, nb, kVecThreads, 0, s,                                      \
-      pc.P.ptr, pc.P.idx, (const T*)pc.P.val, (const T*)ec, (const T*)pc.dinv, pc.e_pos,     \
-      (const T*)pc.zE, r, z, pc.n_dofs, red, rr, ctl, xr)
-  // one lane per DG row: measured faster than 2 or 4 lanes (P has about five
-  // entries per row; fewer rounds of dependent loads per thread count more)
-  DG_FINAL(1);
-#undef DG_FINAL
+  launch_k(precond_final_kernel<T>, nb, kVecThreads, 0, s, pc.P.ptr, pc.P.idx, (const T*)pc.P.val, (const T*)ec, (const T*)pc.dinv, pc.e_pos, (const T*)pc.zE, r, z, pc.n_dofs, red, rr,
+           ctl, xr);
   DG_CUDA(cudaGetLastError());
   if (mk) DG_CUDA(cudaEventRecord(mk->ev[4], s));
 }
 
-// bytes of a CSR matrix read once: values, column indices, row pointers
-static double csr_bytes(const DevCsr& A, size_t tsz) {
+// bytes of a sparse matrix read once: values, column indices and a row number per row
+template <class M>
+static double csr_bytes(const M& A, size_t tsz) {
   return (double)A.nnz * (4.0 + (double)tsz) + 4.0 * (double)(A.rows + 1);
 }
 
@@ -574,11 +521,10 @@ void precond_algorithmic_bytes(const dg_precond& pc, double* total, double* bloc
           tot += 2.0 * csr_bytes(L.A, (size_t)T) + csr_bytes(L.R, (size_t)T) + csr_bytes(L.P, (size_t)T) +
                  T * (6.0 * nc + 2.0 * ncn);
         else if (L.n_cont > 0 && L.coarse_w)   // W (dense), Sb, Sp; b read twice, xo, the coarse output
-          tot += T * (double)L.coarse_w_rows * (double)L.n + csr_bytes(L.Sb, (size_t)T) +
-                 csr_bytes(L.Sp, (size_t)T) + T * (3.0 * nc + ncn);
+          tot += T * (double)L.coarse_w_rows * (double)L.n + csr_bytes(L.S, (size_t)T) +
+                 T * (3.0 * nc + ncn);
         else if (L.n_cont > 0)         // Rpre, Sb, Sp; b read twice, xo, the coarse vectors
-          tot += csr_bytes(L.Rpre, (size_t)T) + csr_bytes(L.Sb, (size_t)T) + csr_bytes(L.Sp, (size_t)T) +
-                 T * (3.0 * nc + 2.0 * ncn);
+          tot += csr_bytes(L.Rpre, (size_t)T) + csr_bytes(L.S, (size_t)T) + T * (3.0 * nc + 2.0 * ncn);
         const bool fused_here = l > 0 && pc.levels[l - 1].coarse_w;
         if (!fused_here)   // dense coarse blocks
           tot += T * (double)L.end_inv_entries + 2.0 * T * (double)(L.n - L.n_cont);

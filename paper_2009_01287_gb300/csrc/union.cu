@@ -35,24 +35,53 @@ void append_rows(Csr& out, const Csr& in, int64_t col_shift) {
 }
 
 template <typename T>
+void upload_slices(DevArena& a, const Csr& C, DevSlices& D, cudaStream_t s) {
+  DG_REQUIRE(C.nnz() < (1LL << 31), "matrix too large for 32-bit indices");
+  const SlicePlan S = plan_slices(C);
+  std::vector<int32_t> idx;
+  std::vector<T> val;
+  fill_slices(C, S, idx, val);
+  D.rows = C.rows;
+  D.nnz = C.nnz();
+  D.n_cta = S.n_cta;
+  D.n_warp = S.n_warp;
+  D.hdr = a.upload(S.hdr, s);
+  D.row = a.upload(S.row, s);
+  D.idx = a.upload(idx, s);
+  D.val = a.upload(val, s);
+}
+
+// [A | B] row by row, B's columns shifted by `shift`
+Csr beside(const Csr& A, const Csr& B, int64_t shift) {
+  Csr C;
+  C.rows = A.rows;
+  C.cols = shift + B.cols;
+  C.ptr.reserve(A.rows + 1);
+  C.ptr.push_back(0);
+  C.idx.reserve(A.idx.size() + B.idx.size());
+  C.val.reserve(A.idx.size() + B.idx.size());
+  for (int64_t i = 0; i < A.rows; ++i) {
+    C.idx.insert(C.idx.end(), A.idx.begin() + A.ptr[i], A.idx.begin() + A.ptr[i + 1]);
+    C.val.insert(C.val.end(), A.val.begin() + A.ptr[i], A.val.begin() + A.ptr[i + 1]);
+    for (int64_t t = B.ptr[i]; t < B.ptr[i + 1]; ++t) {
+      C.idx.push_back((int32_t)(B.idx[t] + shift));
+      C.val.push_back(B.val[t]);
+    }
+    C.ptr.push_back((int64_t)C.idx.size());
+  }
+  return C;
+}
+
+template <typename T>
 void upload_csr_t(DevArena& a, const Csr& C, DevCsr& D, cudaStream_t s) {
   DG_REQUIRE(C.nnz() < (1LL << 31), "matrix too large for 32-bit indices");
   std::vector<int32_t> ptr(C.ptr.begin(), C.ptr.end());
   if (ptr.empty()) ptr.push_back(0);
-  std::vector<T> val(C.val.begin(), C.val.end());
   D.rows = C.rows;
   D.nnz = C.nnz();
-  D.group_all = csr_group_for(C.rows ? (double)C.nnz() / (double)C.rows : 1.0);
-  const CsrTierPlan tp = plan_csr_tiers(C);
-  D.group = tp.group;
-  D.long_min = tp.long_min;
-  D.n_cta = (int)tp.cta.size();
-  D.n_warp = (int)tp.warp.size();
-  if (!tp.cta.empty()) D.cta_rows = a.upload(tp.cta, s);
-  if (!tp.warp.empty()) D.warp_rows = a.upload(tp.warp, s);
   D.ptr = a.upload(ptr, s);
   D.idx = a.upload(C.idx, s);
-  D.val = a.upload(val, s);
+  D.val = a.upload(std::vector<T>(C.val.begin(), C.val.end()), s);
 }
 
 }  // namespace
@@ -122,7 +151,7 @@ void upload_union_precond(dg_precond* pc, const std::vector<InstSrc>& inst, cuda
   P.cols = nlev ? nrows[0] : 0;
   DG_REQUIRE((int64_t)dinv.size() == pc->n_dofs, "instance sizes do not add up");
   upload_csr_t<T>(a, P, pc->P, s);
-  upload_csr_t<T>(a, csr_transpose(P), pc->PT, s);
+  upload_slices<T>(a, csr_transpose(P), pc->PT, s);
   pc->dinv = a.upload(std::vector<T>(dinv.begin(), dinv.end()), s);
   pc->e_pos = a.upload(eb, s);
   // block-solve units over all instances, largest blocks first
@@ -184,9 +213,9 @@ void upload_union_precond(dg_precond* pc, const std::vector<InstSrc>& inst, cuda
       Ac.cols = ncont[l];
       Pc.cols = (l + 1 < nlev) ? nrows[l + 1] : 0;
       Rc.cols = ncont[l];
-      upload_csr_t<T>(a, Ac, D.A, s);
-      upload_csr_t<T>(a, Pc, D.P, s);
-      upload_csr_t<T>(a, Rc, D.R, s);
+      upload_slices<T>(a, Ac, D.A, s);
+      upload_slices<T>(a, Pc, D.P, s);
+      upload_slices<T>(a, Rc, D.R, s);
       D.dinv = a.upload(dinv_c, s);
       D.t1 = a.alloc<T>(ncont[l]);
       D.t2 = a.alloc<T>(ncont[l]);
@@ -194,16 +223,8 @@ void upload_union_precond(dg_precond* pc, const std::vector<InstSrc>& inst, cuda
       Sb.cols = ncont[l];
       Sp.cols = (l + 1 < nlev) ? nrows[l + 1] : 0;
       Rp.cols = ncont[l];
-      upload_csr_t<T>(a, Sb, D.Sb, s);
-      upload_csr_t<T>(a, Sp, D.Sp, s);
-      upload_csr_t<T>(a, Rp, D.Rpre, s);
-      // lanes per row of the fused up-sweep: half the power of two below the
-      // mean length of both operators' rows together (measured faster), and
-      // on a level too small to fill the GPU at that width (rows x lanes under
-      // the resident threads of 152 SMs) twice that, up to a warp per row
-      int g = std::max(1, csr_group_for(ncont[l] ? (double)(Sb.nnz() + Sp.nnz()) / (double)ncont[l] : 1.0) / 2);
-      while (g < 32 && ncont[l] * (int64_t)g < kResidentThreads) g *= 2;
-      D.Sb.group_all = g;
+      if (ncont[l] > 0) upload_slices<T>(a, beside(Sb, Sp, ncont[l]), D.S, s);
+      upload_slices<T>(a, Rp, D.Rpre, s);
     }
     D.n_end = (int)end_off.size();
     D.end_row = a.upload(end_row, s);

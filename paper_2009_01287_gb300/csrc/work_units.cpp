@@ -36,6 +36,63 @@ CsrTierPlan plan_csr_tiers(const Csr& C) {
   return T;
 }
 
+SlicePlan plan_slices(const Csr& C) {
+  SlicePlan S;
+  const CsrTierPlan tiers = plan_csr_tiers(C);
+  auto len = [&](int64_t i) { return C.ptr[i + 1] - C.ptr[i]; };
+  auto lanes_for = [&](int64_t n, int rounds) {
+    int g = 1;
+    while (g < 32 && n > (int64_t)g * rounds) g *= 2;
+    return n > std::min<int64_t>(kCsrCtaRow, 128 * (int64_t)rounds) ? 256 : g;
+  };
+  int rounds = 16;
+  for (; rounds > 4; rounds /= 2) {
+    int64_t lanes = 0;
+    for (int64_t i = 0; i < C.rows; ++i) lanes += lanes_for(len(i), rounds);
+    if (lanes >= kResidentThreads / 2) break;
+  }
+  // rows of a whole CTA: the CTA tier, and the warp tier's above the limit
+  std::vector<char> cta(C.rows, 0);
+  std::vector<int32_t> wide = tiers.cta;
+  for (int32_t i : tiers.warp)
+    if (lanes_for(len(i), rounds) > 32) wide.push_back(i);
+  int64_t at = 0;   // in units of 32 entries
+  for (int32_t i : wide) {
+    cta[i] = 1;
+    const int32_t nr = (int32_t)((len(i) + 255) / 256);
+    S.hdr.insert(S.hdr.end(), {(int32_t)at, nr, 256, (int32_t)S.row.size()});
+    S.row.push_back(i);
+    at += 8 * (int64_t)nr;
+    ++S.n_cta;
+  }
+  // classes of (rounds, lanes), the longest first
+  std::vector<std::pair<int32_t, int32_t>> order;   // (class key, row)
+  order.reserve(C.rows);
+  for (int64_t i = 0; i < C.rows; ++i) {
+    if (cta[i]) continue;
+    const int g = lanes_for(len(i), rounds);
+    order.push_back({-(int32_t)(((len(i) + g - 1) / g) * 64 + g), (int32_t)i});
+  }
+  std::stable_sort(order.begin(), order.end(),
+                   [](const std::pair<int32_t, int32_t>& a, const std::pair<int32_t, int32_t>& b) {
+                     return a.first < b.first;
+                   });
+  for (size_t i = 0; i < order.size();) {
+    const int32_t key = -order[i].first, g = key % 64, nr = key / 64;
+    S.hdr.insert(S.hdr.end(), {(int32_t)at, nr, g, (int32_t)S.row.size()});
+    for (int r = 0; r < 32 / g; ++r) {
+      const bool has = i < order.size() && order[i].first == -key;
+      S.row.push_back(has ? order[i].second : -1);
+      if (has) ++i;
+    }
+    at += nr;
+    ++S.n_warp;
+  }
+  DG_REQUIRE(at < (1LL << 31) && S.row.size() < (1ULL << 31), "matrix too large for its slices");
+  S.entries = 32 * at;
+  return S;
+}
+
 void plan_block_units(const std::vector<int32_t>& dims, const std::vector<int32_t>& slot,
                       const std::vector<int64_t>& inv_off, std::vector<int32_t>& unit,
                       std::vector<int64_t>& ubase, std::vector<int32_t>& brec) {
