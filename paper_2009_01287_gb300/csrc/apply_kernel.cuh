@@ -82,28 +82,49 @@ struct Reduce {
 };
 
 // ============================================================== reductions
-// Deterministic block sum (blockDim.x == NT, a multiple of 32): a fixed
-// shuffle tree inside each warp, then the warp sums, in warp order, by a fixed
-// shuffle tree in warp 0.  Three barriers instead of the log2(NT) + 2 of a
-// shared-memory tree (about 1 us less per reducing kernel on GB300).
+// Deterministic block sum (blockDim.x == NT, a multiple of 32; red: NT
+// doubles): warp 0 adds the NT values from shared memory, NT / 32 per lane in
+// order, then by a fixed shuffle tree.  An FP64 instruction occupies its SM's
+// pipe for 19 cycles whatever its active lanes, so the 12 additions of one
+// warp are cheaper than a shuffle tree in each of eight (45).
+__device__ __forceinline__ double warp0_sum(const double* red, int n) {
+  const int lane = threadIdx.x & 31;
+  double r = red[lane];
+  for (int k = 32; k < n; k += 32) r += red[k + lane];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
+  return r;
+}
 template <int NT>
 __device__ __forceinline__ double block_sum(double v, double* red) {
   static_assert(NT % 32 == 0 && NT <= 1024, "block_sum: NT must be a multiple of 32, at most 1024");
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  if (lane == 0) red[w] = v;
+  red[threadIdx.x] = v;
   __syncthreads();
-  if (w == 0) {
-    double r = lane < NT / 32 ? red[lane] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
-    if (lane == 0) red[NT / 32] = r;
+  if (threadIdx.x < 32) {
+    v = warp0_sum(red, NT);
+    if (threadIdx.x == 0) red[0] = v;   // after the whole warp's reads (the shuffles converge it)
   }
   __syncthreads();
-  const double r = red[NT / 32];
+  v = red[0];
   __syncthreads();
-  return r;
+  return v;
+}
+// two sums, one warp each (red: 2 NT doubles)
+template <int NT>
+__device__ __forceinline__ void block_sum2(double& v1, double& v2, double* red) {
+  static_assert(NT % 32 == 0 && NT >= 64 && NT <= 1024, "block_sum2: at least two warps");
+  red[threadIdx.x] = v1;
+  red[NT + threadIdx.x] = v2;
+  __syncthreads();
+  if (threadIdx.x < 64) {
+    double* mine = red + (threadIdx.x / 32) * NT;
+    const double v = warp0_sum(mine, NT);
+    if ((threadIdx.x & 31) == 0) mine[0] = v;
+  }
+  __syncthreads();
+  v1 = red[0];
+  v2 = red[NT];
+  __syncthreads();
 }
 
 // Last-CTA finalisation of a grid-wide sum (see Reduce): deterministic, the
@@ -131,7 +152,8 @@ __device__ __forceinline__ void reduce_finalize(double tot, const Reduce& R, dou
 
 // Two sums finalised together: the ticket of R1 counts the CTAs; the last one
 // sums both partial arrays in CTA order into R1.out and R2.out, returns true
-// (in every thread of that CTA) and leaves the sums in *v1_out, *v2_out.
+// (in every thread of that CTA) and leaves the sums in *v1_out, *v2_out
+// (red: 2 NT doubles).
 template <int NT>
 __device__ __forceinline__ bool reduce_finalize2(double t1, double t2, const Reduce& R1, const Reduce& R2,
                                                  double* red, double* v1_out, double* v2_out) {
@@ -150,8 +172,7 @@ __device__ __forceinline__ bool reduce_finalize2(double t1, double t2, const Red
       v1 += __ldcg(R1.partial + i);
       v2 += __ldcg(R2.partial + i);
     }
-    v1 = block_sum<NT>(v1, red);
-    v2 = block_sum<NT>(v2, red);
+    block_sum2<NT>(v1, v2, red);
     if (threadIdx.x == 0) {
       *R1.out = v1;
       *R2.out = v2;

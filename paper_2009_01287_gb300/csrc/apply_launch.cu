@@ -24,23 +24,27 @@ __global__ void __launch_bounds__(kThreads) trace_kernel(const ApplyArgs A) {
   }
 }
 
+// Inside PCG, after the solve has stopped: no operator, and alpha = 0, so that
+// the updates riding on the preconditioner change nothing.
+__device__ __forceinline__ bool pcg_stopped(const ApplyArgs& A) {
+  if (!A.pcg_sc || A.pcg_sc[SC_STATUS] == 0.0) return false;
+  if (blockIdx.x == 0 && threadIdx.x == 0) A.pcg_sc[SC_ALPHA] = 0.0;
+  return true;
+}
+
 // End of a persistent operator launch: the last CTA to leave resets the tile
 // counter and sums the tile partials of x . y in tile order.  Inside PCG
 // (pcg_sc set, x = p, y = q) it also forms the step alpha = (r.z) / (p.q) once
-// for the kernels that apply the update r -= alpha q, x += alpha p (alpha = 0
-// once the solve has stopped: iterations queued after the stop change nothing).
+// for the kernels that apply the update r -= alpha q, x += alpha p.
 template <int NT>
 __device__ __forceinline__ void apply_exit(const ApplyArgs& A, double* red) {
   __shared__ unsigned s_last;
   pdl_trigger();   // this CTA's tiles are done: the next kernel may start launching
   // the scalars alpha needs, loaded before the ticket so that their latency
   // overlaps it (no kernel writes them while the operator runs)
-  double rz = 0.0, status = 0.0;
+  double rz = 0.0;
   if (threadIdx.x == 0) {
-    if (A.pcg_sc) {
-      rz = A.pcg_sc[SC_RZ];
-      status = A.pcg_sc[SC_STATUS];
-    }
+    if (A.pcg_sc) rz = A.pcg_sc[SC_RZ];
     __threadfence();
     s_last = (atomicAdd(A.sched + 1, 1u) == gridDim.x - 1) ? 1u : 0u;
   }
@@ -53,7 +57,7 @@ __device__ __forceinline__ void apply_exit(const ApplyArgs& A, double* red) {
       v = block_sum<NT>(v, red);
       if (threadIdx.x == 0) {
         *A.dot_out = v;
-        if (A.pcg_sc) A.pcg_sc[SC_ALPHA] = status == 0.0 ? rz / v : 0.0;
+        if (A.pcg_sc) A.pcg_sc[SC_ALPHA] = rz / v;
       }
     }
     if (threadIdx.x == 0) {
@@ -76,6 +80,7 @@ __global__ void __launch_bounds__(kThreads) apply_kernel(const ApplyArgs A) {
   pdl_entry();
   extern __shared__ __align__(16) double smem[];
   __shared__ double red[kThreads];
+  if (pcg_stopped(A)) return;
   __shared__ int s_next[2];
   for (int t = blockIdx.x, par = 0; t < A.n_tiles; par ^= 1) {
     if (threadIdx.x == 0) s_next[par] = (int)(gridDim.x + atomicAdd(A.sched, 1u));
@@ -103,6 +108,7 @@ __global__ void __launch_bounds__(kThreads) apply_map_kernel(const ApplyArgs A) 
   pdl_entry();
   extern __shared__ __align__(16) double smem[];
   __shared__ double red[kThreads];
+  if (pcg_stopped(A)) return;
   __shared__ int s_next[2];
   for (int t = blockIdx.x, par = 0; t < A.n_tiles; par ^= 1) {
     if (threadIdx.x == 0) s_next[par] = (int)(gridDim.x + atomicAdd(A.sched, 1u));
@@ -172,6 +178,7 @@ __global__ void __launch_bounds__(kThreads3) apply3_kernel(const ApplyArgs A) {
   pdl_entry();
   extern __shared__ __align__(16) double smem[];
   __shared__ double red[kThreads3];
+  if (pcg_stopped(A)) return;
   __shared__ int s_next[2];
   for (int t = blockIdx.x, par = 0; t < A.n_tiles; par ^= 1) {
     if (threadIdx.x == 0) s_next[par] = (int)(gridDim.x + atomicAdd(A.sched, 1u));

@@ -294,6 +294,12 @@ static double pcg_start(const dg_precond* pc, PcgWork& w, const double* b, doubl
   return hsc[SC_BB];
 }
 
+// PCG iterations in one pass of the graph's while node.  A pass costs about
+// 3.5 us beyond its kernels (empty bodies, GB300), so four share it; the
+// iterations of a pass after the one that stopped change nothing and skip the
+// operator (on average one and a half of them, once per solve).
+constexpr int kItersPerBody = 4;
+
 // One graph for a whole solve: the start kernels, then a device-side while
 // node around one PCG iteration whose condition the kernels set.  Captured
 // once per preconditioner, on the workspace copies of b and x, with the limits
@@ -339,7 +345,7 @@ static bool pcg_capture(const dg_mesh* M, const dg_precond* pc, PcgWork& w) {
       ec = cudaStreamBeginCaptureToGraph(w.cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
       if (ec == cudaSuccess) {
         try {
-          pcg_body(M, pc, w, w.x, -1, 0.0, handle, 1, w.cap);
+          for (int u = 0; u < kItersPerBody; ++u) pcg_body(M, pc, w, w.x, -1, 0.0, handle, 1, w.cap);
         } catch (const Error& e) {
           launched = false;
           why = e.what();

@@ -283,7 +283,7 @@ precond_final_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict_
                      const T* __restrict__ zE, const double* r,
                      double* __restrict__ z, int64_t n, Reduce red, Reduce rr, PcgCtl ctl, XrDefer xr) {
   pdl_entry();
-  __shared__ double sred[kVecThreads];
+  __shared__ double sred[2 * kVecThreads];
   double dot = 0.0, dot_rr = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     double ri;
@@ -323,8 +323,8 @@ precond_final_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict_
       c_lim = ctl.maxit < 0 ? sc[SC_MAXIT] : (double)ctl.maxit;
       c_tol2 = ctl.maxit < 0 ? sc[SC_RTOL2] : ctl.rtol2;
     }
-    const double t1 = block_sum<kVecThreads>(dot, sred);
-    const double t2 = block_sum<kVecThreads>(dot_rr, sred);
+    double t1 = dot, t2 = dot_rr;
+    block_sum2<kVecThreads>(t1, t2, sred);
     double rz_new = 0.0, rr_new = 0.0;
     if (reduce_finalize2<kVecThreads>(t1, t2, red, rr, sred, &rz_new, &rr_new) && ctl.sc &&
         threadIdx.x == 0 && c_status == 0.0) {
