@@ -220,10 +220,13 @@ struct ApplyArgs {
   int n_tiles;
   unsigned* sched;            // [0] next tile, [1] exit ticket (both zero between launches)
   BasisOff boff[kMaxP + 1];
-  // mapped squares: per sub-face record its rule size, tables, factors and
-  // penalty; the geometric factors at the Gauss points (volume per element,
-  // faces per record); the volume tables
-  const SubFaceMap* sfm;
+  // mapped squares: the sub-faces whose weights are formed and, per sub-face
+  // record, where a side finds them; the geometric factors at the Gauss points
+  // (volume per element, faces per record); the volume tables
+  const MapFace* mface;
+  const MapFaceTile* mface_tiles;
+  const MapSide* mside;
+  double* mw;
   const double* gvol;
   const int64_t* goff;
   const double* gface;

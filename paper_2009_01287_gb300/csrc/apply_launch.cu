@@ -102,8 +102,15 @@ __global__ void __launch_bounds__(kThreads) apply_kernel(const ApplyArgs A) {
   apply_exit<kThreads>(A, red);
 }
 
-// Persistent operator kernel of mapped squares (same scheduling as on boxes).
+// Weights of every sub-face of a mapped mesh.
 template <bool BR2>
+__global__ void __launch_bounds__(kThreads3) map_face_kernel(const ApplyArgs A) {
+  pdl_entry();
+  extern __shared__ __align__(16) double smem[];
+  map_face_tile<BR2>(A, A.mface_tiles[blockIdx.x], smem);
+}
+
+// Persistent operator kernel of mapped squares (same scheduling as on boxes).
 __global__ void __launch_bounds__(kThreads) apply_map_kernel(const ApplyArgs A) {
   pdl_entry();
   extern __shared__ __align__(16) double smem[];
@@ -114,14 +121,14 @@ __global__ void __launch_bounds__(kThreads) apply_map_kernel(const ApplyArgs A) 
     if (threadIdx.x == 0) s_next[par] = (int)(gridDim.x + atomicAdd(A.sched, 1u));
     const ApplyTile T = A.tiles[t];
     switch (T.p) {
-      case 1: apply_map_tile<1, BR2>(A, T, t, smem, red); break;
-      case 2: apply_map_tile<2, BR2>(A, T, t, smem, red); break;
-      case 3: apply_map_tile<3, BR2>(A, T, t, smem, red); break;
-      case 4: apply_map_tile<4, BR2>(A, T, t, smem, red); break;
-      case 5: apply_map_tile<5, BR2>(A, T, t, smem, red); break;
-      case 6: apply_map_tile<6, BR2>(A, T, t, smem, red); break;
-      case 7: apply_map_tile<7, BR2>(A, T, t, smem, red); break;
-      case 8: apply_map_tile<8, BR2>(A, T, t, smem, red); break;
+      case 1: apply_map_tile<1>(A, T, t, smem, red); break;
+      case 2: apply_map_tile<2>(A, T, t, smem, red); break;
+      case 3: apply_map_tile<3>(A, T, t, smem, red); break;
+      case 4: apply_map_tile<4>(A, T, t, smem, red); break;
+      case 5: apply_map_tile<5>(A, T, t, smem, red); break;
+      case 6: apply_map_tile<6>(A, T, t, smem, red); break;
+      case 7: apply_map_tile<7>(A, T, t, smem, red); break;
+      case 8: apply_map_tile<8>(A, T, t, smem, red); break;
       default: break;
     }
     __syncthreads();
@@ -216,27 +223,22 @@ static int apply_shape_smem(int p) {
 
 static int map_shape_smem(int p) {
   switch (p) {
-    case 1: return MapShape<1>::PART;
-    case 2: return MapShape<2>::PART;
-    case 3: return MapShape<3>::PART;
-    case 4: return MapShape<4>::PART;
-    case 5: return MapShape<5>::PART;
-    case 6: return MapShape<6>::PART;
-    case 7: return MapShape<7>::PART;
-    default: return MapShape<8>::PART;
+    case 1: return MapShape<1>::SMEM;
+    case 2: return MapShape<2>::SMEM;
+    case 3: return MapShape<3>::SMEM;
+    case 4: return MapShape<4>::SMEM;
+    case 5: return MapShape<5>::SMEM;
+    case 6: return MapShape<6>::SMEM;
+    case 7: return MapShape<7>::SMEM;
+    default: return MapShape<8>::SMEM;
   }
 }
 
 int64_t apply_smem_for(const dg_mesh& M) {
   if (M.host.dim == 3) return M.apply3_smem;
-  if (M.host.mapped) {   // the tile's layout plus the item weights (and BR2's lifting vectors)
-    const int per_item = kMapItemDoubles + (M.opts.form == DG_FORM_BR2 ? kMapItemBr2 : 0);
+  if (M.host.mapped) {
     int64_t mx = 0;
-    for (int t = 0; t < M.n_tiles; ++t) {
-      const ApplyTile& T = M.h_tiles[t];
-      const int64_t nit = M.h_item_ptr[t + 1] - M.h_item_ptr[t];
-      mx = std::max<int64_t>(mx, map_shape_smem(T.p) + per_item * nit);
-    }
+    for (int t = 0; t < M.n_tiles; ++t) mx = std::max<int64_t>(mx, map_shape_smem(M.h_tiles[t].p));
     return 8 * mx;
   }
   // the layout of the tile's degree plus its sub-face item partials
@@ -285,7 +287,10 @@ ApplyArgs make_apply_args(const dg_mesh& M, const double* x, double* y, Reduce r
   A.n_tiles = M.n_tiles;
   A.sched = M.d_sched;
   for (int p = 0; p <= kMaxP; ++p) A.boff[p] = M.boff[p];
-  A.sfm = M.d_sfm;
+  A.mface = M.d_mface;
+  A.mface_tiles = M.d_mface_tiles;
+  A.mside = M.d_mside;
+  A.mw = M.d_mw;
   A.gvol = M.d_gvol;
   A.goff = M.d_goff;
   A.gface = M.d_gface;
@@ -320,10 +325,8 @@ int apply_kernel_setup(const dg_mesh& M) {
   const int smem = (int)M.apply_smem;
   DG_REQUIRE(smem <= optin, "operator tile needs too much shared memory");
   if (M.host.mapped) {
-    DG_CUDA(cudaFuncSetAttribute(apply_map_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    DG_CUDA(cudaFuncSetAttribute(apply_map_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    if (br2) DG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, apply_map_kernel<true>, kThreads, smem));
-    else DG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, apply_map_kernel<false>, kThreads, smem));
+    DG_CUDA(cudaFuncSetAttribute(apply_map_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
+    DG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, apply_map_kernel, kThreads, smem));
     return sms * (per > 0 ? per : 1);
   }
   DG_CUDA(cudaFuncSetAttribute(apply_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
@@ -349,11 +352,19 @@ static void launch_modal3(const dg_mesh& M, const ApplyArgs& A, cudaStream_t s) 
   launch_hang3(M, A, s);
 }
 
+static void launch_map_faces(const dg_mesh& M, const ApplyArgs& A, cudaStream_t s) {
+  const int g = (int)M.h_mface_tiles.size();
+  const size_t smem = (size_t)M.mface_smem;
+  if (M.opts.form == DG_FORM_BR2) launch_k(map_face_kernel<true>, g, kThreads3, smem, s, A);
+  else launch_k(map_face_kernel<false>, g, kThreads3, smem, s, A);
+}
+
 void launch_trace(const dg_mesh& M, const double* x, cudaStream_t s) {
   if (M.n_tiles == 0) return;
   const ApplyArgs A = make_apply_args(M, x, nullptr, Reduce{});
   if (M.host.dim == 3) launch_modal3(M, A, s);
   else launch_k(trace_kernel, M.n_tiles, kThreads, 0, s, A);
+  if (M.host.mapped) launch_map_faces(M, A, s);
   DG_CUDA(cudaGetLastError());
 }
 
@@ -375,11 +386,16 @@ void launch_apply(const dg_mesh& M, const double* x, double* y, Reduce red, cuda
   const int smem = (int)M.apply_smem;
   if (with_trace) launch_k(trace_kernel, M.n_tiles, kThreads, 0, s, A);
   if (M.host.mapped) {
-    if (M.opts.form == DG_FORM_BR2) launch_k(apply_map_kernel<true>, grid, kThreads, smem, s, A);
-    else launch_k(apply_map_kernel<false>, grid, kThreads, smem, s, A);
+    if (with_trace) launch_map_faces(M, A, s);
+    launch_k(apply_map_kernel, grid, kThreads, smem, s, A);
   }
   else if (M.opts.form == DG_FORM_BR2) launch_k(apply_kernel<true>, grid, kThreads, smem, s, A);
   else launch_k(apply_kernel<false>, grid, kThreads, smem, s, A);
+  DG_CUDA(cudaGetLastError());
+}
+
+void launch_faces_of_traces(const dg_mesh& M, const double* x, cudaStream_t s) {
+  launch_map_faces(M, make_apply_args(M, x, nullptr, Reduce{}), s);
   DG_CUDA(cudaGetLastError());
 }
 

@@ -13,24 +13,30 @@
 //           the map there (three factors per point, stored at setup); back to
 //           the nodes with the transposed products: four passes of
 //           O((p+1)(p+2)^2) work per element instead of two;
-//   faces   one thread per (sub-face item, Gauss point) evaluates both sides'
-//           traces there (values and a-weighted normal derivatives from the
-//           trace array, tangential derivatives from the trace values) and,
-//           with the point's stored factors (the arc-length weight w and w m
-//           for m = J^-1 n, n = J^-T nu / |J^-T nu| the physical normal),
-//           writes three adjoint weights: of the test function's value, of its
-//           tangential derivative and of its normal derivative; one thread per
-//           side node then sums them over its sub-faces in sub-face order
-//           (deterministic) with the side's basis tables, and the gather adds
-//           the normal-derivative weights through l_k'(0 or 1) / h as on boxes.
+//   faces   (map_face kernel, before the tiles) one thread per (sub-face, Gauss
+//           point) evaluates both sides' traces there (values and a-weighted
+//           normal derivatives from the trace array, tangential derivatives
+//           from the trace values) and, with the point's stored factors (the
+//           arc-length weight w and w m for m = J^-1 n, n = J^-T nu / |J^-T nu|
+//           the physical normal), writes three adjoint weights: of the test
+//           function's value, of its tangential derivative and of its normal
+//           derivative.  Seen from the other side the jump and the normal change
+//           sign: the first and the third weight do, the second does not, so
+//           one evaluation serves both sides.  In the tiles one thread per side
+//           node sums its sub-faces' weights in sub-face order (deterministic)
+//           with the side's basis tables, and the gather adds the
+//           normal-derivative weights through l_k'(0 or 1) / h.
 //   BR2     the mass matrix of a mapped element is not a Kronecker product, so
 //           the lifting takes the block of each element's mass inverse on a
-//           side's nodes (stored at setup): per item the jump projected onto
+//           side's nodes (stored at setup): per sub-face the jump projected onto
 //           both sides' nodes, the two blocks applied, and the lifted values
-//           at the item's points added to the value weights (three more
-//           passes of the tile's items).
-// Every sub-face is evaluated from both of its sides (no atomics): applies are
-// bit-reproducible.
+//           at its points added to the value weights.
+// Applies are bit-reproducible (fixed sums, no atomics on data).
+// Measured (GB300): apply of the 98k-unknown hp mesh on a quadrilateral 58.9 us
+// with every tile evaluating its sub-faces itself (24 of 32 lanes active), 43.9
+// with the weights formed once (22.6 of 27.3 MFLOP; the tiles' kernel 58 -> 36
+// us, the weights' 6); PCG on 24k curved unknowns 70.3 -> 55.3 us per iteration
+// (with the other changes measured beside it).
 #pragma once
 
 #include "apply_kernel.cuh"
@@ -47,14 +53,110 @@ struct MapShape {
   // shared doubles: B, D (2 Q NP), x (EPB NN), stage 1 / 3 (2 EPB NP Q),
   // point fluxes (2 EPB QQ), side sums r, c2 (8 EPB NP)
   static constexpr int SMEM = 2 * Q * NP + EPB * NN + 2 * EPB * NP * Q + 2 * EPB * QQ + 8 * EPB * NP;
-  // then the sub-face item weights: [item][kMapQMax][3]; BR2 adds per item
-  // the weighted jumps at its points and both sides' lifting vectors
-  static constexpr int PART = SMEM;
 };
-constexpr int kMapItemDoubles = 3 * kMapQMax;
-constexpr int kMapItemBr2 = kMapQMax + 4 * kMaxN;   // w [[u]] per point; j-, j+, z-, z+
 
-template <int P, bool BR2>
+// Weights of a tile of sub-faces (MapFaceTile: rules of at most nq points, sides
+// of at most nn nodes).
+template <bool BR2>
+__device__ __forceinline__ void map_face_tile(const ApplyArgs& A, const MapFaceTile& T, double* sm) {
+  const int Q = T.nq, N = T.nn, cnt = T.count;
+  const MapFace* faces = A.mface + T.first;
+  const double2* tr = reinterpret_cast<const double2*>(A.tr);
+  double* sj = sm;                    // BR2: [cnt][Q] w [[u]]
+  double* sp = sj + cnt * Q;          // [cnt][2][N] projections, then
+  double* sz = sp + cnt * 2 * N;      // [cnt][2][N] liftings
+  for (int t = threadIdx.x; t < cnt * Q; t += kThreads3) {
+    const int it = t / Q, g = t - it * Q;
+    const MapFace& f = faces[it];
+    const int qf = f.qf;
+    if (g >= qf) continue;
+    double u0 = 0.0, du0 = 0.0, f0 = 0.0;
+    {
+      const int np = f.np;
+      const double2* src = tr + f.src_o;
+      const double* Bo = A.tab + f.tab_bo + g * np;
+      const double* Do = Bo + qf * np;
+      for (int m = 0; m < np; ++m) {
+        const double2 v = __ldg(src + m);
+        const double b = __ldg(Bo + m);
+        u0 = fma(b, v.x, u0);
+        du0 = fma(__ldg(Do + m), v.x, du0);
+        f0 = fma(b, v.y, f0);
+      }
+    }
+    // the point's factors: w = w_g |J t| dt, w m_t, w m_n s (m = J^-1 n)
+    const double* gf = A.gface + f.geo;
+    const double w = __ldg(gf + g), wmt = __ldg(gf + qf + g), wmn = __ldg(gf + 2 * qf + g);
+    double jmp = u0, flux = fma(f0, wmn, f.aih_o * du0 * wmt), cc = 1.0;   // w (a grad u-) . n
+    if (f.npn > 0) {
+      const int np = f.npn;
+      const double2* src = tr + f.src_n;
+      const double* Bn = A.tab + f.tab_bn + g * np;
+      const double* Dn = Bn + qf * np;
+      double u1 = 0.0, du1 = 0.0, f1 = 0.0;
+      for (int m = 0; m < np; ++m) {
+        const double2 v = __ldg(src + m);
+        const double b = __ldg(Bn + m);
+        u1 = fma(b, v.x, u1);
+        du1 = fma(__ldg(Dn + m), v.x, du1);
+        f1 = fma(b, v.y, f1);
+      }
+      jmp = u0 - u1;
+      flux = 0.5 * (flux + fma(-f1, wmn, f.aih_n * du1 * wmt));
+      cc = 0.5;
+    }
+    double* W = A.mw + f.w + 3 * g;
+    W[0] = BR2 ? -flux : fma(f.sigma * jmp, w, -flux);   // of v-
+    W[1] = -cc * jmp * wmt;                              // of d v- / d t (times a / h and l' at the side sums)
+    W[2] = -cc * jmp * wmn;                              // of a times the outward normal derivative of v-
+    if (BR2) sj[it * Q + g] = w * jmp;
+  }
+  if (!BR2) return;
+  __syncthreads();
+  // BR2 liftings (Section 4.4) on both sides: j = int phi_j [[u]] ds on each
+  // side's nodes, z = (block of that element's mass inverse on the side) j, and
+  // at every point the weight eta coef a w (z-(x_g) + z+(x_g)) of v-
+  for (int t = threadIdx.x; t < cnt * 2 * N; t += kThreads3) {
+    const int it = t / (2 * N), rem = t - it * 2 * N, sd = rem / N, j = rem - sd * N;
+    const MapFace& f = faces[it];
+    const int np = sd == 0 ? f.np : f.npn;
+    if (j >= np) continue;
+    const double* B = A.tab + (sd == 0 ? f.tab_bo : f.tab_bn) + j;
+    double a = 0.0;
+    for (int g = 0; g < f.qf; ++g) a = fma(__ldg(B + g * np), sj[it * Q + g], a);
+    sp[t] = a;
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < cnt * 2 * N; t += kThreads3) {
+    const int it = t / (2 * N), rem = t - it * 2 * N, sd = rem / N, j = rem - sd * N;
+    const MapFace& f = faces[it];
+    const int np = sd == 0 ? f.np : f.npn;
+    if (j >= np) continue;
+    const double* G = A.gbr2 + (sd == 0 ? f.g_o : f.g_n) + j * np;
+    double a = 0.0;
+    for (int i = 0; i < np; ++i) a = fma(__ldg(G + i), sp[t - j + i], a);
+    sz[t] = a;
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < cnt * Q; t += kThreads3) {   // the thread that wrote the point's weights
+    const int it = t / Q, g = t - it * Q;
+    const MapFace& f = faces[it];
+    if (g >= f.qf) continue;
+    const double* z = sz + it * 2 * N;
+    double v = 0.0;
+    for (int i = 0; i < f.np; ++i) v = fma(__ldg(A.tab + f.tab_bo + g * f.np + i), z[i], v);
+    for (int i = 0; i < f.npn; ++i) v = fma(__ldg(A.tab + f.tab_bn + g * f.npn + i), z[N + i], v);
+    double* W = A.mw + f.w + 3 * g;
+    W[0] = fma(f.cbr2 * __ldg(A.gface + f.geo + g), v, W[0]);
+  }
+}
+
+// x with its sign bit flipped where s is negative zero's bit pattern
+__device__ __forceinline__ double flip(double x, int s) {
+  return __hiloint2double(__double2hiint(x) ^ s, __double2loint(x));
+}
+
+template <int P>
 __device__ __forceinline__ void apply_map_tile(const ApplyArgs& A, const ApplyTile& T, int tile, double* sm,
                                                double* red) {
   using S = MapShape<P>;
@@ -68,7 +170,6 @@ __device__ __forceinline__ void apply_map_tile(const ApplyArgs& A, const ApplyTi
   double* sF2 = sF1 + EPB * QQ;
   double* sr = sF2 + EPB * QQ;        // [EPB][4][NP]
   double* sc2 = sr + EPB * 4 * NP;
-  double* part = sm + S::PART;        // [item][kMapQMax][3]
 
   const int tid = threadIdx.x;
   const int count = T.count;
@@ -96,138 +197,7 @@ __device__ __forceinline__ void apply_map_tile(const ApplyArgs& A, const ApplyTi
     sA1[t] = a;
     sA2[t] = b;
   }
-  // ---- faces, pass 1: one thread per (sub-face item, Gauss point)
-  const int ib = A.item_ptr[tile];
-  const int nit = A.item_ptr[tile + 1] - ib;
-  double* br2 = part + kMapItemDoubles * nit;   // BR2: [item][kMapItemBr2]
-  for (int t = tid; t < nit * kMapQMax; t += blockDim.x) {
-    const int it = t / kMapQMax, g = t - it * kMapQMax;
-    const int2 item = A.items[ib + it];
-    const SubFaceMap fm = A.sfm[item.x];
-    const int qf = fm.qf;
-    if (g >= qf) continue;
-    const SubFaceRec f = A.sf[item.x];
-    const int e = (item.y & 0xffff) >> 2, s = item.y & 3;
-    const int k = A.order[T.first + e];
-    const double2* trk = reinterpret_cast<const double2*>(A.tr + A.toff[k]) + s * NP;
-    const double* Bo = A.tab + fm.tab_bo + g * NP;
-    const double* Do = A.tab + fm.tab_bo + (qf + g) * NP;
-    double u0 = 0.0, du0 = 0.0, f0 = 0.0;
-#pragma unroll
-    for (int m = 0; m < NP; ++m) {
-      const double2 v = trk[m];
-      const double b = __ldg(Bo + m);
-      u0 = fma(b, v.x, u0);
-      du0 = fma(__ldg(Do + m), v.x, du0);
-      f0 = fma(b, v.y, f0);
-    }
-    du0 *= A.ih[k];
-    // the point's factors: w = w_g |J t| dt, w m_t, w m_n s (m = J^-1 n)
-    const double* gf = A.gface + fm.geo;
-    const double w = __ldg(gf + g), wmt = __ldg(gf + qf + g), wmn = __ldg(gf + 2 * qf + g);
-    const double Fo = fma(f0, wmn, A.ak[k] * du0 * wmt);   // w (a grad u-) . n
-    double jmp, flux, cc;
-    if (f.nb >= 0) {
-      const int npn = f.pn + 1;
-      const double2* trn = reinterpret_cast<const double2*>(A.tr + A.toff[f.nb]) + f.nb_side * npn;
-      const double* Bn = A.tab + fm.tab_bn + g * npn;
-      const double* Dn = A.tab + fm.tab_bn + (qf + g) * npn;
-      double u1 = 0.0, du1 = 0.0, f1 = 0.0;
-      for (int m = 0; m < npn; ++m) {
-        const double2 v = trn[m];
-        const double b = __ldg(Bn + m);
-        u1 = fma(b, v.x, u1);
-        du1 = fma(__ldg(Dn + m), v.x, du1);
-        f1 = fma(b, v.y, f1);
-      }
-      du1 *= A.ih[f.nb];
-      const double Fn = fma(-f1, wmn, A.ak[f.nb] * du1 * wmt);   // w (a grad u+) . n
-      jmp = u0 - u1;
-      flux = 0.5 * (Fo + Fn);
-      cc = 0.5;
-    } else {
-      jmp = u0;
-      flux = Fo;
-      cc = 1.0;
-    }
-    double* pp = part + ((item.y >> 16) * kMapQMax + g) * 3;
-    if (BR2) {
-      pp[0] = -flux;                                    // the lifting term is added below
-      br2[(item.y >> 16) * kMapItemBr2 + g] = w * jmp;
-    } else {
-      pp[0] = fma(fm.sigma * jmp, w, -flux);   // weight of v-
-    }
-    pp[1] = -cc * jmp * wmt;                 // of d v- / d t (times a / h and l' at the side sums)
-    pp[2] = -cc * jmp * wmn;                 // of a times the outward normal derivative of v-
-  }
   __syncthreads();
-  if (BR2) {
-    // BR2 liftings (Section 4.4) of every sub-face on both of its sides:
-    // j = int phi_j [[u]] ds on each side's nodes, z = (block of that
-    // element's mass inverse on the side) j, and at every point the weight
-    // eta coef a w (z-(x_g) + z+(x_g)) of the own test function's value.
-    // One thread per (item, side node) for j and z, per (item, point) after.
-    for (int t = tid; t < nit * kMaxN; t += blockDim.x) {
-      const int it = t / kMaxN, j = t - it * kMaxN;
-      const int2 item = A.items[ib + it];
-      const SubFaceMap fm = A.sfm[item.x];
-      const SubFaceRec f = A.sf[item.x];
-      double* b = br2 + (item.y >> 16) * kMapItemBr2;
-      if (j < NP) {
-        double a = 0.0;
-        for (int g = 0; g < fm.qf; ++g) a = fma(__ldg(A.tab + fm.tab_bo + g * NP + j), b[g], a);
-        b[kMapQMax + j] = a;
-      }
-      if (f.nb >= 0 && j <= f.pn) {
-        const int npn = f.pn + 1;
-        double a = 0.0;
-        for (int g = 0; g < fm.qf; ++g) a = fma(__ldg(A.tab + fm.tab_bn + g * npn + j), b[g], a);
-        b[kMapQMax + kMaxN + j] = a;
-      }
-    }
-    __syncthreads();
-    for (int t = tid; t < nit * kMaxN; t += blockDim.x) {
-      const int it = t / kMaxN, j = t - it * kMaxN;
-      const int2 item = A.items[ib + it];
-      const SubFaceRec f = A.sf[item.x];
-      const int e = (item.y & 0xffff) >> 2, s = item.y & 3;
-      double* b = br2 + (item.y >> 16) * kMapItemBr2;
-      if (j < NP) {
-        const int k = A.order[T.first + e];
-        const double* Go = A.gbr2 + A.g2off[k] + s * NP * NP + j * NP;
-        double z = 0.0;
-#pragma unroll
-        for (int i = 0; i < NP; ++i) z = fma(__ldg(Go + i), b[kMapQMax + i], z);
-        b[kMapQMax + 2 * kMaxN + j] = z;
-      }
-      if (f.nb >= 0 && j <= f.pn) {
-        const int npn = f.pn + 1;
-        const double* Gn = A.gbr2 + A.g2off[f.nb] + f.nb_side * npn * npn + j * npn;
-        double z = 0.0;
-        for (int i = 0; i < npn; ++i) z = fma(__ldg(Gn + i), b[kMapQMax + kMaxN + i], z);
-        b[kMapQMax + 3 * kMaxN + j] = z;
-      }
-    }
-    __syncthreads();
-    for (int t = tid; t < nit * kMapQMax; t += blockDim.x) {
-      const int it = t / kMapQMax, g = t - it * kMapQMax;
-      const int2 item = A.items[ib + it];
-      const SubFaceMap fm = A.sfm[item.x];
-      if (g >= fm.qf) continue;
-      const SubFaceRec f = A.sf[item.x];
-      const double* b = br2 + (item.y >> 16) * kMapItemBr2;
-      double v = 0.0;
-#pragma unroll
-      for (int i = 0; i < NP; ++i) v = fma(__ldg(A.tab + fm.tab_bo + g * NP + i), b[kMapQMax + 2 * kMaxN + i], v);
-      if (f.nb >= 0) {
-        const int npn = f.pn + 1;
-        for (int i = 0; i < npn; ++i)
-          v = fma(__ldg(A.tab + fm.tab_bn + g * npn + i), b[kMapQMax + 3 * kMaxN + i], v);
-      }
-      part[((item.y >> 16) * kMapQMax + g) * 3] += fm.cbr2 * __ldg(A.gface + fm.geo + g) * v;
-    }
-    __syncthreads();
-  }
   // ---- volume stage 2 and the flux at every Gauss point
   for (int t = tid; t < count * QQ; t += blockDim.x) {
     const int e = t / QQ, rem = t - e * QQ;
@@ -246,30 +216,28 @@ __device__ __forceinline__ void apply_map_tile(const ApplyArgs& A, const ApplyTi
     sF1[t] = fma(g11, ux, g12 * uy);
     sF2[t] = fma(g12, ux, g22 * uy);
   }
-  // ---- faces, pass 2: one thread per side node sums its sub-faces' weights
-  // in sub-face order with the side's basis tables
+  // ---- faces: one thread per side node sums its sub-faces' weights in
+  // sub-face order with the side's basis tables
   for (int t = tid; t < count * 4 * NP; t += blockDim.x) {
     const int e = t / (4 * NP);
     const int s = (t / NP) & 3;
     const int i = t % NP;
     const int k = A.order[T.first + e];
-    const int2 si = A.side_items[(int64_t)(T.first + e) * 4 + s];
-    const int rec0 = A.sf_ptr[4 * k + s];
-    const double aih = A.aih[k];
-    double r = 0.0, c2 = 0.0;
-    for (int j = 0; j < si.y; ++j) {
-      const SubFaceMap fm = A.sfm[rec0 + j];
-      const double* pp = part + (si.x - ib + j) * kMapQMax * 3;
+    const int rec0 = A.sf_ptr[4 * k + s], rec1 = A.sf_ptr[4 * k + s + 1];
+    double r = 0.0, rt = 0.0, c2 = 0.0;
+    for (int j = rec0; j < rec1; ++j) {
+      const MapSide fm = A.mside[j];
+      const double* W = A.mw + fm.w;
       const double* Bo = A.tab + fm.tab_bo + i;
       const double* Do = Bo + fm.qf * NP;
       for (int g = 0; g < fm.qf; ++g) {
         const double b = __ldg(Bo + g * NP);
-        r = fma(b, pp[3 * g], r);
-        r = fma(aih * __ldg(Do + g * NP), pp[3 * g + 1], r);
-        c2 = fma(b, pp[3 * g + 2], c2);
+        r = fma(b, flip(__ldg(W + 3 * g), fm.sign), r);
+        rt = fma(__ldg(Do + g * NP), __ldg(W + 3 * g + 1), rt);
+        c2 = fma(b, flip(__ldg(W + 3 * g + 2), fm.sign), c2);
       }
     }
-    sr[t] = r;
+    sr[t] = fma(A.aih[k], rt, r);
     sc2[t] = c2;
   }
   __syncthreads();

@@ -53,6 +53,11 @@ void upload_tiles(dg_mesh* M, cudaStream_t s) {
   M->d_items = a.upload(M->h_items, s);
   M->d_item_ptr = a.upload(M->h_item_ptr, s);
   M->d_side_items = a.upload(M->h_side_items, s);
+  if (M->host.mapped) {
+    M->d_mface = a.upload(M->h_mface, s);
+    M->d_mface_tiles = a.upload(M->h_mface_tiles, s);
+    M->d_mside = a.upload(M->h_mside, s);
+  }
   if (M->host.dim == 3) {
     M->d_sfm3 = a.upload(M->h_sfm3, s);
     M->d_erec3 = a.upload(M->h_erec3, s);
@@ -93,7 +98,7 @@ void upload_mesh(dg_mesh* M, cudaStream_t s) {
   M->d_sf = a.upload(M->h_sf, s);
   M->d_sfb = M->h_sfb.empty() ? nullptr : a.upload(M->h_sfb, s);
   if (m.mapped) {
-    M->d_sfm = a.upload(M->h_sfm, s);
+    M->d_mw = a.alloc<double>(M->n_mw);
     M->d_gvol = a.upload(M->h_gvol, s);
     M->d_goff = a.upload(M->h_goff, s);
     M->d_gface = a.upload(M->h_gface, s);

@@ -213,6 +213,26 @@ struct SubFaceMap {
                     // larger coefficient of the two sides), 0 for SIPG
 };
 
+// The same sub-face for the kernel that forms its weights, once for both sides,
+// seen from one of them; and, per SubFaceRec, where a side finds them.
+struct MapFace {
+  int32_t src_o, src_n;   // traces of the own and the neighbour's side (double2 units)
+  int32_t np, npn;        // nodes of either (npn = 0 on the boundary)
+  int32_t qf, tab_bo, tab_bn, geo;   // as in SubFaceMap
+  int32_t w;              // first of the 3 qf weights (three per point)
+  int32_t pad;
+  int64_t g_o, g_n;       // BR2: the mass-inverse side blocks
+  double sigma, cbr2;
+  double aih_o, aih_n;    // a / h
+};
+struct MapFaceTile {
+  int32_t first, count, nq, nn;
+};
+struct MapSide {
+  int32_t w, qf, tab_bo;
+  int32_t sign;           // sign bit of the first and third weight (high word)
+};
+
 // Offsets of the degree-p volume tables of mapped meshes: the (p+2)-point
 // Gauss rule (points, weights) and l_j, l_j' at its points ((p+2) x (p+1)).
 struct MapOff {

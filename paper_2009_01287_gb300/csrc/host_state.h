@@ -140,6 +140,11 @@ struct dg_mesh {
   // h_g2off[k])
   std::vector<double> h_gbr2;
   std::vector<int64_t> h_g2off;
+  std::vector<dg::MapFace> h_mface;
+  std::vector<dg::MapFaceTile> h_mface_tiles;
+  std::vector<dg::MapSide> h_mside;
+  int64_t n_mw = 0;                     // weights (doubles)
+  int64_t mface_smem = 0;               // dynamic shared memory of the weights' kernel (BR2)
   // host only: per element the images of its (p+1)^2 Gauss-Lobatto nodes (the
   // LOR cells' vertices) and, at the (p+3)^2 points of the load-vector rule,
   // the image and det J (x, y, det per point; offsets h_roff), so that no
@@ -189,7 +194,10 @@ struct dg_mesh {
   dg::HangTile* d_hang_tiles = nullptr;
   int32_t* d_side3 = nullptr;
   double* d_xm = nullptr;       // cube meshes: modes of the operator's argument
-  dg::SubFaceMap* d_sfm = nullptr;   // mapped squares
+  dg::MapFace* d_mface = nullptr;
+  dg::MapFaceTile* d_mface_tiles = nullptr;
+  dg::MapSide* d_mside = nullptr;
+  double* d_mw = nullptr;
   double* d_gvol = nullptr;          // mapped squares: geometric factors (h_gvol, h_goff, h_gface)
   int64_t* d_goff = nullptr;
   double* d_gface = nullptr;
@@ -283,6 +291,8 @@ void build_mesh_host3(dg_mesh* M, const dg_mesh_desc* desc, const dg_options& op
 // the flop and byte counts of the mapped operator (after the box counts)
 void build_mesh_map(dg_mesh* M, const dg_mesh_desc* desc);
 void map_stats(dg_mesh* M);
+// mapped squares: the sub-faces whose weights the kernels form (after the tiles)
+void build_map_faces(dg_mesh* M);
 // rows of element k of y = A x on a mapped mesh, and their diagonal, and the
 // LOR block of element k (dense (p+1)^2 x (p+1)^2, row-major)
 void host_element_residual_map(const dg_mesh& M, int64_t k, const double* x, double* y);

@@ -627,6 +627,7 @@ void launch_pcg_p_trace(const dg_mesh& M, double* p, const double* z, double* sc
   const ApplyArgs A = make_apply_args(M, p, nullptr, Reduce{});
   launch_k(pcg_p_trace_kernel, M.n_tiles, kThreads, 0, s, A, p, z, sc,
            (cudaGraphConditionalHandle)cond_handle, use_cond, first);
+  if (M.host.mapped) launch_faces_of_traces(M, p, s);
   DG_CUDA(cudaGetLastError());
 }
 

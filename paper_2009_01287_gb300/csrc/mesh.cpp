@@ -239,6 +239,7 @@ void build_tiles(dg_mesh* M) {
   M->n_tiles = (int)M->h_tiles.size();
   M->h_order = order;
   build_face_items(M);
+  if (m.mapped) build_map_faces(M);
 }
 
 void build_face_items(dg_mesh* M) {
@@ -458,7 +459,16 @@ void build_mesh_host(dg_mesh* M, const dg_mesh_desc* desc, const dg_options* opt
     g.tab_x += base;
     g.tab_y += base;
   }
-  if (m.mapped) build_mesh_map(M, desc);   // the mapped records, tables and factors
+  if (m.mapped) {
+    build_mesh_map(M, desc);   // the mapped records, tables and factors
+    // fewer tiles than SMs: half the elements per tile (24k unknowns, 109 tiles:
+    // 3.1 us of 70 per PCG iteration; a quarter was no better)
+    int64_t cnt[kMaxP + 1] = {0}, tiles = 0;
+    for (int64_t k = 0; k < m.n; ++k) ++cnt[m.p[k]];
+    for (int p = 1; p <= kMaxP; ++p) tiles += (cnt[p] + M->tile_epb[p] - 1) / M->tile_epb[p];
+    if (tiles < 152)
+      for (int p = 1; p <= kMaxP; ++p) M->tile_epb[p] = std::max(1, M->tile_epb[p] / 2);
+  }
   build_tiles(M);
   // operation and byte counts of one operator apply, as the kernel does it
   dg_mesh_stats& S = M->stats;

@@ -1,3 +1,4 @@
+#include <climits>
 // Mapped square meshes (Section 2: element maps T_kappa onto general
 // quadrilaterals).  The leaf boxes of the lattice are pre-images; the bilinear
 // map of the lattice domain onto the quadrilateral with the given corners, or
@@ -375,6 +376,83 @@ void build_mesh_map(dg_mesh* M, const dg_mesh_desc* desc) {
     }
 }
 
+void build_map_faces(dg_mesh* M) {
+  const HostMesh& m = M->host;
+  const bool br2 = M->opts.form == DG_FORM_BR2;
+  std::vector<int32_t> toff(m.n);
+  int64_t at = 0;
+  for (int64_t k = 0; k < m.n; ++k) {
+    toff[k] = (int32_t)at;
+    at += 4 * (m.p[k] + 1);
+  }
+  DG_REQUIRE(at < (1LL << 31), "too many side traces");
+  // element and side of every record
+  std::vector<int32_t> elem(m.sf.size()), side(m.sf.size());
+  for (int64_t k = 0; k < m.n; ++k)
+    for (int s = 0; s < 4; ++s)
+      for (int j = m.sf_ptr[4 * k + s]; j < m.sf_ptr[4 * k + s + 1]; ++j) {
+        elem[j] = (int32_t)k;
+        side[j] = s;
+      }
+  M->h_mside.assign(m.sf.size(), MapSide{});
+  std::vector<MapFace> faces;
+  std::vector<int32_t> rec;
+  int64_t w = 0;
+  // the records in item order; a sub-face is formed from its lower-numbered element
+  for (size_t g = 0; g < M->h_items.size(); g += 2) {
+    const int32_t j = M->h_items[g], k = elem[j], s = side[j];
+    const SubFaceRec& f = M->h_sf[j];
+    if (f.nb >= 0 && f.nb < k) continue;
+    const SubFaceMap& r = M->h_sfm[j];
+    MapFace F{};
+    F.np = m.p[k] + 1;
+    F.src_o = toff[k] + s * F.np;
+    F.qf = r.qf;
+    F.tab_bo = r.tab_bo;
+    F.tab_bn = r.tab_bn;
+    F.geo = r.geo;
+    F.w = (int32_t)w;
+    F.sigma = r.sigma;
+    F.cbr2 = r.cbr2;
+    F.aih_o = m.coef[k] / M->h_h[k];
+    if (br2) F.g_o = M->h_g2off[k] + (int64_t)s * F.np * F.np;
+    M->h_mside[j] = {(int32_t)w, r.qf, r.tab_bo, 0};
+    if (f.nb >= 0) {
+      F.npn = f.pn + 1;
+      F.src_n = toff[f.nb] + f.nb_side * F.npn;
+      F.aih_n = m.coef[f.nb] / M->h_h[f.nb];
+      if (br2) F.g_n = M->h_g2off[f.nb] + (int64_t)f.nb_side * F.npn * F.npn;
+      int back = -1;   // the same sub-face seen from the neighbour
+      for (int q = m.sf_ptr[4 * (int64_t)f.nb + f.nb_side]; q < m.sf_ptr[4 * (int64_t)f.nb + f.nb_side + 1]; ++q)
+        if (m.sf[q].nb == k && m.sf[q].t0 == m.sf[j].t0) back = q;
+      DG_REQUIRE(back >= 0 && M->h_sfm[back].qf == r.qf, "mapped sub-face without its other side");
+      M->h_mside[back] = {(int32_t)w, r.qf, M->h_sfm[back].tab_bo, INT32_MIN};
+    }
+    w += 3 * r.qf;
+    DG_REQUIRE(w < (1LL << 31), "too many sub-face points");
+    faces.push_back(F);
+  }
+  M->n_mw = w;
+  // tiles of faces of nearly one rule size, about one point per thread
+  std::stable_sort(faces.begin(), faces.end(), [](const MapFace& x, const MapFace& y) {
+    return x.qf != y.qf ? x.qf > y.qf : x.np + x.npn > y.np + y.npn;
+  });
+  M->h_mface = faces;
+  M->h_mface_tiles.clear();
+  M->mface_smem = 0;
+  for (size_t i = 0; i < faces.size();) {
+    MapFaceTile T{(int32_t)i, 0, faces[i].qf, 0};
+    const int cap = kThreads3 / T.nq;
+    while (i < faces.size() && T.count < cap) {
+      T.nn = std::max(T.nn, std::max(faces[i].np, faces[i].npn));
+      ++T.count;
+      ++i;
+    }
+    M->h_mface_tiles.push_back(T);
+    if (br2) M->mface_smem = std::max<int64_t>(M->mface_smem, 8LL * T.count * (T.nq + 4 * T.nn));
+  }
+}
+
 void map_stats(dg_mesh* M) {
   // operation and byte counts of one mapped operator apply, as the kernel does it
   const HostMesh& m = M->host;
@@ -393,9 +471,11 @@ void map_stats(dg_mesh* M) {
       const double nn = f.nb >= 0 ? m.p[f.nb] + 1.0 : 0.0;
       // per point: three own and three neighbour sums and the weights; per
       // side node and point: three sums
-      fl += qf * (2.0 * 3.0 * (n1 + nn) + 16.0) + 2.0 * 3.0 * n1 * qf;
+      // (the weights once for both sides)
+      const double once = f.nb >= 0 ? 0.5 : 1.0;
+      fl += once * qf * (2.0 * 3.0 * (n1 + nn) + 16.0) + 2.0 * 3.0 * n1 * qf;
       // BR2: both sides' projections, side-block products and values at the points
-      if (M->opts.form == DG_FORM_BR2) fl += 2.0 * (2.0 * qf * (n1 + nn) + n1 * n1 + nn * nn) + 4.0 * qf;
+      if (M->opts.form == DG_FORM_BR2) fl += once * (2.0 * (2.0 * qf * (n1 + nn) + n1 * n1 + nn * nn) + 4.0 * qf);
     }
   }
   S.apply_flops = fl;
