@@ -197,8 +197,12 @@ struct ApplyArgs {
   const int32_t* sf_ptr;
   const SubFaceRec* sf;
   const SubFaceBr2* sfb;      // square meshes, BR2: the multiplied-out liftings
+  const SubFaceModal2* sfm2;  // squares in modes
+  const int2* side2;
+  const int2* hang2;
+  const int4* hang2_tile;
   const SubFaceModal3* sfm3;  // cube meshes
-  const ElemRec3* erec3;
+  const ElemRec3* erec3;      // kernels in modes
   const HangPair* hang3;
   const HangTile* hang_tiles;
   const int2* side3;

@@ -1,8 +1,9 @@
 // Launch code of the matrix-free operator (Section 2, Eq. fe-problem; BR2 of
-// Section 4.4): the trace kernels, the persistent operator kernels of square
-// and cube meshes, their shared-memory sizing and resident grid.  The tile
-// work itself is in apply_kernel.cuh and apply3_kernel.cuh.
+// Section 4.4): the kernels around the tile work of apply_kernel.cuh,
+// apply2_kernel.cuh, apply3_kernel.cuh and apply_map_kernel.cuh, their
+// shared-memory sizing and grids.
 #include "apply_map_kernel.cuh"
+#include "apply2_kernel.cuh"
 #include "kernels.cuh"
 
 namespace dg {
@@ -100,6 +101,84 @@ __global__ void __launch_bounds__(kThreads) apply_kernel(const ApplyArgs A) {
     t = s_next[par];
   }
   apply_exit<kThreads>(A, red);
+}
+
+#define DG_CASES_2 \
+    DG_CASE_2(1) DG_CASE_2(2) DG_CASE_2(3) DG_CASE_2(4) DG_CASE_2(5) DG_CASE_2(6) DG_CASE_2(7) DG_CASE_2(8)
+
+// Modes and traces of x on large square meshes.  UPDATE (inside PCG): p = z + beta p
+// (first: p = z, and the initial scalars and loop condition) takes the place of
+// x.
+template <bool UPDATE>
+__global__ void __launch_bounds__(kThreads3)
+modal2_kernel(const ApplyArgs A, double* p, const double* z, double* sc, cudaGraphConditionalHandle h,
+              int use_cond, int first) {
+  __shared__ __align__(16) double smem[modal2_doubles()];
+  const ApplyTile T = A.tiles[blockIdx.x];
+  const int4 hang = __ldg(A.hang2_tile + blockIdx.x);
+  switch (T.p) {   // the tables: written by no kernel, fetched before the wait
+#define DG_CASE_2(PP) \
+    case PP: modal2_tables<PP>(A, smem); break;
+    DG_CASES_2
+#undef DG_CASE_2
+    default: break;
+  }
+  pdl_entry();
+  double beta = 0.0;
+  if (UPDATE) {
+    if (!first && sc[SC_STATUS] != 0.0) return;   // stopped: the loop condition is already clear
+    if (!first) beta = sc[SC_BETA];
+  }
+  if (A.skip && A.skip[(int64_t)T.inst * A.skip_stride] != 0.0) return;
+  switch (T.p) {
+#define DG_CASE_2(PP) \
+    case PP: modal2_tile<PP, UPDATE>(A, T, hang, smem, p, z, beta, first != 0); break;
+    DG_CASES_2
+#undef DG_CASE_2
+    default: break;
+  }
+  if (UPDATE && first) pcg_first_scalars(sc, h, use_cond);
+}
+
+// The operator of large square meshes, a tile per CTA; the last CTA to leave sums the
+// tile partials of x . y in tile order.
+template <bool BR2>
+__global__ void __launch_bounds__(kThreads3) apply2_kernel(const ApplyArgs A) {
+  __shared__ __align__(16) double smem[apply2_doubles()];
+  const ApplyTile T = A.tiles[blockIdx.x];
+  const int4 hang = __ldg(A.hang2_tile + blockIdx.x);
+  Side2 first;
+  const int n = modal_table_doubles(T.p);
+  for (int i = threadIdx.x; i < n; i += kThreads3) smem[i] = __ldg(A.tab + A.moff3[T.p] + i);
+  switch (T.p) {
+#define DG_CASE_2(PP) \
+    case PP: side2_fetch<PP, BR2>(A, T, hang, first); break;
+    DG_CASES_2
+#undef DG_CASE_2
+    default: break;
+  }
+  pdl_entry();
+  if (pcg_stopped(A)) return;
+  if (A.skip && A.skip[(int64_t)T.inst * A.skip_stride] != 0.0) {
+    if (A.dot_partial && threadIdx.x == 0) A.dot_partial[blockIdx.x] = 0.0;
+  } else {
+    double part = 0.0;
+    switch (T.p) {
+#define DG_CASE_2(PP) \
+      case PP: part = apply2_tile<PP, BR2>(A, T, hang, smem, first); break;
+      DG_CASES_2
+#undef DG_CASE_2
+      default: break;
+    }
+    if (A.dot_partial && threadIdx.x < 32) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
+      if (threadIdx.x == 0) A.dot_partial[blockIdx.x] = part;
+    }
+  }
+  if (!A.dot_partial) return;
+  __syncthreads();   // the tile's partial before the CTA's ticket
+  apply_exit<kThreads3>(A, smem);
 }
 
 // Weights of every sub-face of a mapped mesh.
@@ -241,6 +320,7 @@ int64_t apply_smem_for(const dg_mesh& M) {
     for (int t = 0; t < M.n_tiles; ++t) mx = std::max<int64_t>(mx, map_shape_smem(M.h_tiles[t].p));
     return 8 * mx;
   }
+  if (M.modal2) return 0;   // static
   // the layout of the tile's degree plus its sub-face item partials
   int64_t mx = 0;
   for (int t = 0; t < M.n_tiles; ++t) {
@@ -264,6 +344,10 @@ ApplyArgs make_apply_args(const dg_mesh& M, const double* x, double* y, Reduce r
   A.sf_ptr = M.d_sf_ptr;
   A.sf = M.d_sf;
   A.sfb = M.d_sfb;
+  A.sfm2 = M.d_sfm2;
+  A.side2 = reinterpret_cast<const int2*>(M.d_side2);
+  A.hang2 = reinterpret_cast<const int2*>(M.d_hang2);
+  A.hang2_tile = reinterpret_cast<const int4*>(M.d_hang2_tile);
   A.sfm3 = M.d_sfm3;
   A.erec3 = M.d_erec3;
   A.hang3 = M.d_hang3;
@@ -322,6 +406,7 @@ int apply_kernel_setup(const dg_mesh& M) {
     else DG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, apply3_kernel<false>, kThreads3, smem));
     return sms * (per > 0 ? per : 1);
   }
+  if (M.modal2) return M.n_tiles;   // a CTA per tile
   const int smem = (int)M.apply_smem;
   DG_REQUIRE(smem <= optin, "operator tile needs too much shared memory");
   if (M.host.mapped) {
@@ -359,12 +444,23 @@ static void launch_map_faces(const dg_mesh& M, const ApplyArgs& A, cudaStream_t 
   else launch_k(map_face_kernel<false>, g, kThreads3, smem, s, A);
 }
 
+// what an apply needs of x beside x itself: the side traces (modes, weights)
+static void launch_sides(const dg_mesh& M, const ApplyArgs& A, cudaStream_t s) {
+  if (M.host.dim == 3) {
+    launch_modal3(M, A, s);
+  } else if (M.modal2) {
+    launch_k(modal2_kernel<false>, M.n_tiles, kThreads3, 0, s, A, (double*)nullptr, (const double*)nullptr,
+             (double*)nullptr, (cudaGraphConditionalHandle)0, 0, 0);
+  } else {
+    launch_k(trace_kernel, M.n_tiles, kThreads, 0, s, A);
+    if (M.host.mapped) launch_map_faces(M, A, s);
+  }
+}
+
 void launch_trace(const dg_mesh& M, const double* x, cudaStream_t s) {
   if (M.n_tiles == 0) return;
   const ApplyArgs A = make_apply_args(M, x, nullptr, Reduce{});
-  if (M.host.dim == 3) launch_modal3(M, A, s);
-  else launch_k(trace_kernel, M.n_tiles, kThreads, 0, s, A);
-  if (M.host.mapped) launch_map_faces(M, A, s);
+  launch_sides(M, A, s);
   DG_CUDA(cudaGetLastError());
 }
 
@@ -374,23 +470,23 @@ void launch_apply(const dg_mesh& M, const double* x, double* y, Reduce red, cuda
   DG_REQUIRE(!pcg_sc || red.partial, "the PCG step needs the p . q reduction");
   ApplyArgs A = make_apply_args(M, x, y, red);
   A.pcg_sc = pcg_sc;
+  if (with_trace) launch_sides(M, A, s);
   const int grid = M.n_tiles < M.apply_grid ? M.n_tiles : M.apply_grid;
+  const bool br2 = M.opts.form == DG_FORM_BR2;
+  const size_t smem = (size_t)(M.host.dim == 3 ? M.apply3_smem : M.apply_smem);
   if (M.host.dim == 3) {
-    if (with_trace) launch_modal3(M, A, s);
-    const int smem3 = (int)M.apply3_smem;
-    if (M.opts.form == DG_FORM_BR2) launch_k(apply3_kernel<true>, grid, kThreads3, smem3, s, A);
-    else launch_k(apply3_kernel<false>, grid, kThreads3, smem3, s, A);
-    DG_CUDA(cudaGetLastError());
-    return;
-  }
-  const int smem = (int)M.apply_smem;
-  if (with_trace) launch_k(trace_kernel, M.n_tiles, kThreads, 0, s, A);
-  if (M.host.mapped) {
-    if (with_trace) launch_map_faces(M, A, s);
+    if (br2) launch_k(apply3_kernel<true>, grid, kThreads3, smem, s, A);
+    else launch_k(apply3_kernel<false>, grid, kThreads3, smem, s, A);
+  } else if (M.host.mapped) {
     launch_k(apply_map_kernel, grid, kThreads, smem, s, A);
+  } else if (M.modal2) {
+    if (br2) launch_k(apply2_kernel<true>, M.n_tiles, kThreads3, 0, s, A);
+    else launch_k(apply2_kernel<false>, M.n_tiles, kThreads3, 0, s, A);
+  } else if (br2) {
+    launch_k(apply_kernel<true>, grid, kThreads, smem, s, A);
+  } else {
+    launch_k(apply_kernel<false>, grid, kThreads, smem, s, A);
   }
-  else if (M.opts.form == DG_FORM_BR2) launch_k(apply_kernel<true>, grid, kThreads, smem, s, A);
-  else launch_k(apply_kernel<false>, grid, kThreads, smem, s, A);
   DG_CUDA(cudaGetLastError());
 }
 
@@ -399,9 +495,15 @@ void launch_faces_of_traces(const dg_mesh& M, const double* x, cudaStream_t s) {
   DG_CUDA(cudaGetLastError());
 }
 
-void launch_modal3_update(const dg_mesh& M, double* p, const double* z, double* sc,
+void launch_modal_update(const dg_mesh& M, double* p, const double* z, double* sc,
                           unsigned long long cond_handle, int use_cond, int first, cudaStream_t s) {
   const ApplyArgs A = make_apply_args(M, p, nullptr, Reduce{});
+  if (M.host.dim == 2) {
+    launch_k(modal2_kernel<true>, M.n_tiles, kThreads3, 0, s, A, p, z, sc, (cudaGraphConditionalHandle)cond_handle,
+             use_cond, first);
+    DG_CUDA(cudaGetLastError());
+    return;
+  }
   launch_k(modal3_kernel<true>, M.n_tiles, kThreads3, (size_t)M.modal3_smem, s, A, p, z, sc,
            (cudaGraphConditionalHandle)cond_handle, use_cond, first);
   launch_hang3(M, A, s);
@@ -503,7 +605,7 @@ void tune_tiles(dg_mesh* M, cudaStream_t s, void (*retile)(dg_mesh*, void*), voi
       // highest degrees first: their tiles set the length of the launch
       for (int P = kMaxP; P >= 1; --P) {
         if (!present[P]) continue;
-        const int cap = apply_epb(P), start = M->tile_epb[P];
+        const int cap = M->modal2 ? apply2_epb(P) : apply_epb(P), start = M->tile_epb[P];
         const int cand[3] = {cap, std::max(1, (3 * cap + 3) / 4), std::max(1, cap / 2)};
         int best = start;
         for (int c : cand) {

@@ -258,6 +258,7 @@ static void build_batch_tiles(dg_batch* B) {
   U.h_order = order;
   U.n_tiles = (int)U.h_tiles.size();
   build_face_items(&U);
+  if (U.modal2) build_modal2_tiles(&U);
 }
 
 static void retile_batch(dg_mesh*, void* ctx) { build_batch_tiles((dg_batch*)ctx); }
@@ -269,6 +270,19 @@ static void build_union_mesh(dg_batch* B, cudaStream_t s) {
   U.opts = first.opts;
   U.eta = first.eta;
   for (int p = 0; p <= kMaxP; ++p) U.boff[p] = first.boff[p];
+  // the operator's form: by all instances together
+  int64_t elems[kMaxP + 1] = {0};
+  for (int i = 0; i < B->n_inst; ++i)
+    for (int32_t p : B->meshes[i / B->n_rhs]->host.p) ++elems[p];
+  U.modal2 = modal2_pays(elems);
+  if (U.modal2) {
+    for (int p = 1; p <= kMaxP; ++p) U.tile_epb[p] = apply2_epb(p);
+    for (auto& M : B->meshes) {
+      if (M->modal2) continue;   // large enough by itself
+      build_modal2(M.get());
+      modal2_stats(M.get());
+    }
+  }
   // basis tables are identical in every mesh: take the first mesh's prefix
   const int basis_len = first.boff[kMaxP].d1 + kMaxP + 1;
   U.h_tables.assign(first.h_tables.begin(), first.h_tables.begin() + basis_len);
@@ -279,6 +293,7 @@ static void build_union_mesh(dg_batch* B, cudaStream_t s) {
     U.h_tables.insert(U.h_tables.end(), M.h_tables.begin() + basis_len, M.h_tables.end());
   }
   DG_REQUIRE(U.h_tables.size() < (1ULL << 31), "face tables too large");
+  if (U.modal2) append_modal_tables(&U);
   HostMesh& um = U.host;
   um.n = 0;
   um.off.assign(1, 0);
@@ -310,6 +325,18 @@ static void build_union_mesh(dg_batch* B, cudaStream_t s) {
       g.tab_x += (int32_t)tshift[k];
       g.tab_y += (int32_t)tshift[k];
       U.h_sfb.push_back(g);
+    }
+    if (U.modal2) {
+      for (SubFaceModal2 g : M.h_sfm2) {   // one per record, in the same order
+        g.own_off += (int32_t)U.n_trace2;
+        g.nbr_off += (int32_t)U.n_trace2;
+        g.tab_r += (int32_t)tshift[k];
+        U.h_sfm2.push_back(g);
+      }
+      U.h_kind2.insert(U.h_kind2.end(), M.h_kind2.begin(), M.h_kind2.end());
+      for (int32_t t : M.h_toff3) U.h_toff3.push_back((int32_t)(t + U.n_trace2));
+      U.n_trace2 += M.n_trace2;
+      DG_REQUIRE(U.n_trace2 < (1LL << 31), "too many side traces");
     }
     um.n += m.n;
     U.stats.n_elems += M.stats.n_elems;

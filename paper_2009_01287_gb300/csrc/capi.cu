@@ -50,9 +50,17 @@ void upload_tiles(dg_mesh* M, cudaStream_t s) {
   M->apply_grid = apply_kernel_setup(*M);
   M->d_order = a.upload(M->h_order, s);
   M->d_tiles = a.upload(M->h_tiles, s);
-  M->d_items = a.upload(M->h_items, s);
-  M->d_item_ptr = a.upload(M->h_item_ptr, s);
-  M->d_side_items = a.upload(M->h_side_items, s);
+  if (!M->modal2) {
+    M->d_items = a.upload(M->h_items, s);
+    M->d_item_ptr = a.upload(M->h_item_ptr, s);
+    M->d_side_items = a.upload(M->h_side_items, s);
+  }
+  if (M->modal2) {
+    M->d_erec3 = a.upload(M->h_erec3, s);
+    M->d_side2 = a.upload(M->h_side2, s);
+    M->d_hang2 = a.upload(M->h_hang2, s);
+    M->d_hang2_tile = a.upload(M->h_hang2_tile, s);
+  }
   if (M->host.mapped) {
     M->d_mface = a.upload(M->h_mface, s);
     M->d_mface_tiles = a.upload(M->h_mface_tiles, s);
@@ -89,14 +97,20 @@ void upload_mesh(dg_mesh* M, cudaStream_t s) {
       M->d_xm = a.alloc<double>(M->n_dofs);
       M->d_hang3 = a.upload(M->h_hang3, s);
       M->d_hang_tiles = a.upload(M->h_hang_tiles, s);
+    } else if (M->modal2) {
+      M->d_tr = a.alloc<double>(2 * M->n_trace2);
+      M->d_xm = a.alloc<double>(M->n_dofs);
+      M->d_sfm2 = a.upload(M->h_sfm2, s);
     } else {
       M->d_toff = a.upload(toff, s);
       M->d_tr = a.alloc<double>(toff[m.n]);
     }
   }
   M->d_sf_ptr = a.upload(m.sf_ptr, s);
-  M->d_sf = a.upload(M->h_sf, s);
-  M->d_sfb = M->h_sfb.empty() ? nullptr : a.upload(M->h_sfb, s);
+  if (!M->modal2) {
+    M->d_sf = a.upload(M->h_sf, s);
+    M->d_sfb = M->h_sfb.empty() ? nullptr : a.upload(M->h_sfb, s);
+  }
   if (m.mapped) {
     M->d_mw = a.alloc<double>(M->n_mw);
     M->d_gvol = a.upload(M->h_gvol, s);

@@ -18,11 +18,14 @@ namespace dg {
 constexpr int kMaxP = 8;
 constexpr int kMaxN = kMaxP + 1;
 constexpr int kThreads = 256;   // threads per CTA of the operator kernel on squares
-constexpr int kThreads3 = 128;  // and of its two kernels on cubes
+constexpr int kThreads3 = 128;  // and of the kernels in modes
 // elements of degree p per operator CTA (one thread per node, at most 16)
 constexpr int apply_epb(int p) {
   return (kThreads / ((p + 1) * (p + 1))) > 16 ? 16 : (kThreads / ((p + 1) * (p + 1)));
 }
+
+// and in modes: one line of nodes or modes per lane of a warp
+constexpr int apply2_epb(int p) { return 32 / (p + 1); }
 
 // ------------------------------------------------------------------ errors
 struct Error : std::runtime_error {
@@ -103,6 +106,23 @@ struct SubFaceRec3 {
   double area;       // physical area of the sub-face
 };
 
+// A sub-face of a square mesh as the kernels in modes read it (one per
+// SubFaceRec, seen from the same side).  With J = u- - u+ and F = dn- - dn+
+// (both sides' outward derivatives) on the sub-face, the residual over a is
+// r = cz J + cf F and the normal-derivative coefficient c2 = cc J.  BR2: cz
+// belongs to the own side's lifting and cx to the neighbour's, added to it
+// where both sides are whole (cx is then the sum of both, for the modes both
+// sides have).
+struct alignas(16) SubFaceModal2 {
+  int32_t own_off, nbr_off;  // traces on the sub-face (double2 units): the side's, or restricted to it
+  int32_t nn;                // neighbour's modes, 0 on the boundary
+  int32_t tab_r;             // R of the larger side (rows of kMaxN)
+  double cz, cx, cf, cc;
+};
+// how the kernels take a side: one sub-face, diagonal in modes; a larger side
+// (its number of sub-faces, > 0); BR2, the smaller side of a sub-face
+enum { kSideWhole = 0, kSideSmaller = -1 };
+
 // A same-size or boundary sub-face as the kernels read it, in the Legendre
 // modes of its side (in tile order, by element of the tile and side).  With
 // J = u- - u+ and F = dn- - dn+ (both sides' outward derivatives) the residual
@@ -138,9 +158,9 @@ constexpr int hang3_doubles(int p) { return 4 * (p + 1) * (p + 1); }   // per pa
 // per element in tile order
 struct ElemRec3 {
   int64_t off;       // first DOF
-  int32_t toff;      // its six side traces (double2 units)
+  int32_t toff;      // its side traces (double2 units)
   int32_t pad;
-  double ah, aih;    // a h, a / h
+  double ah, aih;    // a h^(dim - 2), a / h
 };
 
 // Shared-memory budget (doubles) of one 3D operator tile; the tiles' element
@@ -151,8 +171,8 @@ constexpr int kApply3Budget = 9 * 1024;
 constexpr int apply3_epb(int p) {
   return p == 1 ? 16 : p == 2 ? 14 : p == 3 ? 8 : p == 4 ? 5 : p == 5 ? 3 : p == 6 ? 2 : p == 7 ? 2 : 1;
 }
-// doubles of a degree's modal tables (Modal3)
-constexpr int modal3_doubles(int p) {
+// doubles of a degree's modal tables (ModalTab)
+constexpr int modal_table_doubles(int p) {
   return ((p + 2) / 2) * ((p + 2) / 2) + ((p + 1) / 2) * ((p + 1) / 2) + (p + 1) * (p + 1) + 2 * (p + 1);
 }
 // doubles of shared memory one element of degree p needs in a 3D tile (its

@@ -111,8 +111,19 @@ struct dg_mesh {
   std::vector<double> h_h;
   std::vector<dg::SubFaceRec> h_sf;
   std::vector<dg::SubFaceBr2> h_sfb;    // square meshes, BR2: one per h_sf record
+  // squares in modes (modal2): per h_sf record its modal form and kind (0 whole
+  // on both sides, 1 the own side larger, 2 smaller); in tile order the sides
+  // {record or first item of the tile, kSide... or number of sub-faces}, the
+  // items {record, tile-local side} of larger, then (BR2) smaller sides, and
+  // per tile {first item, items of larger sides, all items, most modes of one}
+  bool modal2 = false;
+  std::vector<dg::SubFaceModal2> h_sfm2;
+  std::vector<int8_t> h_kind2;
+  std::vector<int32_t> h_side2, h_hang2, h_hang2_tile;
+  int64_t n_trace2 = 0;                 // length of the trace buffer (double2)
   std::vector<dg::SubFaceRec3> h_sf3;   // cube meshes
-  // cube meshes, for the kernels: same-size and boundary sub-face records and
+  // cube meshes, for the kernels (the element records squares in modes too):
+  // same-size and boundary sub-face records and
   // element records in tile order, the hanging pairs and their tiles, and per
   // (order position, side) {record, 0} or {first result, number of pairs}
   std::vector<dg::SubFaceModal3> h_sfm3;
@@ -121,7 +132,7 @@ struct dg_mesh {
   std::vector<dg::HangTile> h_hang_tiles;
   std::vector<int32_t> h_side3;
   int moff3[dg::kMaxP + 1] = {0};       // modal tables of each degree in h_tables
-  std::vector<int32_t> h_toff3;         // cube meshes: trace offset of every element (double2 units)
+  std::vector<int32_t> h_toff3;         // kernels in modes: trace offset of every element (double2 units)
   std::vector<int32_t> h_resoff3;       // per record of a hanging sub-face, the offset of its results, else -1
   int64_t n_trace3 = 0;                 // length of the trace buffer, results included (double2)
   int64_t hang3_smem = 0;               // dynamic shared memory of the hanging pairs' kernel
@@ -171,7 +182,7 @@ struct dg_mesh {
   std::vector<int32_t> h_side_items;  // 2 per (order position, side): first item, count
   int64_t apply_smem = 0;             // dynamic shared memory of the 2D operator kernel
   // tile shapes: squares, elements per operator tile of each degree (at most
-  // apply_epb(p), the compiled capacity); cubes, the shared-memory budget of a
+  // apply_epb(p) or, in modes, apply2_epb(p), the compiled capacities); cubes, the shared-memory budget of a
   // tile in doubles.  Fixed rules unless the tile tuner chose them.
   int tile_epb[dg::kMaxP + 1];
   int64_t apply3_budget = dg::kApply3Budget;
@@ -188,12 +199,14 @@ struct dg_mesh {
   int32_t* d_sf_ptr = nullptr;
   dg::SubFaceRec* d_sf = nullptr;
   dg::SubFaceBr2* d_sfb = nullptr;
+  dg::SubFaceModal2* d_sfm2 = nullptr;   // squares in modes
+  int32_t *d_side2 = nullptr, *d_hang2 = nullptr, *d_hang2_tile = nullptr;
   dg::SubFaceModal3* d_sfm3 = nullptr;   // cube meshes
   dg::ElemRec3* d_erec3 = nullptr;
   dg::HangPair* d_hang3 = nullptr;
   dg::HangTile* d_hang_tiles = nullptr;
   int32_t* d_side3 = nullptr;
-  double* d_xm = nullptr;       // cube meshes: modes of the operator's argument
+  double* d_xm = nullptr;       // kernels in modes: the modes of the operator's argument
   dg::MapFace* d_mface = nullptr;
   dg::MapFaceTile* d_mface_tiles = nullptr;
   dg::MapSide* d_mside = nullptr;
@@ -273,6 +286,15 @@ void build_mesh_host(dg_mesh* M, const dg_mesh_desc* desc, const dg_options* opt
 void build_tiles(dg_mesh* M);
 // flat sub-face item lists of the tiles (square meshes; after the tiles)
 void build_face_items(dg_mesh* M);
+// Squares in modes: whether a mesh with so many elements of each degree takes
+// them, the tables of every degree, the sub-face records with their restriction
+// tables (after the SIPG records), and the tiles' element records, sides and
+// hanging items (after the tiles).
+bool modal2_pays(const int64_t (&elems)[kMaxP + 1]);
+void append_modal_tables(dg_mesh* M);
+void build_modal2(dg_mesh* M);
+void modal2_stats(dg_mesh* M);
+void build_modal2_tiles(dg_mesh* M);
 // cube meshes: degree-sorted order, tiles and their item lists
 void build_tiles3(dg_mesh* M);
 // upload the host-built operator data (M->host.p/off/sf_ptr, h_* arrays)
@@ -281,7 +303,7 @@ void upload_mesh(dg_mesh* M, cudaStream_t s);
 void upload_tiles(dg_mesh* M, cudaStream_t s);
 // Time the operator kernel over candidate tile shapes and keep the fastest:
 // squares, for each degree present (highest first) the elements per tile in
-// {apply_epb(p), 3/4, 1/2 of it}; cubes, shared-memory budgets for 4, 3 and 2
+// {the capacity, 3/4, 1/2 of it}; cubes, shared-memory budgets for 4, 3 and 2
 // tiles per SM.  retile rebuilds the host tile lists from the tile shapes.
 // Records the choice and the times in M->stats.
 void tune_tiles(dg_mesh* M, cudaStream_t s, void (*retile)(dg_mesh*, void*), void* ctx);

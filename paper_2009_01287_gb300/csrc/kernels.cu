@@ -588,7 +588,7 @@ void launch_pcg_init(const double* b, double* x, double* r, int64_t n, Reduce bb
 
 // p = z + beta p (first: p = z) tile by tile, and the side traces of the new p
 // for the next operator apply, so the apply needs no trace launch of its own
-// (squares; modal3_kernel does the same on cubes).  The last CTA of the
+// (squares; the modal kernels do the same in modes).  The last CTA of the
 // preconditioner's final kernel has advanced the scalars and tested
 // convergence (first: the initial scalars are set here).
 __global__ void __launch_bounds__(kThreads)
@@ -620,8 +620,8 @@ pcg_p_trace_kernel(const ApplyArgs A, double* __restrict__ p, const double* __re
 void launch_pcg_p_trace(const dg_mesh& M, double* p, const double* z, double* sc,
                         unsigned long long cond_handle, int use_cond, int first, cudaStream_t s) {
   if (M.n_tiles == 0) return;
-  if (M.host.dim == 3) {
-    launch_modal3_update(M, p, z, sc, cond_handle, use_cond, first, s);
+  if (M.host.dim == 3 || M.modal2) {
+    launch_modal_update(M, p, z, sc, cond_handle, use_cond, first, s);
     return;
   }
   const ApplyArgs A = make_apply_args(M, p, nullptr, Reduce{});

@@ -96,8 +96,8 @@ enum { TK_PQ = 0, TK_RR = 1, TK_RZ = 2, TK_P = 3, TK_BB = 4, TK_COUNT = 8 };
 
 // mapped squares: the sub-faces' weights from the traces in place
 void launch_faces_of_traces(const dg_mesh& M, const double* x, cudaStream_t s);
-// its form on cube meshes (modes and traces of the new p)
-void launch_modal3_update(const dg_mesh& M, double* p, const double* z, double* sc,
+// its form in modes (cubes, large square meshes)
+void launch_modal_update(const dg_mesh& M, double* p, const double* z, double* sc,
                           unsigned long long cond_handle, int use_cond, int first, cudaStream_t s);
 
 void launch_pcg_init(const double* b, double* x, double* r, int64_t n, Reduce bb, cudaStream_t s);

@@ -240,6 +240,7 @@ void build_tiles(dg_mesh* M) {
   M->h_order = order;
   build_face_items(M);
   if (m.mapped) build_map_faces(M);
+  if (M->modal2) build_modal2_tiles(M);
 }
 
 void build_face_items(dg_mesh* M) {
@@ -284,6 +285,177 @@ void build_face_items(dg_mesh* M) {
       M->h_items[2 * g + 1] = rec[2 * pos + 1] | (pos << 16);
     }
     M->h_item_ptr.push_back((int32_t)(M->h_items.size() / 2));
+  }
+}
+
+// Tiles per SM from which squares take the operator in modes: below it is bound
+// by the chain of phases of a tile, longer than the nodal kernel's (98k unknowns,
+// 4.2 tiles per SM: even stand-alone, 12% behind in a solve; 6.6: 26.2 us against
+// 30.5 stand-alone; apply2_kernel.cuh has more).
+constexpr int64_t kModal2TilesPerSm = 6;
+
+bool modal2_pays(const int64_t (&elems)[kMaxP + 1]) {
+  int64_t tiles = 0;
+  for (int p = 1; p <= kMaxP; ++p) tiles += (elems[p] + apply2_epb(p) - 1) / apply2_epb(p);
+  return tiles >= kModal2TilesPerSm * 152;
+}
+
+void append_modal_tables(dg_mesh* M) {
+  for (int p = 1; p <= kMaxP; ++p) {
+    M->moff3[p] = (int)M->h_tables.size();
+    modal_tables(p, M->h_tables);
+  }
+  M->moff3[0] = M->moff3[1];
+}
+
+// Trace offsets of every element, then of the traces restricted to the
+// sub-faces of larger sides; the sub-face records in modes and the restriction
+// tables they need (after the SIPG records).
+void build_modal2(dg_mesh* M) {
+  const HostMesh& m = M->host;
+  const bool br2 = M->opts.form == DG_FORM_BR2;
+  int64_t at = 0;
+  M->h_toff3.resize(m.n);
+  for (int64_t k = 0; k < m.n; ++k) {
+    M->h_toff3[k] = (int32_t)at;
+    at += 4 * (m.p[k] + 1);
+  }
+  M->h_kind2.assign(m.sf.size(), 0);
+  std::vector<int32_t> res(m.sf.size(), -1);
+  for (int64_t k = 0; k < m.n; ++k)
+    for (int j = m.sf_ptr[4 * k]; j < m.sf_ptr[4 * k + 4]; ++j) {
+      const auto& f = m.sf[j];
+      const int len = f.t1 - f.t0;
+      if (m.size[k] > len) {
+        M->h_kind2[j] = 1;
+        res[j] = (int32_t)at;
+        at += m.p[k] + 1;
+      } else if (f.nb >= 0 && m.size[f.nb] > len) {
+        M->h_kind2[j] = 2;
+      }
+    }
+  DG_REQUIRE(at < (1LL << 31), "too many side traces");
+  M->n_trace2 = at;
+  std::map<std::pair<int, int>, int> index;   // (level, position) -> R
+  auto table = [&](int L, int o) {
+    const auto it = index.find({L, o});
+    if (it != index.end()) return it->second;
+    const int at0 = (int)M->h_tables.size();
+    M->h_tables.resize(at0 + kMaxN * kMaxN);
+    modal_restriction(L, o, M->h_tables.data() + at0);
+    index[{L, o}] = at0;
+    return at0;
+  };
+  auto start = [&](int64_t k, int s) {
+    int axis, c, t0, t1;
+    m.side_segment((int)k, s, axis, c, t0, t1);
+    return t0;
+  };
+  M->h_sfm2.assign(m.sf.size(), SubFaceModal2{});
+  for (int64_t k = 0; k < m.n; ++k)
+    for (int s = 0; s < 4; ++s)
+      for (int j = m.sf_ptr[4 * k + s]; j < m.sf_ptr[4 * k + s + 1]; ++j) {
+        const auto& f = m.sf[j];
+        const SubFaceRec& r = M->h_sf[j];
+        SubFaceModal2& g = M->h_sfm2[j];
+        const bool in = f.nb >= 0;
+        const int len = f.t1 - f.t0;
+        const double a = m.coef[k], h = M->h_h[k], half = in ? 0.5 : 1.0;
+        g.own_off = M->h_kind2[j] == 1 ? res[j] : M->h_toff3[k] + s * (m.p[k] + 1);
+        if (M->h_kind2[j] == 1) g.tab_r = table(ilog2(m.size[k] / len), (f.t0 - start(k, s)) / len);
+        if (in) {
+          g.nn = r.pn + 1;
+          g.nbr_off = M->h_toff3[f.nb] + f.nb_side * g.nn;
+          if (M->h_kind2[j] == 2) {
+            int back = -1;   // the same sub-face seen from the larger side
+            for (int i = m.sf_ptr[4 * (int64_t)f.nb + f.nb_side]; i < m.sf_ptr[4 * (int64_t)f.nb + f.nb_side + 1]; ++i)
+              if (m.sf[i].nb == k) back = i;
+            DG_REQUIRE(back >= 0 && res[back] >= 0, "hanging sub-face without a larger side");
+            g.nbr_off = res[back];
+            g.tab_r = table(ilog2(m.size[f.nb] / len), (f.t0 - start(f.nb, f.nb_side)) / len);
+          }
+        }
+        g.cf = -half * r.len / a;
+        g.cc = -half * r.len / h;
+        if (!br2) {
+          g.cz = r.sigma * r.len / a;
+          continue;
+        }
+        // both sides' lifting energies carry the larger coefficient of the sub-face
+        const double w = in ? std::max(a, m.coef[f.nb]) : a;
+        const double c = w * M->eta * (in ? 0.25 : 1.0) * r.len * r.len / a;
+        g.cz = c * (basis1d(m.p[k]).Minv[0] / (h * h));
+        if (in) {
+          const double hn = M->h_h[f.nb];
+          g.cx = c * (basis1d(r.pn).Minv[0] / (hn * hn));
+          if (M->h_kind2[j] == 0) g.cx += g.cz;
+        }
+      }
+  DG_REQUIRE(M->h_tables.size() < (1ULL << 31), "face tables too large");
+}
+
+// FP64 operations of both kernels in modes (a multiply-add, a product and a sum
+// each counted as one, two flops), and the bytes of their records
+void modal2_stats(dg_mesh* M) {
+  const HostMesh& m = M->host;
+  const bool br2 = M->opts.form == DG_FORM_BR2;
+  double fma = 0.0;
+  for (int64_t k = 0; k < m.n; ++k) {
+    const double a = m.p[k] + 1.0, H = std::floor(a / 2), C = a - H;
+    const double line = C * C + H * H + 2.0 * H;                  // one line between nodes and modes
+    const double stiff = H * H + (C - 1.0) * (C - 1.0);           // one line's stiffness
+    fma += 2.0 * a * (2.0 * line + stiff + 2.0 * (2.0 * a + 4.0));  // + traces, lift
+    for (int j = m.sf_ptr[4 * k]; j < m.sf_ptr[4 * k + 4]; ++j) {
+      fma += 6.0 * a;
+      if (M->h_kind2[j] == 1) fma += (br2 ? 5.0 : 4.0) * 0.5 * a * (a + 1.0);   // R or R^T
+      const double nn = M->h_sfm2[j].nn;
+      if (br2 && M->h_kind2[j] == 2) fma += nn * (nn + 1.0);
+    }
+  }
+  M->stats.apply_flops = 2.0 * fma;
+  M->stats.apply_bytes = 16.0 * (double)M->n_dofs + (double)m.n * (sizeof(ElemRec3) + 32) +
+                         (double)m.sf.size() * sizeof(SubFaceModal2);
+}
+
+void build_modal2_tiles(dg_mesh* M) {
+  const HostMesh& m = M->host;
+  const bool br2 = M->opts.form == DG_FORM_BR2;
+  M->h_erec3.clear();
+  M->h_side2.clear();
+  M->h_hang2.clear();
+  M->h_hang2_tile.clear();
+  for (const ApplyTile& T : M->h_tiles) {
+    const int32_t first = (int32_t)M->h_hang2.size() / 2;
+    int32_t big = 0, width = T.p + 1;   // BR2: most modes on either side of an item
+    std::vector<int32_t> small;
+    for (int e = 0; e < T.count; ++e) {
+      const int64_t k = M->h_order[T.first + e];
+      M->h_erec3.push_back({m.off[k], M->h_toff3[k], 0, m.coef[k], m.coef[k] / M->h_h[k]});
+      for (int s = 0; s < 4; ++s) {
+        const int32_t b = m.sf_ptr[4 * k + s], n = m.sf_ptr[4 * k + s + 1] - b;
+        if (M->h_kind2[b] == 1) {
+          M->h_side2.push_back(big);
+          M->h_side2.push_back(n);
+          for (int j = 0; j < n; ++j) {
+            M->h_hang2.push_back(b + j);
+            M->h_hang2.push_back(4 * e + s);
+            width = std::max(width, M->h_sfm2[b + j].nn);
+          }
+          big += n;
+        } else {
+          const bool sm = br2 && M->h_kind2[b] == 2;
+          M->h_side2.push_back(b);
+          M->h_side2.push_back(sm ? kSideSmaller : kSideWhole);
+          if (sm) {
+            small.push_back(b);
+            small.push_back(4 * e + s);
+            width = std::max(width, M->h_sfm2[b].nn);
+          }
+        }
+      }
+    }
+    M->h_hang2.insert(M->h_hang2.end(), small.begin(), small.end());
+    M->h_hang2_tile.insert(M->h_hang2_tile.end(), {first, big, big + (int32_t)small.size() / 2, width});
   }
 }
 
@@ -469,6 +641,14 @@ void build_mesh_host(dg_mesh* M, const dg_mesh_desc* desc, const dg_options* opt
     if (tiles < 152)
       for (int p = 1; p <= kMaxP; ++p) M->tile_epb[p] = std::max(1, M->tile_epb[p] / 2);
   }
+  int64_t elems[kMaxP + 1] = {0};
+  for (int64_t k = 0; k < m.n; ++k) ++elems[m.p[k]];
+  M->modal2 = !m.mapped && modal2_pays(elems);
+  if (M->modal2) {
+    for (int p = 1; p <= kMaxP; ++p) M->tile_epb[p] = apply2_epb(p);
+    append_modal_tables(M);
+    build_modal2(M);
+  }
   build_tiles(M);
   // operation and byte counts of one operator apply, as the kernel does it
   dg_mesh_stats& S = M->stats;
@@ -504,6 +684,7 @@ void build_mesh_host(dg_mesh* M, const dg_mesh_desc* desc, const dg_options* opt
   S.apply_flops = fl;
   S.apply_bytes = 16.0 * (double)M->n_dofs + (double)m.n * (4 + 8 + 8 + 4 + 16) +
                   (double)m.sf.size() * sizeof(SubFaceRec);
+  if (M->modal2) modal2_stats(M);
   if (m.mapped) map_stats(M);
 }
 

@@ -259,8 +259,8 @@ void build_tiles3(dg_mesh* M) {
       }
     }
     M->h_item_ptr.push_back((int32_t)(M->h_items.size() / 2));
-    M->apply3_smem = std::max<int64_t>(M->apply3_smem, 8 * (modal3_doubles(P) + T.count * (int64_t)apply3_elem_doubles(P)));
-    M->modal3_smem = std::max<int64_t>(M->modal3_smem, 8 * (modal3_doubles(P) + T.count * (int64_t)N2 * (P + 1)));
+    M->apply3_smem = std::max<int64_t>(M->apply3_smem, 8 * (modal_table_doubles(P) + T.count * (int64_t)apply3_elem_doubles(P)));
+    M->modal3_smem = std::max<int64_t>(M->modal3_smem, 8 * (modal_table_doubles(P) + T.count * (int64_t)N2 * (P + 1)));
     M->h_tiles.push_back(T);
     i = j;
   }
