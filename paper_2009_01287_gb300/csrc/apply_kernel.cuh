@@ -195,14 +195,14 @@ struct ApplyArgs {
   const int64_t* toff;        // offset of the element's side traces in tr
   double* tr;                 // side traces: [side][node][u, dn]
   const int32_t* sf_ptr;
-  const SubFaceRec* sf;
-  const SubFaceBr2* sfb;      // square meshes, BR2: the multiplied-out liftings
+  const FaceItem* face_items; // squares, nodal
+  const SubFaceBr2* face_br2; // and BR2: the multiplied-out liftings
   const SubFaceModal2* sfm2;  // squares in modes
   const int2* side2;
   const int2* hang2;
   const int4* hang2_tile;
   const SubFaceModal3* sfm3;  // cube meshes
-  const ElemRec3* erec3;      // kernels in modes
+  const ElemRec3* erec3;
   const HangPair* hang3;
   const HangTile* hang_tiles;
   const int2* side3;
@@ -211,7 +211,6 @@ struct ApplyArgs {
   const double* tab;          // basis + face tables
   const int32_t* order;       // degree-sorted element order
   const ApplyTile* tiles;
-  const int2* items;          // square meshes, SIPG: (record, e_local * 4 + s) per sub-face item
   const int32_t* item_ptr;    // items of tile t: [item_ptr[t], item_ptr[t + 1])
   const int2* side_items;     // per (order position, side): first item, count
   double eta;                 // BR2 penalty
@@ -275,17 +274,17 @@ __device__ __forceinline__ void trace_tile(const ApplyArgs& A, const ApplyTile& 
     const int e = t / (4 * NP);
     const int s = (t / NP) & 3;
     const int i = t % NP;
-    const int k = A.order[T.first + e];
-    const double* xk = A.x + A.off[k];
+    const ElemRec3& el = A.erec3[T.first + e];
+    const double* xk = A.x + el.off;
     const double* dv = A.tab + ((s & 1) ? bo.d1 : bo.d0);
     double acc = 0.0;
 #pragma unroll
     for (int q = 0; q < NP; ++q) acc = fma(__ldg(dv + q), ld_x<RO>(xk + side_node(s, i, q, NP)), acc);
-    const double sg = (s & 1) ? A.aih[k] : -A.aih[k];   // a grad u . n
+    const double sg = (s & 1) ? el.aih : -el.aih;   // a grad u . n
     double2 v;
     v.x = ld_x<RO>(xk + side_node(s, i, (s & 1) ? P : 0, NP));
     v.y = sg * acc;
-    reinterpret_cast<double2*>(A.tr + A.toff[k])[s * NP + i] = v;
+    reinterpret_cast<double2*>(A.tr)[(uint32_t)el.toff + s * NP + i] = v;
   }
 }
 
@@ -311,6 +310,7 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs& A, const ApplyTile& 
   const int nnode = count * NN;           // volume / gather tasks
   const int nside = count * 4 * NP;       // face tasks
   const BasisOff bo = A.boff[P];
+  const ElemRec3* er = A.erec3 + T.first;
 
   for (int i = tid; i < NN; i += blockDim.x) {
     sM[i] = __ldg(A.tab + bo.M + i);
@@ -318,7 +318,7 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs& A, const ApplyTile& 
   }
   for (int t = tid; t < nnode; t += blockDim.x) {
     const int e = t / NN;
-    sx[t] = A.x[A.off[A.order[T.first + e]] + (t - e * NN)];
+    sx[t] = A.x[er[e].off + (t - e * NN)];
   }
   __syncthreads();
   // ---- volume pass 1: contract along x
@@ -344,11 +344,8 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs& A, const ApplyTile& 
     double2* part = reinterpret_cast<double2*>(sm + S::PART);   // [nit][NP]
     for (int t = tid; t < nit * NP; t += blockDim.x) {
       const int it = t / NP, i = t - it * NP;
-      const int2 item = A.items[ib + it];   // sorted by branch; item.y >> 16: sub-face order
-      const SubFaceRec f = A.sf[item.x];
-      const int e = (item.y & 0xffff) >> 2, s = item.y & 3;
-      const int k = A.order[T.first + e];
-      const double2* trk = reinterpret_cast<const double2*>(A.tr + A.toff[k]) + s * NP;
+      const FaceItem f = A.face_items[ib + it];   // sorted by branch; where >> 16: sub-face order
+      const double2* trk = reinterpret_cast<const double2*>(A.tr) + f.own;
       const double* Moo = A.tab + f.tab_oo + i * NP;
       double a = 0.0, c = 0.0;
 #pragma unroll
@@ -359,9 +356,9 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs& A, const ApplyTile& 
         c = fma(w, v.y, c);
       }
       double r, c2;
-      if (f.nb < 0) {
+      if (f.pn < 0) {
         if (BR2) {   // eta [M_oo G_o a]: cz (Z u-)_i, Z = M_oo on the whole side
-          const SubFaceBr2 g = A.sfb[item.x];
+          const SubFaceBr2 g = A.face_br2[ib + it];
           double z = a;
           if (!(g.full & 1)) {
             const double* Z = A.tab + g.tab_z + i * NP;
@@ -377,7 +374,7 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs& A, const ApplyTile& 
       } else {
         const int np = f.pn + 1;
         const double* Mon = A.tab + f.tab_on + i * np;
-        const double2* trn = reinterpret_cast<const double2*>(A.tr + A.toff[f.nb]) + f.nb_side * np;
+        const double2* trn = reinterpret_cast<const double2*>(A.tr) + f.nbr;
         double b = 0.0, d = 0.0;
         for (int m = 0; m < np; ++m) {
           const double w = __ldg(Mon + m);
@@ -387,7 +384,7 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs& A, const ApplyTile& 
         }
         const double jmp = a - b;
         if (BR2) {   // eta/4 [M_oo G_o jo + M_on G_n jn] = cz (Z u- - V u+) + cx (X u- - Y u+)
-          const SubFaceBr2 g = A.sfb[item.x];
+          const SubFaceBr2 g = A.face_br2[ib + it];
           const double* X = A.tab + g.tab_x + i * NP;
           double xx = 0.0;
 #pragma unroll
@@ -413,7 +410,7 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs& A, const ApplyTile& 
         }
         c2 = -0.5 * f.len * jmp;
       }
-      part[(item.y >> 16) * NP + i] = make_double2(r, c2);
+      part[(f.where >> 16) * NP + i] = make_double2(r, c2);
     }
     __syncthreads();
     for (int t = tid; t < nside; t += blockDim.x) {
@@ -437,7 +434,7 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs& A, const ApplyTile& 
   for (int t = tid; t < nnode; t += blockDim.x) {
     const int e = t / NN, node = t - e * NN;
     const int ix = node % NP, iy = node / NP;
-    const int k = A.order[T.first + e];
+    const ElemRec3& el = er[e];
     double y = 0.0;
 #pragma unroll
     for (int q = 0; q < NP; ++q) {
@@ -446,8 +443,8 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs& A, const ApplyTile& 
     }
     const double* d0 = A.tab + bo.d0;
     const double* d1 = A.tab + bo.d1;
-    const double aih = A.aih[k];
-    y *= A.ak[k];
+    const double aih = el.aih;
+    y *= el.ah;
     const double* c2 = sc2 + e * 4 * NP;
     const double* r = sr + e * 4 * NP;
     double g = -__ldg(d0 + ix) * c2[0 * NP + iy];
@@ -459,7 +456,7 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs& A, const ApplyTile& 
     if (ix == P) y += r[1 * NP + iy];
     if (iy == 0) y += r[2 * NP + ix];
     if (iy == P) y += r[3 * NP + ix];
-    A.y[A.off[k] + node] = y;
+    A.y[el.off + node] = y;
     part = fma(y, sx[t], part);
   }
   if (A.dot_partial) {

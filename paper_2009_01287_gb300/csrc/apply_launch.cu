@@ -342,8 +342,8 @@ ApplyArgs make_apply_args(const dg_mesh& M, const double* x, double* y, Reduce r
   A.toff = M.d_toff;
   A.tr = M.d_tr;
   A.sf_ptr = M.d_sf_ptr;
-  A.sf = M.d_sf;
-  A.sfb = M.d_sfb;
+  A.face_items = M.d_face_items;
+  A.face_br2 = M.d_face_br2;
   A.sfm2 = M.d_sfm2;
   A.side2 = reinterpret_cast<const int2*>(M.d_side2);
   A.hang2 = reinterpret_cast<const int2*>(M.d_hang2);
@@ -358,7 +358,6 @@ ApplyArgs make_apply_args(const dg_mesh& M, const double* x, double* y, Reduce r
   A.tab = M.d_tables;
   A.order = M.d_order;
   A.tiles = M.d_tiles;
-  A.items = reinterpret_cast<const int2*>(M.d_items);
   A.item_ptr = M.d_item_ptr;
   A.side_items = reinterpret_cast<const int2*>(M.d_side_items);
   A.eta = M.eta;

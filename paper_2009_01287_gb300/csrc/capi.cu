@@ -50,13 +50,14 @@ void upload_tiles(dg_mesh* M, cudaStream_t s) {
   M->apply_grid = apply_kernel_setup(*M);
   M->d_order = a.upload(M->h_order, s);
   M->d_tiles = a.upload(M->h_tiles, s);
-  if (!M->modal2) {
-    M->d_items = a.upload(M->h_items, s);
+  if (M->host.dim == 2) M->d_erec3 = a.upload(M->h_erec3, s);
+  if (M->host.dim == 2 && !M->modal2 && !M->host.mapped) {
+    M->d_face_items = a.upload(M->h_face_items, s);
+    M->d_face_br2 = a.upload(M->h_face_br2, s);
     M->d_item_ptr = a.upload(M->h_item_ptr, s);
     M->d_side_items = a.upload(M->h_side_items, s);
   }
   if (M->modal2) {
-    M->d_erec3 = a.upload(M->h_erec3, s);
     M->d_side2 = a.upload(M->h_side2, s);
     M->d_hang2 = a.upload(M->h_hang2, s);
     M->d_hang2_tile = a.upload(M->h_hang2_tile, s);
@@ -107,10 +108,6 @@ void upload_mesh(dg_mesh* M, cudaStream_t s) {
     }
   }
   M->d_sf_ptr = a.upload(m.sf_ptr, s);
-  if (!M->modal2) {
-    M->d_sf = a.upload(M->h_sf, s);
-    M->d_sfb = M->h_sfb.empty() ? nullptr : a.upload(M->h_sfb, s);
-  }
   if (m.mapped) {
     M->d_mw = a.alloc<double>(M->n_mw);
     M->d_gvol = a.upload(M->h_gvol, s);

@@ -91,6 +91,18 @@ struct SubFaceBr2 {
   double cz, cx;
 };
 
+// A sub-face as the nodal kernel reads it: one record per item of a tile, in
+// the items' order, with the places of both traces, so that an item's loads are
+// its record and then its traces and tables.
+struct alignas(16) FaceItem {
+  uint32_t own, nbr;         // traces of the two sides (double2 units)
+  int32_t tab_oo, tab_on;    // as in SubFaceRec
+  int32_t pn;                // neighbour degree, -1 on the boundary
+  int32_t where;             // side of the tile (4 e + s) | position in sub-face order << 16
+  int32_t pad[2];
+  double sigma, len;
+};
+
 // One sub-face of a cube mesh seen from one of its sides.  The sub-face is a
 // square; its face integrals factor into two 1D tables, one per tangential
 // axis of the side (the lower-numbered axis first).
@@ -158,7 +170,7 @@ constexpr int hang3_doubles(int p) { return 4 * (p + 1) * (p + 1); }   // per pa
 // per element in tile order
 struct ElemRec3 {
   int64_t off;       // first DOF
-  int32_t toff;      // its side traces (double2 units)
+  int32_t toff;      // its side traces (double2 units; nodal squares: unsigned)
   int32_t pad;
   double ah, aih;    // a h^(dim - 2), a / h
 };

@@ -122,7 +122,7 @@ struct dg_mesh {
   std::vector<int32_t> h_side2, h_hang2, h_hang2_tile;
   int64_t n_trace2 = 0;                 // length of the trace buffer (double2)
   std::vector<dg::SubFaceRec3> h_sf3;   // cube meshes
-  // cube meshes, for the kernels (the element records squares in modes too):
+  // cube meshes, for the kernels (the element records squares too):
   // same-size and boundary sub-face records and
   // element records in tile order, the hanging pairs and their tiles, and per
   // (order position, side) {record, 0} or {first result, number of pairs}
@@ -179,6 +179,8 @@ struct dg_mesh {
   std::vector<int32_t> h_items;       // 2 per item: record index, and (e_local * 4 + s, cubes
                                       // e_local * 6 + s) | (position in sub-face order << 16)
   std::vector<int32_t> h_item_ptr;    // n_tiles + 1
+  std::vector<dg::FaceItem> h_face_items;   // plain squares, nodal: one per item, and (BR2) its lifting
+  std::vector<dg::SubFaceBr2> h_face_br2;
   std::vector<int32_t> h_side_items;  // 2 per (order position, side): first item, count
   int64_t apply_smem = 0;             // dynamic shared memory of the 2D operator kernel
   // tile shapes: squares, elements per operator tile of each degree (at most
@@ -197,8 +199,7 @@ struct dg_mesh {
   int64_t* d_toff = nullptr;    // side-trace offsets (8 (p+1) doubles per element)
   double* d_tr = nullptr;       // side traces written by each apply
   int32_t* d_sf_ptr = nullptr;
-  dg::SubFaceRec* d_sf = nullptr;
-  dg::SubFaceBr2* d_sfb = nullptr;
+  dg::SubFaceBr2* d_face_br2 = nullptr;
   dg::SubFaceModal2* d_sfm2 = nullptr;   // squares in modes
   int32_t *d_side2 = nullptr, *d_hang2 = nullptr, *d_hang2_tile = nullptr;
   dg::SubFaceModal3* d_sfm3 = nullptr;   // cube meshes
@@ -219,7 +220,7 @@ struct dg_mesh {
   double* d_tables = nullptr;
   int32_t* d_order = nullptr;
   dg::ApplyTile* d_tiles = nullptr;
-  int32_t* d_items = nullptr;
+  dg::FaceItem* d_face_items = nullptr;
   int32_t* d_item_ptr = nullptr;
   int32_t* d_side_items = nullptr;
   int n_tiles = 0;
@@ -295,6 +296,8 @@ void append_modal_tables(dg_mesh* M);
 void build_modal2(dg_mesh* M);
 void modal2_stats(dg_mesh* M);
 void build_modal2_tiles(dg_mesh* M);
+// nodal squares: element records and the items' records (after the item lists)
+void build_nodal_tiles(dg_mesh* M);
 // cube meshes: degree-sorted order, tiles and their item lists
 void build_tiles3(dg_mesh* M);
 // upload the host-built operator data (M->host.p/off/sf_ptr, h_* arrays)

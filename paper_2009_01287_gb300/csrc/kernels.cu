@@ -602,7 +602,7 @@ pcg_p_trace_kernel(const ApplyArgs A, double* __restrict__ p, const double* __re
   const int nn = np * np;
   for (int t = threadIdx.x; t < T.count * nn; t += blockDim.x) {
     const int e = t / nn;
-    const int64_t i = A.off[A.order[T.first + e]] + (t - e * nn);
+    const int64_t i = A.erec3[T.first + e].off + (t - e * nn);
     p[i] = first ? z[i] : fma(beta, p[i], z[i]);
   }
   __syncthreads();

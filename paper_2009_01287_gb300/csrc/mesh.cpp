@@ -241,6 +241,7 @@ void build_tiles(dg_mesh* M) {
   build_face_items(M);
   if (m.mapped) build_map_faces(M);
   if (M->modal2) build_modal2_tiles(M);
+  else build_nodal_tiles(M);
 }
 
 void build_face_items(dg_mesh* M) {
@@ -392,6 +393,36 @@ void build_modal2(dg_mesh* M) {
         }
       }
   DG_REQUIRE(M->h_tables.size() < (1ULL << 31), "face tables too large");
+}
+
+void build_nodal_tiles(dg_mesh* M) {
+  const HostMesh& m = M->host;
+  std::vector<int64_t> toff(m.n + 1, 0);
+  for (int64_t k = 0; k < m.n; ++k) toff[k + 1] = toff[k] + 4 * (m.p[k] + 1);
+  DG_REQUIRE(toff[m.n] < (1LL << 32), "too many side traces");
+  M->h_erec3.clear();
+  for (int32_t k : M->h_order)
+    M->h_erec3.push_back({m.off[k], (int32_t)(uint32_t)toff[k], 0, m.coef[k], m.coef[k] / M->h_h[k]});
+  M->h_face_items.clear();
+  M->h_face_br2.clear();
+  if (m.mapped) return;
+  for (size_t t = 0; t < M->h_tiles.size(); ++t)
+    for (int64_t g = M->h_item_ptr[t]; g < M->h_item_ptr[t + 1]; ++g) {
+      const int32_t rec = M->h_items[2 * g], where = M->h_items[2 * g + 1], s = where & 3;
+      const int64_t k = M->h_order[M->h_tiles[t].first + ((where & 0xffff) >> 2)];
+      const SubFaceRec& r = M->h_sf[rec];
+      FaceItem f{};
+      f.own = (uint32_t)(toff[k] + s * (m.p[k] + 1));
+      f.pn = r.nb >= 0 ? r.pn : -1;
+      if (r.nb >= 0) f.nbr = (uint32_t)(toff[r.nb] + r.nb_side * (r.pn + 1));
+      f.tab_oo = r.tab_oo;
+      f.tab_on = r.tab_on;
+      f.where = where;
+      f.sigma = r.sigma;
+      f.len = r.len;
+      M->h_face_items.push_back(f);
+      if (!M->h_sfb.empty()) M->h_face_br2.push_back(M->h_sfb[rec]);
+    }
 }
 
 // FP64 operations of both kernels in modes (a multiply-add, a product and a sum
@@ -631,23 +662,35 @@ void build_mesh_host(dg_mesh* M, const dg_mesh_desc* desc, const dg_options* opt
     g.tab_x += base;
     g.tab_y += base;
   }
+  int64_t elems[kMaxP + 1] = {0};
+  for (int64_t k = 0; k < m.n; ++k) ++elems[m.p[k]];
+  auto tiles = [&] {
+    int64_t t = 0;
+    for (int p = 1; p <= kMaxP; ++p) t += (elems[p] + M->tile_epb[p] - 1) / M->tile_epb[p];
+    return t;
+  };
+  auto halve = [&] {
+    for (int p = 1; p <= kMaxP; ++p) M->tile_epb[p] = std::max(1, M->tile_epb[p] / 2);
+  };
+  M->modal2 = !m.mapped && modal2_pays(elems);
   if (m.mapped) {
     build_mesh_map(M, desc);   // the mapped records, tables and factors
     // fewer tiles than SMs: half the elements per tile (24k unknowns, 109 tiles:
     // 3.1 us of 70 per PCG iteration; a quarter was no better)
-    int64_t cnt[kMaxP + 1] = {0}, tiles = 0;
-    for (int64_t k = 0; k < m.n; ++k) ++cnt[m.p[k]];
-    for (int p = 1; p <= kMaxP; ++p) tiles += (cnt[p] + M->tile_epb[p] - 1) / M->tile_epb[p];
-    if (tiles < 152)
-      for (int p = 1; p <= kMaxP; ++p) M->tile_epb[p] = std::max(1, M->tile_epb[p] / 2);
-  }
-  int64_t elems[kMaxP + 1] = {0};
-  for (int64_t k = 0; k < m.n; ++k) ++elems[m.p[k]];
-  M->modal2 = !m.mapped && modal2_pays(elems);
-  if (M->modal2) {
+    if (tiles() < 152) halve();
+  } else if (M->modal2) {
     for (int p = 1; p <= kMaxP; ++p) M->tile_epb[p] = apply2_epb(p);
     append_modal_tables(M);
     build_modal2(M);
+  } else {
+    // fewer tiles than SMs: fewer elements per tile, down to about four warps of
+    // nodes.  A full tile of 250 nodes is about 800 FP64 warp instructions, 8 us
+    // on its SM (2.5k unknowns, L-shape: 31.3 -> 29.5 us per PCG iteration; down to
+    // two warps the 576 unknowns of 64 elements of degree 2 took 1.3% longer).
+    for (int p = kMaxP; p >= 1; --p) {   // the heaviest tiles first
+      const int least = std::max(1, 128 / ((p + 1) * (p + 1)));
+      if (tiles() < 152) M->tile_epb[p] = std::min(M->tile_epb[p], least);
+    }
   }
   build_tiles(M);
   // operation and byte counts of one operator apply, as the kernel does it
