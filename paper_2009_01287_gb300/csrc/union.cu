@@ -24,13 +24,12 @@ namespace {
 
 void append_rows(Csr& out, const Csr& in, int64_t col_shift) {
   if (out.ptr.empty()) out.ptr.push_back(0);
-  for (int64_t i = 0; i < in.rows; ++i) {
-    for (int64_t t = in.ptr[i]; t < in.ptr[i + 1]; ++t) {
-      out.idx.push_back((int32_t)(in.idx[t] + col_shift));
-      out.val.push_back(in.val[t]);
-    }
-    out.ptr.push_back((int64_t)out.idx.size());
-  }
+  if (in.rows == 0) return;
+  const int64_t at = (int64_t)out.idx.size(), first = in.ptr[0], n = in.ptr[in.rows] - first;
+  out.idx.resize(at + n);
+  for (int64_t t = 0; t < n; ++t) out.idx[at + t] = (int32_t)(in.idx[first + t] + col_shift);
+  out.val.insert(out.val.end(), in.val.begin() + first, in.val.begin() + first + n);
+  for (int64_t i = 0; i < in.rows; ++i) out.ptr.push_back(at + in.ptr[i + 1] - first);
   out.rows += in.rows;
 }
 

@@ -38,7 +38,6 @@ CsrTierPlan plan_csr_tiers(const Csr& C) {
 
 SlicePlan plan_slices(const Csr& C) {
   SlicePlan S;
-  const CsrTierPlan tiers = plan_csr_tiers(C);
   auto len = [&](int64_t i) { return C.ptr[i + 1] - C.ptr[i]; };
   auto lanes_for = [&](int64_t n, int rounds) {
     int g = 1;
@@ -51,11 +50,12 @@ SlicePlan plan_slices(const Csr& C) {
     for (int64_t i = 0; i < C.rows; ++i) lanes += lanes_for(len(i), rounds);
     if (lanes >= kResidentThreads / 2) break;
   }
-  // rows of a whole CTA: the CTA tier, and the warp tier's above the limit
+  // rows of a whole CTA, longest first
   std::vector<char> cta(C.rows, 0);
-  std::vector<int32_t> wide = tiers.cta;
-  for (int32_t i : tiers.warp)
-    if (lanes_for(len(i), rounds) > 32) wide.push_back(i);
+  std::vector<int32_t> wide;
+  for (int64_t i = 0; i < C.rows; ++i)
+    if (lanes_for(len(i), rounds) > 32) wide.push_back((int32_t)i);
+  std::stable_sort(wide.begin(), wide.end(), [&](int32_t x, int32_t y) { return len(x) > len(y); });
   int64_t at = 0;   // in units of 32 entries
   for (int32_t i : wide) {
     cta[i] = 1;
@@ -65,28 +65,36 @@ SlicePlan plan_slices(const Csr& C) {
     at += 8 * (int64_t)nr;
     ++S.n_cta;
   }
-  // classes of (rounds, lanes), the longest first
-  std::vector<std::pair<int32_t, int32_t>> order;   // (class key, row)
-  order.reserve(C.rows);
+  // classes of (rounds, lanes), the longest first: rows counted into them, in
+  // row order within a class
+  constexpr int kClasses = 64 * 129;   // at most 128 rounds of at most 32 lanes
+  std::vector<int32_t> cls(C.rows);
+  std::vector<int64_t> at_class(kClasses + 1, 0);
   for (int64_t i = 0; i < C.rows; ++i) {
     if (cta[i]) continue;
     const int g = lanes_for(len(i), rounds);
-    order.push_back({-(int32_t)(((len(i) + g - 1) / g) * 64 + g), (int32_t)i});
+    cls[i] = (int32_t)(((len(i) + g - 1) / g) * 64 + g);
+    ++at_class[kClasses - 1 - cls[i]];
   }
-  std::stable_sort(order.begin(), order.end(),
-                   [](const std::pair<int32_t, int32_t>& a, const std::pair<int32_t, int32_t>& b) {
-                     return a.first < b.first;
-                   });
-  for (size_t i = 0; i < order.size();) {
-    const int32_t key = -order[i].first, g = key % 64, nr = key / 64;
-    S.hdr.insert(S.hdr.end(), {(int32_t)at, nr, g, (int32_t)S.row.size()});
-    for (int r = 0; r < 32 / g; ++r) {
-      const bool has = i < order.size() && order[i].first == -key;
-      S.row.push_back(has ? order[i].second : -1);
-      if (has) ++i;
+  for (int64_t k = 0, sum = 0; k <= kClasses; ++k) {
+    const int64_t n = at_class[k];
+    at_class[k] = sum;
+    sum += n;
+  }
+  std::vector<int32_t> order(at_class[kClasses]);
+  {
+    std::vector<int64_t> pos(at_class);
+    for (int64_t i = 0; i < C.rows; ++i)
+      if (!cta[i]) order[pos[kClasses - 1 - cls[i]]++] = (int32_t)i;
+  }
+  for (int k = 0; k < kClasses; ++k) {
+    const int32_t key = kClasses - 1 - k, g = key % 64, nr = key / 64;
+    for (int64_t i = at_class[k]; i < at_class[k + 1];) {
+      S.hdr.insert(S.hdr.end(), {(int32_t)at, nr, g, (int32_t)S.row.size()});
+      for (int r = 0; r < 32 / g; ++r) S.row.push_back(i < at_class[k + 1] ? order[i++] : -1);
+      at += nr;
+      ++S.n_warp;
     }
-    at += nr;
-    ++S.n_warp;
   }
   DG_REQUIRE(at < (1LL << 31) && S.row.size() < (1ULL << 31), "matrix too large for its slices");
   S.entries = 32 * at;

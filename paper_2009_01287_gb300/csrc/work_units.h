@@ -37,8 +37,8 @@ void plan_block_units(const std::vector<int32_t>& dims, const std::vector<int32_
 // number of rounds, in row order; entry j of a row is read by lane j mod lanes
 // in round j / lanes, so that every round of a slice is 32 consecutive entries.
 // rounds is the largest of 16, 8, 4 that still gives half the GPU's threads a
-// lane; rows of more than 128 * rounds entries, and the CTA tier of
-// plan_csr_tiers, make slices of 256 lanes.
+// lane; rows of more than 128 * rounds entries or more than kCsrCtaRow make
+// slices of 256 lanes.
 struct SlicePlan {
   std::vector<int32_t> hdr;   // 4 per slice, see DevSlices
   std::vector<int32_t> row;
@@ -58,10 +58,13 @@ void fill_slices(const Csr& C, const SlicePlan& S, std::vector<int32_t>& idx, st
       const int32_t row = S.row[h[3] + r];
       if (row < 0) continue;
       const int64_t b = C.ptr[row], len = C.ptr[row + 1] - b;
-      for (int64_t j = 0; j < len; ++j) {
-        const int64_t e = 32 * (int64_t)h[0] + (j / lanes) * width + r * lanes + j % lanes;
-        idx[e] = C.idx[b + j];
-        val[e] = (T)C.val[b + j];
+      int64_t e = 32 * (int64_t)h[0] + r * lanes;
+      for (int64_t j = 0; j < len; j += lanes, e += width) {   // a round
+        const int64_t n = len - j < lanes ? len - j : lanes;
+        for (int64_t u = 0; u < n; ++u) {
+          idx[e + u] = C.idx[b + j + u];
+          val[e + u] = (T)C.val[b + j + u];
+        }
       }
     }
   }
