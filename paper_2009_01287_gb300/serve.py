@@ -31,8 +31,10 @@ from __future__ import annotations
 import dataclasses
 import hashlib
 import heapq
+import itertools
 import threading
 import time
+import weakref
 from collections import OrderedDict
 from typing import Dict, List, Optional
 
@@ -78,10 +80,31 @@ class Result:
         return self.finished - self.arrival
 
 
+_map_tokens: dict = {}   # id -> (reference, token); an id alone is taken again after its object is gone
+_map_lock = threading.Lock()
+_map_count = itertools.count()
+
+
+def _map_token(f) -> int:
+    """A number of this map object's own, never given to another."""
+    with _map_lock:
+        known = _map_tokens.get(id(f))
+        if known is None or known[0]() is not f:
+            try:
+                ref = weakref.ref(f)
+            except TypeError:   # takes no weak reference: kept
+                ref = lambda: f   # noqa: E731
+            known = (ref, next(_map_count))
+            _map_tokens[id(f)] = known
+            for k in [k for k, (ref, _) in _map_tokens.items() if ref() is None]:
+                del _map_tokens[k]
+        return known[1]
+
+
 def mesh_key(m: MeshDesc) -> str:
     """Cache key of a mesh: its boxes, degrees, coefficient and geometry (the
-    corners' values; a caller's map by the identity of the map object, which
-    must not change while the server holds the mesh)."""
+    corners' values; a caller's map by the map object, which must not change
+    while the server holds the mesh)."""
     h = hashlib.sha1()
     for a in (m.lo, m.size, m.p, np.asarray(m.extent)):
         h.update(np.ascontiguousarray(a).tobytes())
@@ -92,7 +115,7 @@ def mesh_key(m: MeshDesc) -> str:
         h.update(b"corners")
         h.update(np.ascontiguousarray(m.corners, dtype=np.float64).tobytes())
     if getattr(m, "mapping", None) is not None:
-        h.update(b"map%d" % id(m.mapping))
+        h.update(b"map%d" % _map_token(m.mapping))
     h.update(repr((m.dim, m.lattice_h)).encode())
     return h.hexdigest()
 
