@@ -249,34 +249,41 @@ def operator_rooflines(B, ctx, M, mesh, peak_tf, peaks, three, tkey, mapped=Fals
         ap.append(t.apply_ms)
     apply_ms, trace_ms = statistics.mean(ap), statistics.mean(tr)
     st = M.stats
-    tfl = trace_flops(mesh)
+    separable = not (three or mapped)
+    # boxes: the tiles' kernel alone; cubes and mapped squares: with the kernels
+    # that form the modes or the sub-face weights, which share the work counted
+    tfl = trace_flops(mesh) if separable else 0.0
     kfl = st.apply_flops - tfl
-    ach = kfl / (apply_ms / 1e3) / 1e12
-    name = ("apply3_kernel (BR2 operator on cubes, FP64)" if three else
-            "apply_map_kernel (SIPG operator on mapped squares, FP64)" if mapped else
+    op_ms = apply_ms if separable else apply_ms + trace_ms
+    ach = kfl / (op_ms / 1e3) / 1e12
+    name = ("modal3_kernel + hang3_kernel + apply3_kernel (BR2 operator on cubes, FP64)" if three else
+            "trace_kernel + map_face_kernel + apply_map_kernel (SIPG operator on mapped squares, FP64)" if mapped else
             "apply_kernel (SIPG operator, FP64)")
     model = ("FMAs of the kernel as formulated (x2), counted on the host from the mesh: volume 8 n^3, face "
              "terms 8 n (n + n_nb) per sub-face side, test-function normal derivatives 8 n^2 per element "
              "(n = p+1)")
     if mapped:
-        model = ("FMAs of the kernel as formulated (x2), counted on the host from the mesh: volume at q = p+2 "
-                 "Gauss points 4 n q (n + q) plus 24 q^2 for the geometric factors, per sub-face side and "
-                 "Gauss point 6 (n + n_nb) + 60 (traces, geometry) and 6 n (side sums), test-function normal "
-                 "derivatives 8 n^2 per element (n = p+1)")
-    separable = not (three or mapped)
+        model = ("FMAs of the kernels as formulated (x2), counted on the host from the mesh: volume at q = p+2 "
+                 "Gauss points, per sub-face and Gauss point both sides' traces and the three weights once, per "
+                 "side the sums of the weights, test-function normal derivatives (n = p+1)")
+    if three:
+        model = ("FP64 operations of the three kernels (x2), counted on the host from the mesh: per line of modes "
+                 "the transforms by parity, half a stiffness product, traces and lifts, per side mode five, per "
+                 "hanging sub-face four or five restrictions")
     main = {"kernel": name, "bound": "alu", "achieved": ach, "peak": peak_tf, "unit": "TFLOP/s",
             "frac": ach / peak_tf, "traffic": traffic(tkey),
-            "flops_per_launch": kfl, "launch_ms": apply_ms,
+            "flops_per_launch": kfl, "launch_ms": op_ms,
             "flops_model": model,
             "flops_scope_model_per_launch": scope_model_flops(mesh) if separable else None,
             "frac_scope_model": (scope_model_flops(mesh) / (apply_ms / 1e3) / 1e12 / peak_tf
                                   if separable else None),
             "algorithmic_bytes": st.apply_bytes,
-            "hbm_gbs": st.apply_bytes / (apply_ms / 1e3) / 1e9,
-            "hbm_frac": st.apply_bytes / (apply_ms / 1e3) / 1e9 / peaks["hbm_gbs"],
+            "hbm_gbs": st.apply_bytes / (op_ms / 1e3) / 1e9,
+            "hbm_frac": st.apply_bytes / (op_ms / 1e3) / 1e9 / peaks["hbm_gbs"],
             "peak_source": "FP64 FMA-chain probe (dg_fp64_fma_probe) in this run; HBM of measured"}
-    trace = {"kernel": "trace3_kernel" if three else "trace_kernel", "bound": "hbm",
-             "launch_ms": trace_ms, "flops_per_launch": tfl,
+    trace = {"kernel": ("modal3_kernel + hang3_kernel" if three else "trace_kernel + map_face_kernel" if mapped
+                        else "trace_kernel"), "bound": "hbm",
+             "launch_ms": trace_ms, "flops_per_launch": tfl if separable else None,
              "note": "inside PCG the traces are written by the p-update kernel, not by this kernel"}
     # side traces: read x once, write u and dn at every side node
     import numpy as np

@@ -178,8 +178,9 @@ typedef struct {
                              per-element and per-sub-face records read once     */
   int64_t device_bytes;   /* device memory held by the mesh handle              */
   int32_t tile_elems[9];  /* squares: elements per operator tile of degree p
-                             (index p), fixed rule min(16, 256/(p+1)^2) (half of
-                             it on mapped meshes of few tiles) unless tuned     */
+                             (index p), fixed rule min(16, 256/(p+1)^2), fewer on
+                             meshes of fewer tiles than SMs, 32/(p+1) on large
+                             ones in Legendre modes, unless tuned               */
   int64_t tile_smem_budget; /* cubes: shared-memory budget of an operator tile
                                (bytes)                                           */
   int32_t tiles_tuned;    /* 1: chosen by timing (dg_options.tune_tiles)        */

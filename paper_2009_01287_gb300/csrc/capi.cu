@@ -718,8 +718,8 @@ extern "C" dg_status dg_pcg_solve_noalloc(const dg_mesh* mesh, const dg_precond*
       throw Error(DG_EINVAL, "dg_pcg_solve_noalloc: n_dofs " + std::to_string(mesh->n_dofs) +
                                  " exceeds the static scratch limit of " +
                                  std::to_string(kNoAllocMaxDofs));
-    // implied by the DOF limit (a tile holds at least three elements' nodes, 243
-    // or more), kept as a guard of the partials' slice
+    // a guard of the partials' slice: a full tile holds at least 64 nodes, 32 when
+    // tuned (meshes of fewer tiles than SMs aside)
     if (mesh->n_tiles > kNoAllocMaxTiles)
       throw Error(DG_EINVAL, "dg_pcg_solve_noalloc: mesh needs more operator tiles than the static scratch holds");
     DG_REQUIRE(pc && b && x, "null argument");
