@@ -465,6 +465,7 @@ def inspect_lib():
         L.dginspect_apply.argtypes = [vp, vp, vp]
         L.dginspect_item_sizes.argtypes = [vp, vp]
         L.dginspect_items.argtypes = [vp, vp, vp, vp, vp]
+        L.dginspect_hanging3.argtypes = [vp, vp, vp, vp]
         L.dginspect_block_units.argtypes = [C.c_int64, vp, vp, vp, vp, vp, vp, C.c_int64]
         L.dginspect_block_units.restype = C.c_int64
         L.dginspect_csr_tiers.argtypes = [C.c_int64, vp, vp, vp, vp, vp]
@@ -570,8 +571,8 @@ class HostSetup:
         return b
 
     def face_items(self):
-        """The operator's tiles and sub-face items as the kernels read them:
-        (item_ptr, items (n, 2), chunk per tile, info (n, 3): interior,
+        """The operator's tiles and their sub-faces as flat lists (squares: as
+        the nodal kernel reads them): (item_ptr, items (n, 2), chunk per tile, info (n, 3): interior,
         neighbour degree, whole-side flags)."""
         L = inspect_lib()
         s = np.zeros(3, dtype=np.int64)
@@ -583,6 +584,19 @@ class HostSetup:
         info = np.zeros(3 * max(ni, 1), dtype=np.int32)
         L.dginspect_items(self.h, ptr.ctypes.data, items.ctypes.data, chunk.ctypes.data, info.ctypes.data)
         return ptr, items[:2 * ni].reshape(ni, 2), chunk[:nt], info[:3 * ni].reshape(ni, 3)
+
+    def hanging3(self):
+        """Cubes: the hanging sub-faces as the kernels take them: (pairs (n, 6):
+        trace of the larger and of the smaller side, result of either, places of
+        a trace of either; sides in tile order (m, 3): element, first result,
+        number of results)."""
+        L = inspect_lib()
+        cnt = np.zeros(2, dtype=np.int64)
+        L.dginspect_hanging3(self.h, cnt.ctypes.data, None, None)
+        pairs = np.zeros((max(int(cnt[0]), 1), 6), dtype=np.int64)
+        sides = np.zeros((max(int(cnt[1]), 1), 3), dtype=np.int64)
+        L.dginspect_hanging3(self.h, cnt.ctypes.data, pairs.ctypes.data, sides.ctypes.data)
+        return pairs[:cnt[0]], sides[:cnt[1]]
 
     def __del__(self):
         try:

@@ -204,7 +204,6 @@ struct ApplyTile {
   int32_t first;     // index into the degree-sorted element order
   int32_t count;
   int32_t inst;      // batch instance of the tile's elements (0 for a single mesh)
-  int32_t chunk;     // 3D: sub-face items sorted together (the whole tile)
 };
 
 // ------------------------------------------------------------------ mapped squares

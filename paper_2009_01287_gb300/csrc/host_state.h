@@ -173,11 +173,11 @@ struct dg_mesh {
   dg::BasisOff boff[dg::kMaxP + 1];
   std::vector<dg::ApplyTile> h_tiles;
   std::vector<int32_t> h_order;      // degree-sorted element order
-  // square meshes, SIPG: the sub-face work of every tile as a flat list of
+  // squares: the sub-face work of every tile as a flat list of
   // (record, tile-local side) items, and per element side (in tile order) the
   // first item and the item count
-  std::vector<int32_t> h_items;       // 2 per item: record index, and (e_local * 4 + s, cubes
-                                      // e_local * 6 + s) | (position in sub-face order << 16)
+  std::vector<int32_t> h_items;       // 2 per item: record index, and (e_local * 4 + s) |
+                                      // (position in sub-face order << 16)
   std::vector<int32_t> h_item_ptr;    // n_tiles + 1
   std::vector<dg::FaceItem> h_face_items;   // plain squares, nodal: one per item, and (BR2) its lifting
   std::vector<dg::SubFaceBr2> h_face_br2;

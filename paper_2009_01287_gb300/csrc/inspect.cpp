@@ -3,8 +3,11 @@
 // AMG hierarchy - and the host mirror of the operator, without a GPU, so that
 // they can be compared with an independent implementation on a CPU machine.
 // Not part of the solver ABI (include/dg.h); every call is synchronous.
+#include <algorithm>
 #include <cstring>
 #include <memory>
+#include <utility>
+#include <vector>
 
 #include "dg_internal.h"
 #include "host_state.h"
@@ -106,27 +109,82 @@ void* dginspect_create(const dg_mesh_desc* desc, const dg_options* opts, int wit
 
 void dginspect_destroy(void* h) { delete (Inspect*)h; }
 
+namespace {
+// The sub-faces of every tile as a flat list of (record, tile-local side)
+// items.  Squares: as the nodal kernel reads them.  Cubes (their kernels take
+// the sides' records and the hanging pairs instead): in chunks of at most
+// kCubeChunk items, each sorted by the kind of sub-face - interior first, then
+// the BR2 whole-side flags, then the neighbour degree - with the item's
+// position in sub-face order in the high half of the side field.
+constexpr int64_t kCubeChunk = 4096;
+struct ItemList {
+  std::vector<int32_t> ptr, item, chunk;
+};
+ItemList item_list(const dg_mesh& M) {
+  ItemList L;
+  const HostMesh& m = M.host;
+  if (m.dim == 2) {
+    L.ptr = M.h_item_ptr;
+    L.item = M.h_items;
+    for (int t = 0; t < M.n_tiles; ++t) L.chunk.push_back(L.ptr[t + 1] - L.ptr[t]);
+    return L;
+  }
+  const bool br2 = M.opts.form == DG_FORM_BR2;
+  L.ptr.push_back(0);
+  for (const ApplyTile& T : M.h_tiles) {
+    const int64_t t0 = (int64_t)L.item.size() / 2;
+    for (int e = 0; e < T.count; ++e) {
+      const int64_t k = M.h_order[T.first + e];
+      for (int s = 0; s < 6; ++s)
+        for (int32_t j = m.sf_ptr[6 * k + s]; j < m.sf_ptr[6 * k + s + 1]; ++j)
+          L.item.insert(L.item.end(), {j, 6 * e + s});
+    }
+    const int64_t t1 = (int64_t)L.item.size() / 2, chunk = std::min(t1 - t0, kCubeChunk);
+    for (int64_t c0 = t0; c0 < t1; c0 += chunk) {
+      const int64_t c1 = std::min(c0 + chunk, t1);
+      const std::vector<int32_t> rec(L.item.begin() + 2 * c0, L.item.begin() + 2 * c1);
+      std::vector<std::pair<int32_t, int32_t>> key;   // (kind, position in the chunk)
+      for (int64_t g = c0; g < c1; ++g) {
+        const SubFaceRec3& f = M.h_sf3[L.item[2 * g]];
+        const bool in = f.nb >= 0;
+        const int zv = (br2 && !(f.full & 1)) ? 1 : 0, yy = (br2 && in && !(f.full & 2)) ? 1 : 0;
+        key.push_back({((in ? 0 : 1) << 12) | (zv << 11) | (yy << 10) | (in ? 16 - f.pn : 0), (int32_t)(g - c0)});
+      }
+      std::sort(key.begin(), key.end());
+      for (int64_t g = c0; g < c1; ++g) {
+        const int32_t pos = key[g - c0].second;
+        L.item[2 * g] = rec[2 * pos];
+        L.item[2 * g + 1] = rec[2 * pos + 1] | (pos << 16);
+      }
+    }
+    L.ptr.push_back((int32_t)t1);
+    L.chunk.push_back((int32_t)chunk);
+  }
+  return L;
+}
+}  // namespace
+
 // the operator's tiles and sub-face items: out = [n_tiles, n_items, dim]
 void dginspect_item_sizes(void* h, int64_t* out) {
   const dg_mesh& M = ((Inspect*)h)->mesh;
   out[0] = M.n_tiles;
-  out[1] = (int64_t)M.h_items.size() / 2;
+  out[1] = (int64_t)item_list(M).item.size() / 2;
   out[2] = M.host.dim;
 }
 
-// item_ptr (n_tiles + 1), items (2 per item, as the kernels read them), per
-// tile its chunk length (cubes; squares: the tile's item count), and per item
-// the fields its branches depend on: interior (0/1), neighbour degree, the
-// whole-side flags (BR2 records; 0 without them)
+// item_ptr (n_tiles + 1), items (2 per item, see item_list), per tile its
+// chunk length (cubes; squares: the tile's item count), and per item the
+// fields its kind depends on: interior (0/1), neighbour degree, the whole-side
+// flags (BR2 records; 0 without them)
 void dginspect_items(void* h, int32_t* item_ptr, int32_t* items, int32_t* chunk, int32_t* info) {
   const dg_mesh& M = ((Inspect*)h)->mesh;
-  std::memcpy(item_ptr, M.h_item_ptr.data(), M.h_item_ptr.size() * sizeof(int32_t));
-  std::memcpy(items, M.h_items.data(), M.h_items.size() * sizeof(int32_t));
-  for (int t = 0; t < M.n_tiles; ++t)
-    chunk[t] = M.host.dim == 3 ? M.h_tiles[t].chunk : M.h_item_ptr[t + 1] - M.h_item_ptr[t];
-  const int64_t n = (int64_t)M.h_items.size() / 2;
+  const ItemList L = item_list(M);
+  std::copy(L.ptr.begin(), L.ptr.end(), item_ptr);
+  std::copy(L.item.begin(), L.item.end(), items);
+  std::copy(L.chunk.begin(), L.chunk.end(), chunk);
+  const int64_t n = (int64_t)L.item.size() / 2;
   for (int64_t g = 0; g < n; ++g) {
-    const int32_t r = M.h_items[2 * g];
+    const int32_t r = L.item[2 * g];
     if (M.host.dim == 3) {
       const SubFaceRec3& f = M.h_sf3[r];
       info[3 * g] = f.nb >= 0 ? 1 : 0;
@@ -138,6 +196,30 @@ void dginspect_items(void* h, int32_t* item_ptr, int32_t* items, int32_t* chunk,
       info[3 * g + 1] = f.pn;
       info[3 * g + 2] = M.h_sfb.empty() ? 0 : M.h_sfb[r].full;
     }
+  }
+}
+
+// Cubes: the hanging sub-faces as the kernels take them.  counts = [pairs,
+// sides]; with the arrays given, per pair {trace of the larger side, of the
+// smaller, result of the larger, of the smaller, places of a larger and of a
+// smaller trace} and per side, in tile order, {element, first result, number
+// of results; 0 on a side without hanging sub-faces}.
+void dginspect_hanging3(void* h, int64_t* counts, int64_t* pairs, int64_t* sides) {
+  const dg_mesh& M = ((Inspect*)h)->mesh;
+  counts[0] = (int64_t)M.h_hang3.size();
+  counts[1] = (int64_t)M.h_side3.size() / 2;
+  if (!pairs || !sides) return;
+  for (const HangTile& T : M.h_hang_tiles)
+    for (int i = T.first; i < T.first + T.count; ++i) {
+      const HangPair& p = M.h_hang3[i];
+      const int64_t v[6] = {p.src_b, p.src_s, p.dst_b, p.dst_s, (T.p + 1) * (T.p + 1), p.ns * p.ns};
+      std::copy(v, v + 6, pairs + 6 * (int64_t)i);
+    }
+  for (int64_t i = 0; i < counts[1]; ++i) {
+    const bool hanging = M.h_side3[2 * i + 1] > 0;
+    sides[3 * i] = M.h_order[i / 6];
+    sides[3 * i + 1] = hanging ? M.h_side3[2 * i] : 0;
+    sides[3 * i + 2] = M.h_side3[2 * i + 1];
   }
 }
 

@@ -149,11 +149,9 @@ constexpr int kTilesPerSm = 3;
 // a run of elements of equal (p, nq), nq = max(p, neighbour degrees) + 1, both
 // descending, of at most apply3_epb(p) elements (scaled with the tile's
 // shared-memory budget, and halved on small meshes until there are kTilesPerSm
-// tiles per SM).  The tile's sub-faces are
-// also listed flat as (record, side) items in host order.
+// tiles per SM).  A side may have any number of sub-faces.
 void build_tiles3(dg_mesh* M) {
   const HostMesh& m = M->host;
-  const bool br2 = M->opts.form == DG_FORM_BR2;
   std::vector<int32_t> nq(m.n);
   for (int64_t k = 0; k < m.n; ++k) {
     int q = m.p[k] + 1;
@@ -182,9 +180,6 @@ void build_tiles3(dg_mesh* M) {
     if (tiles >= kTilesPerSm * 152 || !more) break;
   }
   M->h_tiles.clear();
-  M->h_items.clear();
-  M->h_item_ptr.assign(1, 0);
-  M->h_side_items.assign(12 * (size_t)m.n, 0);
   M->h_sfm3.clear();
   M->h_erec3.clear();
   M->h_side3.assign(12 * (size_t)m.n, 0);
@@ -205,12 +200,6 @@ void build_tiles3(dg_mesh* M) {
       M->h_erec3.push_back({m.off[k], M->h_toff3[k], 0, a * h, a / h});
       for (int s = 0; s < 6; ++s) {
         const int b = m.sf_ptr[6 * (int64_t)k + s], c = m.sf_ptr[6 * (int64_t)k + s + 1] - b;
-        M->h_side_items[12 * pos + 2 * s] = (int32_t)(M->h_items.size() / 2);
-        M->h_side_items[12 * pos + 2 * s + 1] = c;
-        for (int q = 0; q < c; ++q) {
-          M->h_items.push_back(b + q);
-          M->h_items.push_back((int32_t)(6 * e + s));
-        }
         int32_t* sd = &M->h_side3[12 * pos + 2 * s];
         if (M->h_resoff3[b] >= 0) {   // hanging: its results, one after another
           sd[0] = M->h_resoff3[b];
@@ -233,32 +222,6 @@ void build_tiles3(dg_mesh* M) {
         M->h_sfm3.push_back(r);
       }
     }
-    // Host order of the items: by the branches their threads take - interior
-    // first, then the BR2 whole-face flags, then the neighbour degree; the high
-    // half of the side field keeps the item's position in sub-face order.
-    {
-      const int64_t t0 = M->h_item_ptr.back(), t1 = (int64_t)M->h_items.size() / 2;
-      DG_REQUIRE(t1 - t0 < 65536, "3D operator: too many sub-faces in a tile");
-      T.chunk = (int32_t)(t1 - t0);
-      std::vector<std::pair<int32_t, int32_t>> key;   // (branch key, position in the tile)
-      const std::vector<int32_t> rec(M->h_items.begin() + 2 * t0, M->h_items.end());
-      for (int64_t g = t0; g < t1; ++g) {
-        const SubFaceRec3& f = M->h_sf3[M->h_items[2 * g]];
-        const bool in = f.nb >= 0;
-        const int zv = (br2 && !(f.full & 1)) ? 1 : 0, yy = (br2 && in && !(f.full & 2)) ? 1 : 0;
-        key.push_back({((in ? 0 : 1) << 12) | (zv << 11) | (yy << 10) | (in ? 16 - f.pn : 0), (int32_t)(g - t0)});
-      }
-      std::stable_sort(key.begin(), key.end(),
-                       [](const std::pair<int32_t, int32_t>& x, const std::pair<int32_t, int32_t>& y) {
-                         return x.first < y.first;
-                       });
-      for (int64_t g = t0; g < t1; ++g) {
-        const int32_t pos = key[g - t0].second;
-        M->h_items[2 * g] = rec[2 * pos];
-        M->h_items[2 * g + 1] = rec[2 * pos + 1] | (pos << 16);
-      }
-    }
-    M->h_item_ptr.push_back((int32_t)(M->h_items.size() / 2));
     M->apply3_smem = std::max<int64_t>(M->apply3_smem, 8 * (modal_table_doubles(P) + T.count * (int64_t)apply3_elem_doubles(P)));
     M->modal3_smem = std::max<int64_t>(M->modal3_smem, 8 * (modal_table_doubles(P) + T.count * (int64_t)N2 * (P + 1)));
     M->h_tiles.push_back(T);
