@@ -466,6 +466,7 @@ def inspect_lib():
         L.dginspect_item_sizes.argtypes = [vp, vp]
         L.dginspect_items.argtypes = [vp, vp, vp, vp, vp]
         L.dginspect_hanging3.argtypes = [vp, vp, vp, vp]
+        L.dginspect_place_traces3.argtypes = [vp, C.c_int64]
         L.dginspect_block_units.argtypes = [C.c_int64, vp, vp, vp, vp, vp, vp, C.c_int64]
         L.dginspect_block_units.restype = C.c_int64
         L.dginspect_csr_tiers.argtypes = [C.c_int64, vp, vp, vp, vp, vp]
@@ -585,12 +586,14 @@ class HostSetup:
         L.dginspect_items(self.h, ptr.ctypes.data, items.ctypes.data, chunk.ctypes.data, info.ctypes.data)
         return ptr, items[:2 * ni].reshape(ni, 2), chunk[:nt], info[:3 * ni].reshape(ni, 3)
 
-    def hanging3(self):
-        """Cubes: the hanging sub-faces as the kernels take them: (pairs (n, 6):
+    def hanging3(self, first: int = 0):
+        """Cubes, their traces placed from `first` on: the hanging sub-faces as the kernels take them: (pairs (n, 6):
         trace of the larger and of the smaller side, result of either, places of
         a trace of either; sides in tile order (m, 3): element, first result,
-        number of results)."""
+        number of results; whole sides: own trace, 0)."""
         L = inspect_lib()
+        if first:
+            L.dginspect_place_traces3(self.h, first)
         cnt = np.zeros(2, dtype=np.int64)
         L.dginspect_hanging3(self.h, cnt.ctypes.data, None, None)
         pairs = np.zeros((max(int(cnt[0]), 1), 6), dtype=np.int64)

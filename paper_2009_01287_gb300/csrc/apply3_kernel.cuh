@@ -163,7 +163,7 @@ __device__ __forceinline__ void hang3_tile(const ApplyArgs& A, const HangTile& T
   };
   for (int t = tid; t < cnt * 2 * NP; t += kThreads3) {   // R along the first axis
     const int it = t / (2 * NP), rem = t - it * 2 * NP, w = rem / NP, n = rem - w * NP;
-    load(trd + 2 * ((int64_t)hp[it].src_b + n * NP) + w, 2);
+    load(trd + 2 * (hp[it].src_b + n * NP) + w, 2);
     line_restrict<NP>(v, o, A.tab + hp[it].tab_ra);
     store(sY + (it * 2 + w) * N2 + n * NP, 1);
   }
@@ -211,7 +211,7 @@ __device__ __forceinline__ void hang3_tile(const ApplyArgs& A, const HangTile& T
     load(sY + (it * 2 + w) * N2 + i, NP);
     line_restrict_t<NP>(v, o, A.tab + h.tab_rb);
     if (BR2) store(sX + it * 2 * N2 + i, NP);   // R^T J: the lifting, and c2
-    double* dst = A.tr + 2 * ((int64_t)h.dst_b + i) + (w == 0 ? 1 : 0);
+    double* dst = A.tr + 2 * (h.dst_b + i) + (w == 0 ? 1 : 0);
     const double c = w == 0 ? h.cc_b : 1.0;
 #pragma unroll
     for (int q = 0; q < NP; ++q) dst[2 * q * NP] = w == 0 ? c * o[q] : o[q];
@@ -253,7 +253,7 @@ __device__ __forceinline__ void hang3_tile(const ApplyArgs& A, const HangTile& T
     const int it = t / NP, i = t - it * NP;
     load(sY + it * 2 * N2 + i, NP);
     line_restrict_t<NP>(v, o, A.tab + hp[it].tab_rb);
-    store(A.tr + 2 * ((int64_t)hp[it].dst_b + i), 2 * NP);
+    store(A.tr + 2 * (hp[it].dst_b + i), 2 * NP);
   }
 }
 
@@ -281,10 +281,9 @@ __device__ __forceinline__ void apply3_tile(const ApplyArgs& A, const ApplyTile&
   // (diagonal in modes), hanging sides from their pairs' results, in order
   for (int t = tid; t < cnt * 6 * N2; t += kThreads3) {
     const int es = t / N2, q = t - es * N2;
-    const int2 sd = __ldg(A.side3 + (int64_t)T.first * 6 + es);   // {record, 0} or {first result, pairs}
+    const SubFaceModal3& f = A.sfm3[(int64_t)T.first * 6 + es];
     double r, c;
-    if (sd.y == 0) {
-      const SubFaceModal3& f = A.sfm3[sd.x];
+    if (f.pairs == 0) {
       const int i = q % NP, j = q / NP, nn = f.nn;
       const double2 o = __ldg(tr + f.own_off + q);
       double J = o.x, F = o.y;
@@ -297,12 +296,13 @@ __device__ __forceinline__ void apply3_tile(const ApplyArgs& A, const ApplyTile&
       r = fma(BR2 && in ? f.czx : f.cz, J, f.cf * F);
       c = f.cc * J;
     } else {
-      const double2* src = tr + sd.x + q;
-      const double2 f = __ldg(src);
-      r = f.x;
-      c = f.y;
-      for (int g = 1; g < sd.y; ++g) {
-        const double2 n = __ldg(src + g * N2);
+      const double2* src = tr + f.own_off + q;
+      const int pairs = f.pairs;
+      const double2 first = __ldg(src);
+      r = first.x;
+      c = first.y;
+      for (int g = 1; g < pairs; ++g) {
+        const double2 n = __ldg(src + (int64_t)g * N2);
         r += n.x;
         c += n.y;
       }

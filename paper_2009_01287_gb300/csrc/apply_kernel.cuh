@@ -211,7 +211,6 @@ struct ApplyArgs {
   const ElemRec3* erec3;
   const HangPair* hang3;
   const HangTile* hang_tiles;
-  const int2* side3;
   double* xm;
   int moff3[kMaxP + 1];
   const double* tab;          // basis + face tables
@@ -290,7 +289,7 @@ __device__ __forceinline__ void trace_tile(const ApplyArgs& A, const ApplyTile& 
     double2 v;
     v.x = ld_x<RO>(xk + side_node(s, i, (s & 1) ? P : 0, NP));
     v.y = sg * acc;
-    reinterpret_cast<double2*>(A.tr)[(uint32_t)el.toff + s * NP + i] = v;
+    reinterpret_cast<double2*>(A.tr)[el.toff + s * NP + i] = v;
   }
 }
 

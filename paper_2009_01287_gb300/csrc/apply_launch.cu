@@ -352,7 +352,6 @@ ApplyArgs make_apply_args(const dg_mesh& M, const double* x, double* y, Reduce r
   A.erec3 = M.d_erec3;
   A.hang3 = M.d_hang3;
   A.hang_tiles = M.d_hang_tiles;
-  A.side3 = reinterpret_cast<const int2*>(M.d_side3);
   A.xm = M.d_xm;
   for (int p = 0; p <= kMaxP; ++p) A.moff3[p] = M.moff3[p];
   A.tab = M.d_tables;

@@ -350,7 +350,7 @@ static void build_union_mesh(dg_batch* B, cudaStream_t s) {
         U.h_sfm2.push_back(g);
       }
       U.h_kind2.insert(U.h_kind2.end(), M.h_kind2.begin(), M.h_kind2.end());
-      for (int32_t t : M.h_toff3) U.h_toff3.push_back((int32_t)(t + U.n_trace2));
+      for (int64_t t : M.h_toff3) U.h_toff3.push_back(t + U.n_trace2);
       U.n_trace2 += M.n_trace2;
       DG_REQUIRE(U.n_trace2 < (1LL << 31), "too many side traces");
     }

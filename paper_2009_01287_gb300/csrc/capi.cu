@@ -70,7 +70,6 @@ void upload_tiles(dg_mesh* M, cudaStream_t s) {
   if (M->host.dim == 3) {
     M->d_sfm3 = a.upload(M->h_sfm3, s);
     M->d_erec3 = a.upload(M->h_erec3, s);
-    M->d_side3 = a.upload(M->h_side3, s);
   }
   DG_CUDA(cudaStreamSynchronize(s));
 }

@@ -135,24 +135,26 @@ struct alignas(16) SubFaceModal2 {
 // (its number of sub-faces, > 0); BR2, the smaller side of a sub-face
 enum { kSideWhole = 0, kSideSmaller = -1 };
 
-// A same-size or boundary sub-face as the kernels read it, in the Legendre
-// modes of its side (in tile order, by element of the tile and side).  With
-// J = u- - u+ and F = dn- - dn+ (both sides' outward derivatives) the residual
-// over a h is r = cz J + cf F and the normal-derivative coefficient c2 = cc J,
-// mode by mode.
+// A side of a cube as the kernels read it, in its Legendre modes (one per side,
+// in tile order).  pairs = 0: one same-size or boundary sub-face; with J = u- -
+// u+ and F = dn- - dn+ (both sides' outward derivatives) the residual over a h
+// is r = cz J + cf F and the normal-derivative coefficient c2 = cc J, mode by
+// mode.  pairs > 0: the results of so many hanging pairs, one after another
+// from own_off.  Places in the trace buffer are 64-bit: cubes of degree 1 have
+// three of them per unknown.
 struct SubFaceModal3 {
   int32_t nn;        // neighbour degree + 1, 0 on the boundary
-  int32_t nbr_off;   // the neighbour's trace (double2 units in the trace buffer)
-  int32_t own_off;   // the own trace
-  int32_t pad;
+  int32_t pairs;
+  int64_t nbr_off;   // the neighbour's trace (double2 units in the trace buffer)
+  int64_t own_off;   // the own trace
   double cz;         // SIPG: sigma area; BR2: the own lifting's factor
   double czx;        // BR2, modes both sides have: plus the neighbour lifting's
   double cf, cc;
 };
 // A sub-face between a larger and a smaller side (J, F seen from the larger).
 struct HangPair {
-  int32_t src_b, src_s;     // traces of the larger and the smaller side
-  int32_t dst_b, dst_s;     // results (r, c2) of either
+  int64_t src_b, src_s;     // traces of the larger and the smaller side (double2 units)
+  int64_t dst_b, dst_s;     // results (r, c2) of either
   int32_t tab_ra, tab_rb;   // R per tangential axis (rows of kMaxN)
   int32_t ns;               // the smaller element's degree + 1
   int32_t pad;
@@ -170,8 +172,7 @@ constexpr int hang3_doubles(int p) { return 4 * (p + 1) * (p + 1); }   // per pa
 // per element in tile order
 struct ElemRec3 {
   int64_t off;       // first DOF
-  int32_t toff;      // its side traces (double2 units; nodal squares: unsigned)
-  int32_t pad;
+  int64_t toff;      // its side traces (double2 units)
   double ah, aih;    // a h^(dim - 2), a / h
 };
 

@@ -122,18 +122,15 @@ struct dg_mesh {
   std::vector<int32_t> h_side2, h_hang2, h_hang2_tile;
   int64_t n_trace2 = 0;                 // length of the trace buffer (double2)
   std::vector<dg::SubFaceRec3> h_sf3;   // cube meshes
-  // cube meshes, for the kernels (the element records squares too):
-  // same-size and boundary sub-face records and
-  // element records in tile order, the hanging pairs and their tiles, and per
-  // (order position, side) {record, 0} or {first result, number of pairs}
+  // cube meshes, for the kernels (the element records squares too): side and
+  // element records in tile order, the hanging pairs and their tiles
   std::vector<dg::SubFaceModal3> h_sfm3;
   std::vector<dg::ElemRec3> h_erec3;
   std::vector<dg::HangPair> h_hang3;
   std::vector<dg::HangTile> h_hang_tiles;
-  std::vector<int32_t> h_side3;
   int moff3[dg::kMaxP + 1] = {0};       // modal tables of each degree in h_tables
-  std::vector<int32_t> h_toff3;         // kernels in modes: trace offset of every element (double2 units)
-  std::vector<int32_t> h_resoff3;       // per record of a hanging sub-face, the offset of its results, else -1
+  std::vector<int64_t> h_toff3;         // kernels in modes: trace offset of every element (double2 units)
+  std::vector<int64_t> h_resoff3;       // per record of a hanging sub-face, the offset of its results, else -1
   int64_t n_trace3 = 0;                 // length of the trace buffer, results included (double2)
   int64_t hang3_smem = 0;               // dynamic shared memory of the hanging pairs' kernel
   int64_t modal3_smem = 0;              // dynamic shared memory of the modes / traces kernel
@@ -206,7 +203,6 @@ struct dg_mesh {
   dg::ElemRec3* d_erec3 = nullptr;
   dg::HangPair* d_hang3 = nullptr;
   dg::HangTile* d_hang_tiles = nullptr;
-  int32_t* d_side3 = nullptr;
   double* d_xm = nullptr;       // kernels in modes: the modes of the operator's argument
   dg::MapFace* d_mface = nullptr;
   dg::MapFaceTile* d_mface_tiles = nullptr;
@@ -298,7 +294,12 @@ void modal2_stats(dg_mesh* M);
 void build_modal2_tiles(dg_mesh* M);
 // nodal squares: element records and the items' records (after the item lists)
 void build_nodal_tiles(dg_mesh* M);
-// cube meshes: degree-sorted order, tiles and their item lists
+// cube meshes: trace offsets of every element's sides from `first` on (0 but
+// for a test of places beyond 32 bits), result offsets of both sides of every
+// hanging sub-face, and the hanging pairs with their restriction tables and
+// tiles (after the records)
+void build_modal3(dg_mesh* M, int64_t first);
+// cube meshes: degree-sorted order, tiles and their records (after build_modal3)
 void build_tiles3(dg_mesh* M);
 // upload the host-built operator data (M->host.p/off/sf_ptr, h_* arrays)
 void upload_mesh(dg_mesh* M, cudaStream_t s);

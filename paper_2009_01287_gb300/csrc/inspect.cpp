@@ -199,15 +199,23 @@ void dginspect_items(void* h, int32_t* item_ptr, int32_t* items, int32_t* chunk,
   }
 }
 
+// Cubes: the traces placed from `first` on, as where a mesh of so many places
+// lies before them.
+void dginspect_place_traces3(void* h, int64_t first) {
+  dg_mesh& M = ((Inspect*)h)->mesh;
+  build_modal3(&M, first);
+  build_tiles3(&M);
+}
+
 // Cubes: the hanging sub-faces as the kernels take them.  counts = [pairs,
 // sides]; with the arrays given, per pair {trace of the larger side, of the
 // smaller, result of the larger, of the smaller, places of a larger and of a
 // smaller trace} and per side, in tile order, {element, first result, number
-// of results; 0 on a side without hanging sub-faces}.
+// of results; on a side without hanging sub-faces its own trace and 0}.
 void dginspect_hanging3(void* h, int64_t* counts, int64_t* pairs, int64_t* sides) {
   const dg_mesh& M = ((Inspect*)h)->mesh;
   counts[0] = (int64_t)M.h_hang3.size();
-  counts[1] = (int64_t)M.h_side3.size() / 2;
+  counts[1] = (int64_t)M.h_sfm3.size();
   if (!pairs || !sides) return;
   for (const HangTile& T : M.h_hang_tiles)
     for (int i = T.first; i < T.first + T.count; ++i) {
@@ -216,10 +224,9 @@ void dginspect_hanging3(void* h, int64_t* counts, int64_t* pairs, int64_t* sides
       std::copy(v, v + 6, pairs + 6 * (int64_t)i);
     }
   for (int64_t i = 0; i < counts[1]; ++i) {
-    const bool hanging = M.h_side3[2 * i + 1] > 0;
     sides[3 * i] = M.h_order[i / 6];
-    sides[3 * i + 1] = hanging ? M.h_side3[2 * i] : 0;
-    sides[3 * i + 2] = M.h_side3[2 * i + 1];
+    sides[3 * i + 1] = M.h_sfm3[i].own_off;
+    sides[3 * i + 2] = M.h_sfm3[i].pairs;
   }
 }
 

@@ -318,7 +318,7 @@ void build_modal2(dg_mesh* M) {
   int64_t at = 0;
   M->h_toff3.resize(m.n);
   for (int64_t k = 0; k < m.n; ++k) {
-    M->h_toff3[k] = (int32_t)at;
+    M->h_toff3[k] = at;
     at += 4 * (m.p[k] + 1);
   }
   M->h_kind2.assign(m.sf.size(), 0);
@@ -362,11 +362,11 @@ void build_modal2(dg_mesh* M) {
         const bool in = f.nb >= 0;
         const int len = f.t1 - f.t0;
         const double a = m.coef[k], h = M->h_h[k], half = in ? 0.5 : 1.0;
-        g.own_off = M->h_kind2[j] == 1 ? res[j] : M->h_toff3[k] + s * (m.p[k] + 1);
+        g.own_off = M->h_kind2[j] == 1 ? res[j] : (int32_t)(M->h_toff3[k] + s * (m.p[k] + 1));
         if (M->h_kind2[j] == 1) g.tab_r = table(ilog2(m.size[k] / len), (f.t0 - start(k, s)) / len);
         if (in) {
           g.nn = r.pn + 1;
-          g.nbr_off = M->h_toff3[f.nb] + f.nb_side * g.nn;
+          g.nbr_off = (int32_t)(M->h_toff3[f.nb] + f.nb_side * g.nn);
           if (M->h_kind2[j] == 2) {
             int back = -1;   // the same sub-face seen from the larger side
             for (int i = m.sf_ptr[4 * (int64_t)f.nb + f.nb_side]; i < m.sf_ptr[4 * (int64_t)f.nb + f.nb_side + 1]; ++i)
@@ -402,7 +402,7 @@ void build_nodal_tiles(dg_mesh* M) {
   DG_REQUIRE(toff[m.n] < (1LL << 32), "too many side traces");
   M->h_erec3.clear();
   for (int32_t k : M->h_order)
-    M->h_erec3.push_back({m.off[k], (int32_t)(uint32_t)toff[k], 0, m.coef[k], m.coef[k] / M->h_h[k]});
+    M->h_erec3.push_back({m.off[k], toff[k], m.coef[k], m.coef[k] / M->h_h[k]});
   M->h_face_items.clear();
   M->h_face_br2.clear();
   if (m.mapped) return;
@@ -461,7 +461,7 @@ void build_modal2_tiles(dg_mesh* M) {
     std::vector<int32_t> small;
     for (int e = 0; e < T.count; ++e) {
       const int64_t k = M->h_order[T.first + e];
-      M->h_erec3.push_back({m.off[k], M->h_toff3[k], 0, m.coef[k], m.coef[k] / M->h_h[k]});
+      M->h_erec3.push_back({m.off[k], M->h_toff3[k], m.coef[k], m.coef[k] / M->h_h[k]});
       for (int s = 0; s < 4; ++s) {
         const int32_t b = m.sf_ptr[4 * k + s], n = m.sf_ptr[4 * k + s + 1] - b;
         if (M->h_kind2[b] == 1) {

@@ -182,7 +182,6 @@ void build_tiles3(dg_mesh* M) {
   M->h_tiles.clear();
   M->h_sfm3.clear();
   M->h_erec3.clear();
-  M->h_side3.assign(12 * (size_t)m.n, 0);
   M->apply3_smem = 0;
   M->modal3_smem = 0;
   for (int64_t i = 0; i < m.n;) {
@@ -194,20 +193,19 @@ void build_tiles3(dg_mesh* M) {
     T.first = (int32_t)i;
     T.count = (int32_t)(j - i);
     for (int64_t e = 0; e < T.count; ++e) {
-      const int64_t pos = i + e;
-      const int32_t k = order[pos];
+      const int32_t k = order[i + e];
       const double a = m.coef[k], h = M->h_h[k];
-      M->h_erec3.push_back({m.off[k], M->h_toff3[k], 0, a * h, a / h});
+      M->h_erec3.push_back({m.off[k], M->h_toff3[k], a * h, a / h});
       for (int s = 0; s < 6; ++s) {
         const int b = m.sf_ptr[6 * (int64_t)k + s], c = m.sf_ptr[6 * (int64_t)k + s + 1] - b;
-        int32_t* sd = &M->h_side3[12 * pos + 2 * s];
+        SubFaceModal3 r{};
         if (M->h_resoff3[b] >= 0) {   // hanging: its results, one after another
-          sd[0] = M->h_resoff3[b];
-          sd[1] = c;
+          r.pairs = c;
+          r.own_off = M->h_resoff3[b];
+          M->h_sfm3.push_back(r);
           continue;
         }
         const SubFaceRec3& f = M->h_sf3[b];
-        SubFaceModal3 r{};
         r.own_off = M->h_toff3[k] + s * N2;
         if (f.nb >= 0) {
           r.nn = f.pn + 1;
@@ -218,7 +216,6 @@ void build_tiles3(dg_mesh* M) {
         r.czx = fs.cz + fs.cx;
         r.cf = fs.cf;
         r.cc = fs.cc;
-        sd[0] = (int32_t)M->h_sfm3.size();
         M->h_sfm3.push_back(r);
       }
     }
@@ -231,31 +228,26 @@ void build_tiles3(dg_mesh* M) {
   M->h_order = order;
 }
 
-// Trace offsets of every element's sides, result offsets of both sides of
-// every hanging sub-face, and the hanging pairs with their restriction tables
-// and tiles (after the records).
-static void build_modal3(dg_mesh* M) {
+void build_modal3(dg_mesh* M, int64_t first) {
   const HostMesh& m = M->host;
   for (int p = 1; p <= kMaxP; ++p) {
     M->moff3[p] = (int)M->h_tables.size();
     modal_tables(p, M->h_tables);
   }
   M->moff3[0] = M->moff3[1];
-  int64_t at = 0;
+  int64_t at = first;
   M->h_toff3.resize(m.n);
   for (int64_t k = 0; k < m.n; ++k) {
-    M->h_toff3[k] = (int32_t)at;
+    M->h_toff3[k] = at;
     at += 6 * (m.p[k] + 1) * (m.p[k] + 1);
-    DG_REQUIRE(at < (1LL << 31), "too many side traces");
   }
   M->h_resoff3.assign(m.sf3.size(), -1);
   for (int64_t k = 0; k < m.n; ++k)
     for (int j = m.sf_ptr[6 * k]; j < m.sf_ptr[6 * k + 6]; ++j) {
       const auto& f = m.sf3[j];
       if (f.nb < 0 || m.size[f.nb] == m.size[k]) continue;
-      M->h_resoff3[j] = (int32_t)at;
+      M->h_resoff3[j] = at;
       at += (m.p[k] + 1) * (m.p[k] + 1);
-      DG_REQUIRE(at < (1LL << 31), "too many side traces");
     }
   M->n_trace3 = at;
   std::map<std::pair<int, int>, int> index;   // (level, position) -> R
@@ -407,7 +399,7 @@ void build_mesh_host3(dg_mesh* M, const dg_mesh_desc* desc, const dg_options& o)
       r.tab_on[d] += base;
       r.tab_nn[d] += base;
     }
-  build_modal3(M);
+  build_modal3(M, 0);
   build_tiles3(M);
   // operation and byte counts of one operator apply, as the kernels do it
   dg_mesh_stats& S = M->stats;

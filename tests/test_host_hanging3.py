@@ -50,3 +50,16 @@ def test_every_pair_once(built_lib, form):
 
 def test_side_of_many_sub_faces(built_lib):
     assert _check(built_lib, beside(256, 1, 1), "sipg") == (65536, 65536)
+
+
+def test_places_beyond_32_bits(built_lib):
+    """Cubes of degree 1 have three places of traces per unknown, so a mesh the
+    32-bit unknowns admit can need 64-bit places."""
+    mesh = inputs.small_hp_mesh(1, base=3, depth=2, prob=0.3, pmax=4, dim=3)
+    hs = built_lib.HostSetup(mesh, built_lib.make_options(), amg=False)
+    pairs, sides = hs.hanging3()
+    first = 3 * (1 << 31)
+    far, far_sides = hs.hanging3(first)
+    assert np.array_equal(far[:, :4], pairs[:, :4] + first) and np.array_equal(far[:, 4:], pairs[:, 4:])
+    assert np.array_equal(far_sides[:, 1], sides[:, 1] + first)
+    assert np.array_equal(far_sides[:, [0, 2]], sides[:, [0, 2]])
