@@ -471,6 +471,8 @@ def inspect_lib():
         L.dginspect_block_units.restype = C.c_int64
         L.dginspect_csr_tiers.argtypes = [C.c_int64, vp, vp, vp, vp, vp]
         L.dginspect_csr_tiers.restype = C.c_int
+        L.dginspect_modal_tables.argtypes = [C.c_int, C.c_int, C.c_int, vp, vp]
+        L.dginspect_modal_tables.restype = C.c_int
         _inspect = L
     return _inspect
 
@@ -493,6 +495,20 @@ def plan_block_units(dims, slot, inv_off):
         raise DGError(DG_EINVAL, L.dginspect_last_error().decode())
     m = int(np.sum(unit[:n, 1][unit[:n, 3] != 0]))
     return unit[:n].copy(), ubase[:n].copy(), brec[:m].copy()
+
+
+def modal_tables(p: int, L: int = 0, o: int = 0):
+    """The host's tables of degree p in Legendre modes - node to mode of the even
+    modes (from sums of mirrored nodes) and of the odd ones (from differences),
+    1D stiffness, phi_k(1), phi_k'(1) - and the restriction of modes to the
+    o-th of 2^L parts (9 x 9)."""
+    out = np.zeros(4 * 81)
+    R = np.zeros((9, 9))
+    inspect_lib().dginspect_modal_tables(p, L, o, out.ctypes.data, R.ctypes.data)
+    n, H, HC = p + 1, (p + 1) // 2, (p + 2) // 2
+    cut = np.cumsum([HC * HC, H * H, n * n, n, n])
+    E, O, K, s, q = np.split(out[:cut[-1]], cut[:-1])
+    return E.reshape(HC, HC), O.reshape(H, H), K.reshape(n, n), s, q, R
 
 
 def plan_csr_tiers(ptr):

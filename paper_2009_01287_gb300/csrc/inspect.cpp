@@ -82,6 +82,16 @@ int dginspect_csr_tiers(int64_t rows, const int64_t* ptr, int32_t* out2, int64_t
   }
 }
 
+// The tables of a degree in modes (modal_tables) into out, (level, position)'s
+// restriction (modal_restriction) into R; returns the tables' length.
+int dginspect_modal_tables(int p, int L, int o, double* out, double* R) {
+  std::vector<double> t;
+  modal_tables(p, t);
+  std::copy(t.begin(), t.end(), out);
+  modal_restriction(L, o, R);
+  return (int)t.size();
+}
+
 void* dginspect_create(const dg_mesh_desc* desc, const dg_options* opts, int with_amg) {
   try {
     std::unique_ptr<Inspect> I(new Inspect());
