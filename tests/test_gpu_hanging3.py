@@ -16,7 +16,7 @@ def test_operator_on_a_side_of_many_sub_faces(built_lib, cuda_device, form):
     import torch
     from paper_2009_01287_gb300 import inputs
     B = built_lib
-    mesh = beside(256, 2, 1)
+    mesh = beside(256, 1, 1)
     opts = B.make_options(form=B.DG_FORM_BR2 if form == "br2" else B.DG_FORM_SIPG, eta=100.0)
     M = B.Mesh(mesh, opts)
     x = inputs.random_vector(M.n_dofs, 3)
