@@ -81,6 +81,8 @@ class Result:
 
 
 _map_tokens: dict = {}   # id -> (reference, token); an id alone is taken again after its object is gone
+_map_kept: "OrderedDict[int, tuple]" = OrderedDict()   # id -> (object, token) of objects without weak references
+_MAP_KEPT = 64   # at most so many of them are kept alive; one that comes back later gets a new token
 _map_lock = threading.Lock()
 _map_count = itertools.count()
 
@@ -89,16 +91,21 @@ def _map_token(f) -> int:
     """A number of this map object's own, never given to another."""
     with _map_lock:
         known = _map_tokens.get(id(f))
-        if known is None or known[0]() is not f:
-            try:
-                ref = weakref.ref(f)
-            except TypeError:   # takes no weak reference: kept
-                ref = lambda: f   # noqa: E731
-            known = (ref, next(_map_count))
-            _map_tokens[id(f)] = known
-            for k in [k for k, (ref, _) in _map_tokens.items() if ref() is None]:
-                del _map_tokens[k]
-        return known[1]
+        if known is not None and known[0]() is f:
+            return known[1]
+        try:
+            ref = weakref.ref(f)
+        except TypeError:
+            # no weak reference: the object itself is kept, so that its id stays its own
+            token = _map_kept.pop(id(f), (f, None))[1]
+            _map_kept[id(f)] = (f, next(_map_count) if token is None else token)
+            while len(_map_kept) > _MAP_KEPT:
+                _map_kept.popitem(last=False)
+            return _map_kept[id(f)][1]
+        for k in [k for k, (r, _) in _map_tokens.items() if r() is None]:
+            del _map_tokens[k]
+        _map_tokens[id(f)] = (ref, next(_map_count))
+        return _map_tokens[id(f)][1]
 
 
 def mesh_key(m: MeshDesc) -> str:
