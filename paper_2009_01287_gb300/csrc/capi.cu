@@ -220,16 +220,21 @@ struct PcgWork {
   unsigned* tick = nullptr;  // reduction tickets (TK_*)
   double* hsc = nullptr;     // pinned: scalars read back (SC_COUNT) + limits sent (2)
   DevArena arena;
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr;
+  cudaGraph_t graph = nullptr, graph_single = nullptr;
+  // one solve, four iterations to a pass of the while node, and one to a pass
+  cudaGraphExec_t exec = nullptr, exec_single = nullptr;
   cudaStream_t cap = nullptr;
   bool graph_failed = false;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   void drop_graph() {
-    if (exec) cudaGraphExecDestroy(exec);
-    if (graph) cudaGraphDestroy(graph);
-    exec = nullptr;
-    graph = nullptr;
+    for (cudaGraphExec_t* e : {&exec, &exec_single}) {
+      if (*e) cudaGraphExecDestroy(*e);
+      *e = nullptr;
+    }
+    for (cudaGraph_t* g : {&graph, &graph_single}) {
+      if (*g) cudaGraphDestroy(*g);
+      *g = nullptr;
+    }
   }
   ~PcgWork() {
     drop_graph();
@@ -312,24 +317,34 @@ static double pcg_start(const dg_precond* pc, PcgWork& w, const double* b, doubl
 // PCG iterations in one pass of the graph's while node.  A pass costs about
 // 3.5 us beyond its kernels (empty bodies, GB300), so four share it; the
 // iterations of a pass after the one that stopped change nothing and skip the
-// operator (on average one and a half of them, once per solve).
+// operator, but apply the preconditioner (one and a half of them on average).
+// A short solve can lose more by these than it gains: cut off after one
+// iteration, 98k unknowns took 233 us with four to a pass and 139 with one, 430k
+// on cubes 799 and 422, 576 unknowns 134 and 89; cut off after eight four are
+// faster (518 us and 561, 1.85 and 1.97 ms, 248 and 288).  So a solve takes one
+// to a pass where its limit would leave more behind than the passes cost, a
+// preconditioner apply (10 us at least) counted as three of them, or where its
+// tolerance is one that few iterations reach.  (Instead, a node for the first
+// iterations before the one of four: 40 us on every solve, 5% at 576 unknowns.)
 constexpr int kItersPerBody = 4;
+constexpr double kSingleRtol = 0.2;
+static bool one_per_pass(double rtol, int maxit) {
+  const int64_t passes = ((int64_t)maxit + kItersPerBody - 1) / kItersPerBody;
+  return rtol >= kSingleRtol || 3 * (kItersPerBody * passes - maxit) > maxit - passes;
+}
 
 // One graph for a whole solve: the start kernels, then a device-side while
-// node around one PCG iteration whose condition the kernels set.  Captured
-// once per preconditioner, on the workspace copies of b and x, with the limits
-// read from device scalars.
-static bool pcg_capture(const dg_mesh* M, const dg_precond* pc, PcgWork& w) {
-  if (w.exec) return true;
-  if (w.graph_failed) return false;
-  const char* env = std::getenv("DG_PCG_GRAPH");
-  if (env && env[0] == '0') return false;  // host-driven loop requested
+// node around `per_body` PCG iterations whose condition the kernels set.
+// Captured once per preconditioner, on the workspace copies of b and x, with
+// the limits read from device scalars.
+static bool pcg_capture_one(const dg_mesh* M, const dg_precond* pc, PcgWork& w, int per_body, cudaGraph_t& graph,
+                            cudaGraphExec_t& exec) {
   cudaGraphConditionalHandle handle = 0;
   bool ok = false;
   std::string why;
-  if (cudaGraphCreate(&w.graph, 0) == cudaSuccess &&
-      cudaGraphConditionalHandleCreate(&handle, w.graph, 0, cudaGraphCondAssignDefault) == cudaSuccess &&
-      cudaStreamBeginCaptureToGraph(w.cap, w.graph, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed) ==
+  if (cudaGraphCreate(&graph, 0) == cudaSuccess &&
+      cudaGraphConditionalHandleCreate(&handle, graph, 0, cudaGraphCondAssignDefault) == cudaSuccess &&
+      cudaStreamBeginCaptureToGraph(w.cap, graph, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed) ==
           cudaSuccess) {
     cudaGraphNodeParams cp{};
     cp.type = cudaGraphNodeTypeConditional;
@@ -360,7 +375,7 @@ static bool pcg_capture(const dg_mesh* M, const dg_precond* pc, PcgWork& w) {
       ec = cudaStreamBeginCaptureToGraph(w.cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
       if (ec == cudaSuccess) {
         try {
-          for (int u = 0; u < kItersPerBody; ++u) pcg_body(M, pc, w, w.x, -1, 0.0, handle, 1, w.cap);
+          for (int u = 0; u < per_body; ++u) pcg_body(M, pc, w, w.x, -1, 0.0, handle, 1, w.cap);
         } catch (const Error& e) {
           launched = false;
           why = e.what();
@@ -371,23 +386,31 @@ static bool pcg_capture(const dg_mesh* M, const dg_precond* pc, PcgWork& w) {
     }
     cudaError_t ei = cudaSuccess;
     if (ok) {
-      ei = cudaGraphInstantiate(&w.exec, w.graph, 0);
+      ei = cudaGraphInstantiate(&exec, graph, 0);
       ok = ei == cudaSuccess;
     }
     if (!ok && std::getenv("DG_VERBOSE"))
       std::fprintf(stderr, "dg: capture: launch [%s] capture %s instantiate %s\n", why.c_str(),
                    cudaGetErrorString(ec), cudaGetErrorString(ei));
   }
-  const cudaError_t cap_err = cudaGetLastError();
-  if (!ok) {
-    if (std::getenv("DG_VERBOSE"))
-      std::fprintf(stderr, "dg: PCG graph capture failed (%s), using the host-driven loop\n",
-                   cudaGetErrorString(cap_err));
-    w.drop_graph();
-    w.graph_failed = true;
-    return false;
-  }
-  return true;
+  if (!ok && std::getenv("DG_VERBOSE"))
+    std::fprintf(stderr, "dg: PCG graph capture failed (%s), using the host-driven loop\n",
+                 cudaGetErrorString(cudaPeekAtLastError()));
+  cudaGetLastError();
+  return ok;
+}
+
+static bool pcg_capture(const dg_mesh* M, const dg_precond* pc, PcgWork& w) {
+  if (w.exec) return true;
+  if (w.graph_failed) return false;
+  const char* env = std::getenv("DG_PCG_GRAPH");
+  if (env && env[0] == '0') return false;  // host-driven loop requested
+  if (pcg_capture_one(M, pc, w, kItersPerBody, w.graph, w.exec) &&
+      pcg_capture_one(M, pc, w, 1, w.graph_single, w.exec_single))
+    return true;
+  w.drop_graph();
+  w.graph_failed = true;
+  return false;
 }
 
 // Solve into the workspace copy of x.  solve_ms spans everything the solve
@@ -409,7 +432,7 @@ static void pcg_run(const dg_mesh* M, const dg_precond* pc, const double* b, dou
   if (b != w.b) DG_CUDA(cudaMemcpyAsync(w.b, b, w.n * sizeof(double), cudaMemcpyDeviceToDevice, s));
   DG_CUDA(cudaMemcpyAsync(w.sc + SC_MAXIT, w.hsc + SC_COUNT, 2 * sizeof(double), cudaMemcpyHostToDevice, s));
   if (use_graph) {
-    DG_CUDA(cudaGraphLaunch(w.exec, s));
+    DG_CUDA(cudaGraphLaunch(one_per_pass(rtol, maxit) ? w.exec_single : w.exec, s));
   } else if (pcg_start(pc, w, w.b, w.x, w.hsc, s) > 0.0) {
     // host-driven loop, status read back every 8 iterations
     for (int it = 0; it < maxit;) {
