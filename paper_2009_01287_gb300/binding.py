@@ -471,6 +471,10 @@ def inspect_lib():
         L.dginspect_block_units.restype = C.c_int64
         L.dginspect_csr_tiers.argtypes = [C.c_int64, vp, vp, vp, vp, vp]
         L.dginspect_csr_tiers.restype = C.c_int
+        L.dginspect_modal2_pays.argtypes = [vp, C.c_int64]
+        L.dginspect_modal2_pays.restype = C.c_int
+        L.dginspect_modal2_places.argtypes = [vp]
+        L.dginspect_modal2_places.restype = C.c_int64
         L.dginspect_modal_tables.argtypes = [C.c_int, C.c_int, C.c_int, vp, vp]
         L.dginspect_modal_tables.restype = C.c_int
         _inspect = L
@@ -495,6 +499,14 @@ def plan_block_units(dims, slot, inv_off):
         raise DGError(DG_EINVAL, L.dginspect_last_error().decode())
     m = int(np.sum(unit[:n, 1][unit[:n, 3] != 0]))
     return unit[:n].copy(), ubase[:n].copy(), brec[:m].copy()
+
+
+def modal2_pays(elems, places: int) -> bool:
+    """Whether squares with elems[p] elements of degree p (0..8) and so many
+    places of traces take the operator in modes."""
+    e = np.ascontiguousarray(elems, dtype=np.int64)
+    assert e.shape == (9,)
+    return bool(inspect_lib().dginspect_modal2_pays(e.ctypes.data, places))
 
 
 def modal_tables(p: int, L: int = 0, o: int = 0):
@@ -601,6 +613,10 @@ class HostSetup:
         info = np.zeros(3 * max(ni, 1), dtype=np.int32)
         L.dginspect_items(self.h, ptr.ctypes.data, items.ctypes.data, chunk.ctypes.data, info.ctypes.data)
         return ptr, items[:2 * ni].reshape(ni, 2), chunk[:nt], info[:3 * ni].reshape(ni, 3)
+
+    def modal2_places(self) -> int:
+        """Squares: the places of the side traces in modes."""
+        return int(inspect_lib().dginspect_modal2_places(self.h))
 
     def hanging3(self, first: int = 0):
         """Cubes, their traces placed from `first` on: the hanging sub-faces as the kernels take them: (pairs (n, 6):

@@ -273,10 +273,12 @@ static void build_union_mesh(dg_batch* B, cudaStream_t s) {
   U.eta = first.eta;
   for (int p = 0; p <= kMaxP; ++p) U.boff[p] = first.boff[p];
   // the operator's form: by all instances together
-  int64_t elems[kMaxP + 1] = {0};
-  for (int i = 0; i < B->n_inst; ++i)
-    for (int32_t p : B->meshes[i / B->n_rhs]->host.p) ++elems[p];
-  U.modal2 = modal2_pays(elems);
+  int64_t elems[kMaxP + 1] = {0}, places = 0;
+  for (auto& M : B->meshes) {
+    for (int32_t p : M->host.p) elems[p] += B->n_rhs;
+    places += B->n_rhs * modal2_places(M->host);
+  }
+  U.modal2 = modal2_pays(elems, places);
   if (U.modal2) {
     for (int p = 1; p <= kMaxP; ++p) U.tile_epb[p] = apply2_epb(p);
     const int nth = std::max(1, std::min<int>(B->n_problems, (int)std::thread::hardware_concurrency()));

@@ -283,11 +283,13 @@ void build_mesh_host(dg_mesh* M, const dg_mesh_desc* desc, const dg_options* opt
 void build_tiles(dg_mesh* M);
 // flat sub-face item lists of the tiles (square meshes; after the tiles)
 void build_face_items(dg_mesh* M);
-// Squares in modes: whether a mesh with so many elements of each degree takes
-// them, the tables of every degree, the sub-face records with their restriction
+// Squares in modes: whether a mesh with so many elements of each degree and
+// places of traces takes them, these places (of the sides, and restricted to the
+// sub-faces of larger sides), the tables of every degree, the sub-face records with their restriction
 // tables (after the SIPG records), and the tiles' element records, sides and
 // hanging items (after the tiles).
-bool modal2_pays(const int64_t (&elems)[kMaxP + 1]);
+bool modal2_pays(const int64_t (&elems)[kMaxP + 1], int64_t places);
+int64_t modal2_places(const HostMesh& m);
 void append_modal_tables(dg_mesh* M);
 void build_modal2(dg_mesh* M);
 void modal2_stats(dg_mesh* M);

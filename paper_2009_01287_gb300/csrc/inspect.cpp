@@ -82,6 +82,16 @@ int dginspect_csr_tiers(int64_t rows, const int64_t* ptr, int32_t* out2, int64_t
   }
 }
 
+// Whether squares with so many elements of each degree (0..8) and places of
+// traces take the operator in modes (modal2_pays).
+int dginspect_modal2_pays(const int64_t* elems, int64_t places) {
+  int64_t e[kMaxP + 1];
+  std::copy(elems, elems + kMaxP + 1, e);
+  return modal2_pays(e, places) ? 1 : 0;
+}
+// the places of a mesh's traces in modes (squares)
+int64_t dginspect_modal2_places(void* h) { return modal2_places(((Inspect*)h)->mesh.host); }
+
 // The tables of a degree in modes (modal_tables) into out, (level, position)'s
 // restriction (modal_restriction) into R; returns the tables' length.
 int dginspect_modal_tables(int p, int L, int o, double* out, double* R) {

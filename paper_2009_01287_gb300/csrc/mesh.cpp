@@ -295,10 +295,21 @@ void build_face_items(dg_mesh* M) {
 // 30.5 stand-alone; apply2_kernel.cuh has more).
 constexpr int64_t kModal2TilesPerSm = 6;
 
-bool modal2_pays(const int64_t (&elems)[kMaxP + 1]) {
+bool modal2_pays(const int64_t (&elems)[kMaxP + 1], int64_t places) {
+  if (places >= (1LL << 31)) return false;   // records in modes hold them in 32 bits, nodal ones do not
   int64_t tiles = 0;
   for (int p = 1; p <= kMaxP; ++p) tiles += (elems[p] + apply2_epb(p) - 1) / apply2_epb(p);
   return tiles >= kModal2TilesPerSm * 152;
+}
+
+int64_t modal2_places(const HostMesh& m) {
+  int64_t n = 0;
+  for (int64_t k = 0; k < m.n; ++k) {
+    n += 4 * (m.p[k] + 1);
+    for (int j = m.sf_ptr[4 * k]; j < m.sf_ptr[4 * k + 4]; ++j)
+      if (m.size[k] > m.sf[j].t1 - m.sf[j].t0) n += m.p[k] + 1;
+  }
+  return n;
 }
 
 void append_modal_tables(dg_mesh* M) {
@@ -672,7 +683,7 @@ void build_mesh_host(dg_mesh* M, const dg_mesh_desc* desc, const dg_options* opt
   auto halve = [&] {
     for (int p = 1; p <= kMaxP; ++p) M->tile_epb[p] = std::max(1, M->tile_epb[p] / 2);
   };
-  M->modal2 = !m.mapped && modal2_pays(elems);
+  M->modal2 = !m.mapped && modal2_pays(elems, modal2_places(m));
   if (m.mapped) {
     build_mesh_map(M, desc);   // the mapped records, tables and factors
     // fewer tiles than SMs: half the elements per tile (24k unknowns, 109 tiles:
