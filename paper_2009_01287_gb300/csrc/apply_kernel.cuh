@@ -194,13 +194,7 @@ __device__ __forceinline__ bool reduce_finalize2(double t1, double t2, const Red
 struct ApplyArgs {
   const double* x;
   double* y;
-  const int64_t* off;
-  const double* ih;           // 1 / h per element
-  const double* aih;          // a / h per element (a: the diffusion coefficient)
-  const double* ak;           // a per element
-  const int64_t* toff;        // offset of the element's side traces in tr
-  double* tr;                 // side traces: [side][node][u, dn]
-  const int32_t* sf_ptr;
+  double* tr;                 // side traces: (u, dn) per side and node
   const FaceItem* face_items; // squares, nodal
   const SubFaceBr2* face_br2; // and BR2: the multiplied-out liftings
   const SubFaceModal2* sfm2;  // squares in modes
@@ -214,23 +208,26 @@ struct ApplyArgs {
   double* xm;
   int moff3[kMaxP + 1];
   const double* tab;          // basis + face tables
-  const int32_t* order;       // degree-sorted element order
   const ApplyTile* tiles;
   const int32_t* item_ptr;    // items of tile t: [item_ptr[t], item_ptr[t + 1])
   const int2* side_items;     // per (order position, side): first item, count
-  double eta;                 // BR2 penalty
   double* dot_partial;        // optional reduction of x . y (see Reduce)
   double* dot_out;
-  unsigned* dot_ticket;
   double* pcg_sc;             // PCG scalars: with the x . y sum, alpha = (r.z) / (p.q)
   const double* skip;         // batch: tiles whose instance has skip[inst * skip_stride] != 0 are idle
   int skip_stride;
   int n_tiles;
   unsigned* sched;            // [0] next tile, [1] exit ticket (both zero between launches)
   BasisOff boff[kMaxP + 1];
-  // mapped squares: the sub-faces whose weights are formed and, per sub-face
-  // record, where a side finds them; the geometric factors at the Gauss points
-  // (volume per element, faces per record); the volume tables
+  // mapped squares: per element the first DOF, a / h and the first sub-face of
+  // every side, the elements of the tiles; the sub-faces whose weights are
+  // formed and, per sub-face record, where a side finds them; the geometric
+  // factors at the Gauss points (volume per element, faces per record); the
+  // volume tables
+  const int64_t* off;
+  const double* aih;
+  const int32_t* sf_ptr;
+  const int32_t* order;
   const MapFace* mface;
   const MapFaceTile* mface_tiles;
   const MapSide* mside;

@@ -336,10 +336,7 @@ ApplyArgs make_apply_args(const dg_mesh& M, const double* x, double* y, Reduce r
   A.x = x;
   A.y = y;
   A.off = M.d_off;
-  A.ih = M.d_ih;
   A.aih = M.d_aih;
-  A.ak = M.d_ak;
-  A.toff = M.d_toff;
   A.tr = M.d_tr;
   A.sf_ptr = M.d_sf_ptr;
   A.face_items = M.d_face_items;
@@ -359,10 +356,8 @@ ApplyArgs make_apply_args(const dg_mesh& M, const double* x, double* y, Reduce r
   A.tiles = M.d_tiles;
   A.item_ptr = M.d_item_ptr;
   A.side_items = reinterpret_cast<const int2*>(M.d_side_items);
-  A.eta = M.eta;
   A.dot_partial = red.partial;
   A.dot_out = red.out;
-  A.dot_ticket = red.ticket;
   A.pcg_sc = nullptr;
   A.skip = M.skip_status;
   A.skip_stride = M.skip_stride;

@@ -258,9 +258,12 @@ static void build_batch_tiles(dg_batch* B) {
   }
   U.h_order = order;
   U.n_tiles = (int)U.h_tiles.size();
+  if (U.modal2) {
+    build_modal2_tiles(&U);
+    return;
+  }
   build_face_items(&U);
-  if (U.modal2) build_modal2_tiles(&U);
-  else build_nodal_tiles(&U);
+  build_nodal_tiles(&U);
 }
 
 static void retile_batch(dg_mesh*, void* ctx) { build_batch_tiles((dg_batch*)ctx); }

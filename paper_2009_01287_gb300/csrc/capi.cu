@@ -48,7 +48,6 @@ void upload_tiles(dg_mesh* M, cudaStream_t s) {
   DevArena& a = M->tile_arena;
   M->apply_smem = apply_smem_for(*M);
   M->apply_grid = apply_kernel_setup(*M);
-  M->d_order = a.upload(M->h_order, s);
   M->d_tiles = a.upload(M->h_tiles, s);
   if (M->host.dim == 2) M->d_erec3 = a.upload(M->h_erec3, s);
   if (M->host.dim == 2 && !M->modal2 && !M->host.mapped) {
@@ -63,6 +62,7 @@ void upload_tiles(dg_mesh* M, cudaStream_t s) {
     M->d_hang2_tile = a.upload(M->h_hang2_tile, s);
   }
   if (M->host.mapped) {
+    M->d_order = a.upload(M->h_order, s);
     M->d_mface = a.upload(M->h_mface, s);
     M->d_mface_tiles = a.upload(M->h_mface_tiles, s);
     M->d_mside = a.upload(M->h_mside, s);
@@ -78,36 +78,27 @@ void upload_mesh(dg_mesh* M, cudaStream_t s) {
   const HostMesh& m = M->host;
   // upload
   DevArena& a = M->arena;
-  M->d_p = a.upload(m.p, s);
-  M->d_off = a.upload(m.off, s);
-  {
-    std::vector<double> ih(m.n), aih(m.n);
-    std::vector<int64_t> toff(m.n + 1, 0);
-    for (int64_t k = 0; k < m.n; ++k) {
-      ih[k] = 1.0 / M->h_h[k];
-      aih[k] = m.coef[k] / M->h_h[k];
-      const int64_t np = m.p[k] + 1;
-      toff[k + 1] = toff[k] + 8 * np;
-    }
-    M->d_ih = a.upload(ih, s);
-    M->d_aih = a.upload(aih, s);
-    M->d_ak = a.upload(m.coef, s);
-    if (m.dim == 3) {
-      M->d_tr = a.alloc<double>(2 * M->n_trace3);
-      M->d_xm = a.alloc<double>(M->n_dofs);
-      M->d_hang3 = a.upload(M->h_hang3, s);
-      M->d_hang_tiles = a.upload(M->h_hang_tiles, s);
-    } else if (M->modal2) {
-      M->d_tr = a.alloc<double>(2 * M->n_trace2);
-      M->d_xm = a.alloc<double>(M->n_dofs);
-      M->d_sfm2 = a.upload(M->h_sfm2, s);
-    } else {
-      M->d_toff = a.upload(toff, s);
-      M->d_tr = a.alloc<double>(toff[m.n]);
-    }
+  if (m.dim == 3) {
+    M->d_tr = a.alloc<double>(2 * M->n_trace3);
+    M->d_xm = a.alloc<double>(M->n_dofs);
+    M->d_hang3 = a.upload(M->h_hang3, s);
+    M->d_hang_tiles = a.upload(M->h_hang_tiles, s);
+  } else if (M->modal2) {
+    M->d_tr = a.alloc<double>(2 * M->n_trace2);
+    M->d_xm = a.alloc<double>(M->n_dofs);
+    M->d_sfm2 = a.upload(M->h_sfm2, s);
+  } else {
+    int64_t n = 0;
+    for (int32_t p : m.p) n += 8 * (p + 1);
+    M->d_tr = a.alloc<double>(n);
   }
-  M->d_sf_ptr = a.upload(m.sf_ptr, s);
+  std::vector<double> aih;   // until upload_tiles has synchronised
   if (m.mapped) {
+    aih.resize(m.n);
+    for (int64_t k = 0; k < m.n; ++k) aih[k] = m.coef[k] / M->h_h[k];
+    M->d_off = a.upload(m.off, s);
+    M->d_aih = a.upload(aih, s);
+    M->d_sf_ptr = a.upload(m.sf_ptr, s);
     M->d_mw = a.alloc<double>(M->n_mw);
     M->d_gvol = a.upload(M->h_gvol, s);
     M->d_goff = a.upload(M->h_goff, s);

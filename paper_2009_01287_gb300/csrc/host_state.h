@@ -170,7 +170,7 @@ struct dg_mesh {
   dg::BasisOff boff[dg::kMaxP + 1];
   std::vector<dg::ApplyTile> h_tiles;
   std::vector<int32_t> h_order;      // degree-sorted element order
-  // squares: the sub-face work of every tile as a flat list of
+  // nodal and mapped squares: the sub-face work of every tile as a flat list of
   // (record, tile-local side) items, and per element side (in tile order) the
   // first item and the item count
   std::vector<int32_t> h_items;       // 2 per item: record index, and (e_local * 4 + s) |
@@ -188,14 +188,12 @@ struct dg_mesh {
   dg::DevArena tile_arena;            // device copies of the tile lists (rebuilt when tuned)
   // device
   dg::DevArena arena;
-  int32_t* d_p = nullptr;
-  int64_t* d_off = nullptr;
-  double* d_ih = nullptr;       // 1 / h
-  double* d_aih = nullptr;      // a / h (normal derivatives of traces and test functions)
-  double* d_ak = nullptr;       // a
-  int64_t* d_toff = nullptr;    // side-trace offsets (8 (p+1) doubles per element)
   double* d_tr = nullptr;       // side traces written by each apply
+  // mapped squares: DOF offsets, a / h, sub-faces and element order
+  int64_t* d_off = nullptr;
+  double* d_aih = nullptr;
   int32_t* d_sf_ptr = nullptr;
+  int32_t* d_order = nullptr;
   dg::SubFaceBr2* d_face_br2 = nullptr;
   dg::SubFaceModal2* d_sfm2 = nullptr;   // squares in modes
   int32_t *d_side2 = nullptr, *d_hang2 = nullptr, *d_hang2_tile = nullptr;
@@ -214,7 +212,6 @@ struct dg_mesh {
   double* d_gbr2 = nullptr;          // mapped squares, BR2 (h_gbr2, h_g2off)
   int64_t* d_g2off = nullptr;
   double* d_tables = nullptr;
-  int32_t* d_order = nullptr;
   dg::ApplyTile* d_tiles = nullptr;
   dg::FaceItem* d_face_items = nullptr;
   int32_t* d_item_ptr = nullptr;
@@ -281,7 +278,7 @@ namespace dg {
 void build_mesh_host(dg_mesh* M, const dg_mesh_desc* desc, const dg_options* opts);
 // degree-sorted element order and operator tiles from M->host.p
 void build_tiles(dg_mesh* M);
-// flat sub-face item lists of the tiles (square meshes; after the tiles)
+// flat sub-face item lists of the tiles (nodal and mapped squares; after the tiles)
 void build_face_items(dg_mesh* M);
 // Squares in modes: whether a mesh with so many elements of each degree and
 // places of traces takes them, these places (of the sides, and restricted to the

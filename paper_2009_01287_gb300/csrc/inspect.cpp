@@ -140,10 +140,11 @@ constexpr int64_t kCubeChunk = 4096;
 struct ItemList {
   std::vector<int32_t> ptr, item, chunk;
 };
-ItemList item_list(const dg_mesh& M) {
+ItemList item_list(dg_mesh& M) {
   ItemList L;
   const HostMesh& m = M.host;
   if (m.dim == 2) {
+    if (M.h_item_ptr.empty()) build_face_items(&M);   // in modes: not kept
     L.ptr = M.h_item_ptr;
     L.item = M.h_items;
     for (int t = 0; t < M.n_tiles; ++t) L.chunk.push_back(L.ptr[t + 1] - L.ptr[t]);
@@ -186,7 +187,7 @@ ItemList item_list(const dg_mesh& M) {
 
 // the operator's tiles and sub-face items: out = [n_tiles, n_items, dim]
 void dginspect_item_sizes(void* h, int64_t* out) {
-  const dg_mesh& M = ((Inspect*)h)->mesh;
+  dg_mesh& M = ((Inspect*)h)->mesh;
   out[0] = M.n_tiles;
   out[1] = (int64_t)item_list(M).item.size() / 2;
   out[2] = M.host.dim;
@@ -197,7 +198,7 @@ void dginspect_item_sizes(void* h, int64_t* out) {
 // fields its kind depends on: interior (0/1), neighbour degree, the whole-side
 // flags (BR2 records; 0 without them)
 void dginspect_items(void* h, int32_t* item_ptr, int32_t* items, int32_t* chunk, int32_t* info) {
-  const dg_mesh& M = ((Inspect*)h)->mesh;
+  dg_mesh& M = ((Inspect*)h)->mesh;
   const ItemList L = item_list(M);
   std::copy(L.ptr.begin(), L.ptr.end(), item_ptr);
   std::copy(L.item.begin(), L.item.end(), items);

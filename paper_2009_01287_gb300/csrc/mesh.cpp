@@ -238,10 +238,13 @@ void build_tiles(dg_mesh* M) {
   }
   M->n_tiles = (int)M->h_tiles.size();
   M->h_order = order;
+  if (M->modal2) {
+    build_modal2_tiles(M);
+    return;
+  }
   build_face_items(M);
   if (m.mapped) build_map_faces(M);
-  if (M->modal2) build_modal2_tiles(M);
-  else build_nodal_tiles(M);
+  build_nodal_tiles(M);
 }
 
 void build_face_items(dg_mesh* M) {

@@ -29,3 +29,18 @@ def test_places_of_a_mesh(built_lib):
                            p=np.array([3] + [1] * 16, dtype=np.int32), extent=(8, 4), lattice_h=0.125)
     hs = built_lib.HostSetup(mesh, built_lib.make_options(), amg=False)
     assert hs.modal2_places() == 4 * 4 + 16 * 4 * 2 + 4 * 4
+
+
+def test_items_of_a_mesh_in_modes(built_lib):
+    """The nodal kernel's item lists, formed for inspection only where the
+    operator takes modes: every sub-face once."""
+    n = 912 * 3 + 1   # a strip of degree 8, three elements to a tile
+    mesh = inputs.MeshDesc(dim=2, lo=np.stack([np.arange(n), np.zeros(n)], axis=1).astype(np.int32),
+                           size=np.ones(n, dtype=np.int32), p=np.full(n, 8, dtype=np.int32), extent=(n, 1),
+                           lattice_h=1.0 / n)
+    hs = built_lib.HostSetup(mesh, built_lib.make_options(), amg=False)
+    assert built_lib.modal2_pays(_elems(8, n), hs.modal2_places())
+    ptr, items, chunk, info = hs.face_items()
+    assert np.array_equal(np.sort(items[:, 0]), np.arange(4 * n))
+    assert np.array_equal(np.diff(ptr), chunk) and ptr[-1] == 4 * n
+    assert int((info[:, 0] == 1).sum()) == 2 * (n - 1)
