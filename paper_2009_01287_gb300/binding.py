@@ -471,6 +471,8 @@ def inspect_lib():
         L.dginspect_block_units.restype = C.c_int64
         L.dginspect_csr_tiers.argtypes = [C.c_int64, vp, vp, vp, vp, vp]
         L.dginspect_csr_tiers.restype = C.c_int
+        L.dginspect_on_threads.argtypes = [C.c_int, C.c_int, vp]
+        L.dginspect_on_threads.restype = C.c_int
         L.dginspect_modal2_pays.argtypes = [vp, C.c_int64]
         L.dginspect_modal2_pays.restype = C.c_int
         L.dginspect_modal2_places.argtypes = [vp]

@@ -14,7 +14,6 @@
 #include <cmath>
 #include <cstdlib>
 #include <memory>
-#include <exception>
 #include <thread>
 
 #include "kernels.cuh"
@@ -284,25 +283,12 @@ static void build_union_mesh(dg_batch* B, cudaStream_t s) {
   U.modal2 = modal2_pays(elems, places);
   if (U.modal2) {
     for (int p = 1; p <= kMaxP; ++p) U.tile_epb[p] = apply2_epb(p);
-    const int nth = std::max(1, std::min<int>(B->n_problems, (int)std::thread::hardware_concurrency()));
-    std::vector<std::exception_ptr> errs(nth);
-    std::vector<std::thread> pool;
-    for (int t = 0; t < nth; ++t)
-      pool.emplace_back([&, t] {
-        try {
-          for (int k = t; k < B->n_problems; k += nth) {
-            dg_mesh* M = B->meshes[k].get();
-            if (M->modal2) continue;   // large enough by itself
-            build_modal2(M);
-            modal2_stats(M);
-          }
-        } catch (...) {
-          errs[t] = std::current_exception();
-        }
-      });
-    for (auto& th : pool) th.join();
-    for (auto& e : errs)
-      if (e) std::rethrow_exception(e);
+    on_threads(B->n_problems, [&](int k) {
+      dg_mesh* M = B->meshes[k].get();
+      if (M->modal2) return;   // large enough by itself
+      build_modal2(M);
+      modal2_stats(M);
+    });
   }
   // basis tables are identical in every mesh: take the first mesh's prefix
   const int basis_len = first.boff[kMaxP].d1 + kMaxP + 1;

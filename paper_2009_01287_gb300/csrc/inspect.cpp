@@ -82,6 +82,20 @@ int dginspect_csr_tiers(int64_t rows, const int64_t* ptr, int32_t* out2, int64_t
   }
 }
 
+// on_threads over n items: done[k] counts the calls of item k; item `fails`
+// throws.  Returns 1 if the exception came back.
+int dginspect_on_threads(int n, int fails, int32_t* done) {
+  try {
+    on_threads(n, [&](int k) {
+      ++done[k];
+      if (k == fails) throw Error(DG_EINVAL, "item failed");
+    });
+    return 0;
+  } catch (const Error&) {
+    return 1;
+  }
+}
+
 // Whether squares with so many elements of each degree (0..8) and places of
 // traces take the operator in modes (modal2_pays).
 int dginspect_modal2_pays(const int64_t* elems, int64_t places) {

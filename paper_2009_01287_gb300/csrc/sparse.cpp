@@ -16,8 +16,11 @@
 //              does not shrink below 0.9 n, or at kAmgMaxLevels levels; the
 //              last level is inverted densely.
 #include <algorithm>
+#include <atomic>
 #include <cstdlib>
 #include <cstdio>
+#include <exception>
+#include <mutex>
 #include <chrono>
 #include <thread>
 #include <cmath>
@@ -116,6 +119,32 @@ SerialSetup::~SerialSetup() { t_serial = prev; }
 
 int setup_threads() {
   return t_serial ? 1 : (int)std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
+}
+
+void on_threads(int n, const std::function<void(int)>& f) {
+  std::atomic<int> next{0};
+  std::mutex m;
+  std::exception_ptr first;
+  auto work = [&] {
+    for (int k; (k = next.fetch_add(1)) < n;) {
+      try {
+        f(k);
+      } catch (...) {
+        std::lock_guard<std::mutex> lock(m);
+        if (!first) first = std::current_exception();
+      }
+    }
+  };
+  std::vector<std::thread> pool;
+  const int more = std::min<int>(n, (int)std::thread::hardware_concurrency()) - 1;
+  try {
+    if (more > 0) pool.reserve(more);
+    for (int t = 0; t < more; ++t) pool.emplace_back(work);
+  } catch (const std::exception&) {
+  }
+  work();
+  for (auto& th : pool) th.join();
+  if (first) std::rethrow_exception(first);
 }
 
 Csr csr_multiply(const Csr& A, const Csr& B) {

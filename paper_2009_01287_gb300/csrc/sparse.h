@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cstdint>
+#include <functional>
 #include <vector>
 
 namespace dg {
@@ -31,6 +32,10 @@ struct SerialSetup {
 // Threads a setup step may use on this thread: 1 under SerialSetup, else the
 // hardware threads (at most 16).
 int setup_threads();
+// f(k) for every k < n, on up to n hardware threads besides this one and on this
+// one, in any order.  Where no further thread can be started the ones there are
+// do the work; the first exception of an f is thrown here once all have ended.
+void on_threads(int n, const std::function<void(int)>& f);
 
 // Deterministic smoothed-aggregation AMG hierarchy (setup only).
 struct AmgLevel {
