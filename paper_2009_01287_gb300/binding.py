@@ -473,7 +473,7 @@ def inspect_lib():
         L.dginspect_csr_tiers.restype = C.c_int
         L.dginspect_on_threads.argtypes = [C.c_int, C.c_int, vp]
         L.dginspect_on_threads.restype = C.c_int
-        L.dginspect_modal2_pays.argtypes = [vp, C.c_int64]
+        L.dginspect_modal2_pays.argtypes = [vp, C.c_int64, C.c_int]
         L.dginspect_modal2_pays.restype = C.c_int
         L.dginspect_modal2_places.argtypes = [vp]
         L.dginspect_modal2_places.restype = C.c_int64
@@ -503,12 +503,12 @@ def plan_block_units(dims, slot, inv_off):
     return unit[:n].copy(), ubase[:n].copy(), brec[:m].copy()
 
 
-def modal2_pays(elems, places: int) -> bool:
+def modal2_pays(elems, places: int, br2: bool = False) -> bool:
     """Whether squares with elems[p] elements of degree p (0..8) and so many
     places of traces take the operator in modes."""
     e = np.ascontiguousarray(elems, dtype=np.int64)
     assert e.shape == (9,)
-    return bool(inspect_lib().dginspect_modal2_pays(e.ctypes.data, places))
+    return bool(inspect_lib().dginspect_modal2_pays(e.ctypes.data, places, int(br2)))
 
 
 def modal_tables(p: int, L: int = 0, o: int = 0):

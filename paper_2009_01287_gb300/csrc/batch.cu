@@ -280,7 +280,7 @@ static void build_union_mesh(dg_batch* B, cudaStream_t s) {
     for (int32_t p : M->host.p) elems[p] += B->n_rhs;
     places += B->n_rhs * modal2_places(M->host);
   }
-  U.modal2 = modal2_pays(elems, places);
+  U.modal2 = modal2_pays(elems, places, U.opts.form == DG_FORM_BR2);
   if (U.modal2) {
     for (int p = 1; p <= kMaxP; ++p) U.tile_epb[p] = apply2_epb(p);
     on_threads(B->n_problems, [&](int k) {
@@ -289,6 +289,9 @@ static void build_union_mesh(dg_batch* B, cudaStream_t s) {
       build_modal2(M);
       modal2_stats(M);
     });
+  } else {
+    for (auto& M : B->meshes)
+      if (M->modal2) nodal2_stats(M.get());   // in modes by itself
   }
   // basis tables are identical in every mesh: take the first mesh's prefix
   const int basis_len = first.boff[kMaxP].d1 + kMaxP + 1;

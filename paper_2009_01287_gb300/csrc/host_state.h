@@ -285,11 +285,12 @@ void build_face_items(dg_mesh* M);
 // sub-faces of larger sides), the tables of every degree, the sub-face records with their restriction
 // tables (after the SIPG records), and the tiles' element records, sides and
 // hanging items (after the tiles).
-bool modal2_pays(const int64_t (&elems)[kMaxP + 1], int64_t places);
+bool modal2_pays(const int64_t (&elems)[kMaxP + 1], int64_t places, bool br2);
 int64_t modal2_places(const HostMesh& m);
 void append_modal_tables(dg_mesh* M);
 void build_modal2(dg_mesh* M);
 void modal2_stats(dg_mesh* M);
+void nodal2_stats(dg_mesh* M);
 void build_modal2_tiles(dg_mesh* M);
 // nodal squares: element records and the items' records (after the item lists)
 void build_nodal_tiles(dg_mesh* M);

@@ -98,10 +98,10 @@ int dginspect_on_threads(int n, int fails, int32_t* done) {
 
 // Whether squares with so many elements of each degree (0..8) and places of
 // traces take the operator in modes (modal2_pays).
-int dginspect_modal2_pays(const int64_t* elems, int64_t places) {
+int dginspect_modal2_pays(const int64_t* elems, int64_t places, int br2) {
   int64_t e[kMaxP + 1];
   std::copy(elems, elems + kMaxP + 1, e);
-  return modal2_pays(e, places) ? 1 : 0;
+  return modal2_pays(e, places, br2 != 0) ? 1 : 0;
 }
 // the places of a mesh's traces in modes (squares)
 int64_t dginspect_modal2_places(void* h) { return modal2_places(((Inspect*)h)->mesh.host); }

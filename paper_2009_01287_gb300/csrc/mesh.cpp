@@ -292,16 +292,27 @@ void build_face_items(dg_mesh* M) {
   }
 }
 
-// Tiles per SM from which squares take the operator in modes: below it is bound
-// by the chain of phases of a tile, longer than the nodal kernel's (98k unknowns,
-// 4.2 tiles per SM: even stand-alone, 12% behind in a solve; 6.6: 26.2 us against
-// 30.5 stand-alone; apply2_kernel.cuh has more).
+// Tiles per SM from which squares take the operator in modes; below, it is bound
+// by the chain of phases of a tile, longer than the nodal kernel's.  Whole apply
+// and PCG iteration (mixed), nodal / in modes, meshes of 82k to 320k unknowns of
+// degrees up to 2 ... 8, SIPG: 4.5 tiles per SM 24.6 / 24.2 and 58.4 / 57.3 us by
+// the nodal kernel alone; 6.1 to 6.4 tiles 15 to 28% faster applies, iterations
+// from 8% faster to 2.5% slower (67.9 / 69.5 us, 127k unknowns: the nodal traces
+// ride on the p update); 6.8 to 11.2 tiles 14 to 31% and 1 to 11% faster.
+// BR2 has seven CTAs of a tile on an SM, and just over so many tiles the last
+// ones, light but alone, set the length of the launch: from 7.6 to 8.7 tiles per
+// SM applies were up to 14% slower than nodal (50.5 / 57.5 us, 230k unknowns) and
+// 4% faster at best, iterations 5% slower to 3% faster; at 6.2 to 7.4 applies 2 to
+// 27%, at 9 to 13.5 1 to 18% faster.
 constexpr int64_t kModal2TilesPerSm = 6;
+constexpr double kModal2Br2Gap[2] = {7.5, 9.0};
 
-bool modal2_pays(const int64_t (&elems)[kMaxP + 1], int64_t places) {
+bool modal2_pays(const int64_t (&elems)[kMaxP + 1], int64_t places, bool br2) {
   if (places >= (1LL << 31)) return false;   // records in modes hold them in 32 bits, nodal ones do not
   int64_t tiles = 0;
   for (int p = 1; p <= kMaxP; ++p) tiles += (elems[p] + apply2_epb(p) - 1) / apply2_epb(p);
+  const double per_sm = (double)tiles / 152.0;
+  if (br2 && per_sm >= kModal2Br2Gap[0] && per_sm < kModal2Br2Gap[1]) return false;
   return tiles >= kModal2TilesPerSm * 152;
 }
 
@@ -504,6 +515,42 @@ void build_modal2_tiles(dg_mesh* M) {
   }
 }
 
+// operation and byte counts of one nodal apply, as the kernel does it, and the
+// largest level difference across a sub-face
+void nodal2_stats(dg_mesh* M) {
+  const HostMesh& m = M->host;
+  dg_mesh_stats& S = M->stats;
+  const bool br2 = M->opts.form == DG_FORM_BR2;
+  double fl = 0.0;
+  for (int64_t k = 0; k < m.n; ++k) {
+    const double n1 = m.p[k] + 1.0;
+    fl += 2.0 * (4.0 * n1 * n1 * n1 + 4.0 * n1 * n1 + 4.0 * n1 * n1);  // volume, own dn, gather
+    for (int j = m.sf_ptr[4 * k]; j < m.sf_ptr[4 * k + 4]; ++j) {
+      const auto& f = m.sf[j];
+      // BR2 products (SubFaceBr2): Z and X on the own trace, V and Y on the
+      // neighbour's; Z and V are not formed on the own element's whole side,
+      // Y not on the neighbour's whole side
+      const bool own_whole = m.size[k] == f.t1 - f.t0;
+      if (f.nb < 0) {
+        fl += 2.0 * (2.0 * n1 * n1);
+        if (br2 && !own_whole) fl += 2.0 * (n1 * n1);
+        continue;
+      }
+      const double nn = m.p[f.nb] + 1.0;
+      fl += 2.0 * (2.0 * n1 * n1 + 2.0 * n1 * nn);
+      if (br2) {
+        const bool nb_whole = m.size[f.nb] == f.t1 - f.t0;
+        fl += 2.0 * (n1 * n1 + (own_whole ? 0.0 : n1 * n1 + n1 * nn) + (nb_whole ? 0.0 : n1 * nn));
+      }
+      const int lg = std::abs(ilog2(m.size[k]) - ilog2(m.size[f.nb]));
+      S.max_level_gap = std::max<int64_t>(S.max_level_gap, lg);
+    }
+  }
+  S.apply_flops = fl;
+  S.apply_bytes = 16.0 * (double)M->n_dofs + (double)m.n * (4 + 8 + 8 + 4 + 16) +
+                  (double)m.sf.size() * sizeof(SubFaceRec);
+}
+
 void build_mesh_host(dg_mesh* M, const dg_mesh_desc* desc, const dg_options* opts) {
   HostMesh& m = M->host;
   dg_options o{};
@@ -686,7 +733,7 @@ void build_mesh_host(dg_mesh* M, const dg_mesh_desc* desc, const dg_options* opt
   auto halve = [&] {
     for (int p = 1; p <= kMaxP; ++p) M->tile_epb[p] = std::max(1, M->tile_epb[p] / 2);
   };
-  M->modal2 = !m.mapped && modal2_pays(elems, modal2_places(m));
+  M->modal2 = !m.mapped && modal2_pays(elems, modal2_places(m), o.form == DG_FORM_BR2);
   if (m.mapped) {
     build_mesh_map(M, desc);   // the mapped records, tables and factors
     // fewer tiles than SMs: half the elements per tile (24k unknowns, 109 tiles:
@@ -707,40 +754,11 @@ void build_mesh_host(dg_mesh* M, const dg_mesh_desc* desc, const dg_options* opt
     }
   }
   build_tiles(M);
-  // operation and byte counts of one operator apply, as the kernel does it
-  dg_mesh_stats& S = M->stats;
-  S = dg_mesh_stats{};
-  S.n_elems = m.n;
-  S.n_dofs = M->n_dofs;
-  S.n_subfaces = (int64_t)m.sf.size();
-  double fl = 0.0;
-  for (int64_t k = 0; k < m.n; ++k) {
-    const double n1 = m.p[k] + 1.0;
-    fl += 2.0 * (4.0 * n1 * n1 * n1 + 4.0 * n1 * n1 + 4.0 * n1 * n1);  // volume, own dn, gather
-    for (int j = m.sf_ptr[4 * k]; j < m.sf_ptr[4 * k + 4]; ++j) {
-      const auto& f = m.sf[j];
-      // BR2 products (SubFaceBr2): Z and X on the own trace, V and Y on the
-      // neighbour's; Z and V are not formed on the own element's whole side,
-      // Y not on the neighbour's whole side
-      const bool own_whole = m.size[k] == f.t1 - f.t0;
-      if (f.nb < 0) {
-        fl += 2.0 * (2.0 * n1 * n1);
-        if (o.form == DG_FORM_BR2 && !own_whole) fl += 2.0 * (n1 * n1);
-        continue;
-      }
-      const double nn = m.p[f.nb] + 1.0;
-      fl += 2.0 * (2.0 * n1 * n1 + 2.0 * n1 * nn);
-      if (o.form == DG_FORM_BR2) {
-        const bool nb_whole = m.size[f.nb] == f.t1 - f.t0;
-        fl += 2.0 * (n1 * n1 + (own_whole ? 0.0 : n1 * n1 + n1 * nn) + (nb_whole ? 0.0 : n1 * nn));
-      }
-      const int lg = std::abs(ilog2(m.size[k]) - ilog2(m.size[f.nb]));
-      S.max_level_gap = std::max<int64_t>(S.max_level_gap, lg);
-    }
-  }
-  S.apply_flops = fl;
-  S.apply_bytes = 16.0 * (double)M->n_dofs + (double)m.n * (4 + 8 + 8 + 4 + 16) +
-                  (double)m.sf.size() * sizeof(SubFaceRec);
+  M->stats = dg_mesh_stats{};
+  M->stats.n_elems = m.n;
+  M->stats.n_dofs = M->n_dofs;
+  M->stats.n_subfaces = (int64_t)m.sf.size();
+  nodal2_stats(M);
   if (M->modal2) modal2_stats(M);
   if (m.mapped) map_stats(M);
 }

@@ -21,6 +21,17 @@ def test_places_beyond_32_bits_stay_nodal(built_lib):
     assert not pays(_elems(1, 2 * n - 1), 8 * (2 * n - 1))
 
 
+def test_br2_just_over_a_wave_stays_nodal(built_lib):
+    """BR2 holds seven tiles on an SM: from 7.5 to 9 of them per SM the nodal
+    operator is as fast or faster.  Degree 7: four elements to a tile."""
+    pays = built_lib.modal2_pays
+    for per_sm, br2 in [(5.9, False), (6, True), (7.49, True), (7.5, False), (8, False), (8.99, False), (9, True),
+                        (20, True)]:
+        elems = _elems(7, 4 * int(np.ceil(per_sm * 152)))
+        assert pays(elems, 10 ** 6, br2=True) == br2, per_sm
+        assert pays(elems, 10 ** 6, br2=False) == (per_sm >= 6)
+
+
 def test_places_of_a_mesh(built_lib):
     """A square of edge 4 and degree 3 beside sixteen unit squares of degree 1:
     the sides' traces, and those of the large one restricted to four sub-faces."""
