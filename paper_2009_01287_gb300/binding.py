@@ -471,6 +471,8 @@ def inspect_lib():
         L.dginspect_block_units.restype = C.c_int64
         L.dginspect_csr_tiers.argtypes = [C.c_int64, vp, vp, vp, vp, vp]
         L.dginspect_csr_tiers.restype = C.c_int
+        L.dginspect_slices.argtypes = [C.c_int64, vp, vp, vp, vp, vp, vp]
+        L.dginspect_slices.restype = C.c_int
         L.dginspect_on_threads.argtypes = [C.c_int, C.c_int, vp]
         L.dginspect_on_threads.restype = C.c_int
         L.dginspect_modal2_pays.argtypes = [vp, C.c_int64, C.c_int]
@@ -501,6 +503,25 @@ def plan_block_units(dims, slot, inv_off):
         raise DGError(DG_EINVAL, L.dginspect_last_error().decode())
     m = int(np.sum(unit[:n, 1][unit[:n, 3] != 0]))
     return unit[:n].copy(), ubase[:n].copy(), brec[:m].copy()
+
+
+def plan_slices(ptr):
+    """The library's slices of a sparse matrix with row pointers `ptr`, entry j
+    of value j and column j mod 1000 (host planning only): (number of whole-CTA
+    slices, hdr (n, 4), row per slot, columns, values)."""
+    L = inspect_lib()
+    ptr = np.ascontiguousarray(ptr, dtype=np.int64)
+    n = np.zeros(4, dtype=np.int64)
+
+    def call(*arrays):
+        if L.dginspect_slices(len(ptr) - 1, ptr.ctypes.data, n.ctypes.data, *arrays) != 0:
+            raise DGError(DG_EINVAL, L.dginspect_last_error().decode())
+
+    call(None, None, None, None)
+    hdr = np.zeros((int(n[0] + n[1]) + 1, 4), dtype=np.int32)
+    row, idx, val = np.zeros(n[2] + 1, dtype=np.int32), np.zeros(n[3] + 1, dtype=np.int32), np.zeros(n[3] + 1)
+    call(hdr.ctypes.data, row.ctypes.data, idx.ctypes.data, val.ctypes.data)
+    return int(n[0]), hdr[:-1], row[:-1], idx[:-1], val[:-1]
 
 
 def modal2_pays(elems, places: int, br2: bool = False) -> bool:

@@ -82,6 +82,40 @@ int dginspect_csr_tiers(int64_t rows, const int64_t* ptr, int32_t* out2, int64_t
   }
 }
 
+// The slices of a sparse matrix with the given row pointers, entry j of value j
+// and column j mod 1000 (plan_slices, fill_slices).  sizes = [n_cta, n_warp,
+// slots, entries]; with the arrays given, hdr (4 per slice), row (per slot), idx
+// and val (per entry).  0, or -1 with the message.
+int dginspect_slices(int64_t rows, const int64_t* ptr, int64_t* sizes, int32_t* hdr, int32_t* row, int32_t* idx,
+                     double* val) {
+  try {
+    Csr C;
+    C.rows = rows;
+    C.ptr.assign(ptr, ptr + rows + 1);
+    for (int64_t j = 0; j < C.ptr[rows]; ++j) {
+      C.idx.push_back((int32_t)(j % 1000));
+      C.val.push_back((double)j);
+    }
+    const SlicePlan S = plan_slices(C);
+    sizes[0] = S.n_cta;
+    sizes[1] = S.n_warp;
+    sizes[2] = (int64_t)S.row.size();
+    sizes[3] = S.entries;
+    if (!hdr) return 0;
+    std::vector<int32_t> i;
+    std::vector<double> v;
+    fill_slices(C, S, i, v);
+    std::copy(S.hdr.begin(), S.hdr.end(), hdr);
+    std::copy(S.row.begin(), S.row.end(), row);
+    std::copy(i.begin(), i.end(), idx);
+    std::copy(v.begin(), v.end(), val);
+    return 0;
+  } catch (const std::exception& e) {
+    g_err = e.what();
+    return -1;
+  }
+}
+
 // on_threads over n items: done[k] counts the calls of item k; item `fails`
 // throws.  Returns 1 if the exception came back.
 int dginspect_on_threads(int n, int fails, int32_t* done) {
