@@ -25,6 +25,10 @@ Beside it the same line carries
                 problems, the batched form (256
                 problems x 4 right-hand sides in one launch) and a bounded
                 sample of the served form.
+The line on stdout is short (LINE_LIMIT characters): every key that names, times
+or qualifies the measurement whole, of the others the figures; --record FILE
+keeps the record with all of them.
+
 --workload hp2d-br2 | hp2d-coef | hp2d-map | hp2d-curved | hp3d | batched | serving runs one of them as
 the line.
 
@@ -235,6 +239,7 @@ def time_solves(B, ctx, M, pc, b, x, tol, steps, warmup):
 def operator_rooflines(B, ctx, M, mesh, peak_tf, peaks, three, tkey, mapped=False):
     """The operator kernel and the trace kernel, each timed alone with CUDA
     events (L2 flushed before every launch)."""
+    import numpy as np
     torch = ctx.torch
     n = M.n_dofs
     xin = torch.randn(n, dtype=torch.float64, device=ctx.dev)
@@ -249,15 +254,18 @@ def operator_rooflines(B, ctx, M, mesh, peak_tf, peaks, three, tkey, mapped=Fals
         ap.append(t.apply_ms)
     apply_ms, trace_ms = statistics.mean(ap), statistics.mean(tr)
     st = M.stats
-    separable = not (three or mapped)
-    # boxes: the tiles' kernel alone; cubes and mapped squares: with the kernels
-    # that form the modes or the sub-face weights, which share the work counted
+    modes = not (three or mapped) and B.modal2_pays(np.bincount(mesh.p, minlength=9), 0,
+                                                    M.opts.form == B.DG_FORM_BR2)
+    separable = not (three or mapped or modes)
+    # nodal boxes: the tiles' kernel alone; in modes and on mapped squares: with the
+    # kernels that form the modes or the sub-face weights, which share the work counted
     tfl = trace_flops(mesh) if separable else 0.0
     kfl = st.apply_flops - tfl
     op_ms = apply_ms if separable else apply_ms + trace_ms
     ach = kfl / (op_ms / 1e3) / 1e12
     name = ("modal3_kernel + hang3_kernel + apply3_kernel (BR2 operator on cubes, FP64)" if three else
             "trace_kernel + map_face_kernel + apply_map_kernel (SIPG operator on mapped squares, FP64)" if mapped else
+            "modal2_kernel + apply2_kernel (operator in modes, FP64)" if modes else
             "apply_kernel (SIPG operator, FP64)")
     model = ("FMAs of the kernel as formulated (x2), counted on the host from the mesh: volume 8 n^3, face "
              "terms 8 n (n + n_nb) per sub-face side, test-function normal derivatives 8 n^2 per element "
@@ -266,10 +274,10 @@ def operator_rooflines(B, ctx, M, mesh, peak_tf, peaks, three, tkey, mapped=Fals
         model = ("FMAs of the kernels as formulated (x2), counted on the host from the mesh: volume at q = p+2 "
                  "Gauss points, per sub-face and Gauss point both sides' traces and the three weights once, per "
                  "side the sums of the weights, test-function normal derivatives (n = p+1)")
-    if three:
-        model = ("FP64 operations of the three kernels (x2), counted on the host from the mesh: per line of modes "
-                 "the transforms by parity, half a stiffness product, traces and lifts, per side mode five, per "
-                 "hanging sub-face four or five restrictions")
+    if three or modes:
+        model = ("FP64 operations of the kernels (x2, a lone sum or product as well), counted on the host from the "
+                 "mesh: per line of modes the transforms by parity, half a stiffness product, traces and lifts, per "
+                 "side mode five or six, per hanging sub-face four or five restrictions")
     main = {"kernel": name, "bound": "alu", "achieved": ach, "peak": peak_tf, "unit": "TFLOP/s",
             "frac": ach / peak_tf, "traffic": traffic(tkey),
             "flops_per_launch": kfl, "launch_ms": op_ms,
@@ -281,12 +289,11 @@ def operator_rooflines(B, ctx, M, mesh, peak_tf, peaks, three, tkey, mapped=Fals
             "hbm_gbs": st.apply_bytes / (op_ms / 1e3) / 1e9,
             "hbm_frac": st.apply_bytes / (op_ms / 1e3) / 1e9 / peaks["hbm_gbs"],
             "peak_source": "FP64 FMA-chain probe (dg_fp64_fma_probe) in this run; HBM of measured"}
-    trace = {"kernel": ("modal3_kernel + hang3_kernel" if three else "trace_kernel + map_face_kernel" if mapped
+    trace = {"kernel": ("modal3_kernel + hang3_kernel" if three else "modal2_kernel" if modes else "trace_kernel + map_face_kernel" if mapped
                         else "trace_kernel"), "bound": "hbm",
              "launch_ms": trace_ms, "flops_per_launch": tfl if separable else None,
              "note": "inside PCG the traces are written by the p-update kernel, not by this kernel"}
     # side traces: read x once, write u and dn at every side node
-    import numpy as np
     npd = mesh.p.astype(np.float64) + 1.0
     side_nodes = float(np.sum(6.0 * npd ** 2 if three else 4.0 * npd))
     tb = 8.0 * n + 16.0 * side_nodes
@@ -580,6 +587,56 @@ def cpu_baseline(workload: str, seed: int, solve: bool):
 
 
 # ---------------------------------------------------------------- main line
+LINE_LIMIT = 2600   # characters of the line on stdout
+# never shortened
+CONTRACT = ("impl", "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better",
+            "scaling", "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks")
+# what a short record keeps of a nested one
+FIGURES = ("kernel", "bound", "achieved", "peak", "frac", "launch_ms", "value", "unit", "cores", "kind",
+           "iters", "iters_mixed", "iters_fp64", "rel_err_mixed", "rel_err_fp64", "time_to_tol_ms_mixed",
+           "time_to_tol_ms_fp64", "ms_per_step", "n_dofs", "instances", "p50_latency_s", "p99_latency_s", "setup_s",
+           "wall_s_with_setup", "error")
+
+
+def _short(v, depth=0):
+    """Numbers to six digits, of nested records the figures, no lists of records."""
+    if isinstance(v, float):
+        return float(f"{v:.6g}")
+    if isinstance(v, dict):
+        if depth == 0 and all(isinstance(w, dict) for w in v.values()):   # sub-lines by name
+            return {k: _short(w, 1) for k, w in v.items()}
+        return {k: _short(w, depth + 1) for k, w in v.items()
+                if (k in FIGURES or isinstance(w, (int, float))) and not isinstance(w, (dict, list))}
+    if isinstance(v, list):
+        return None if v and not isinstance(v[0], (int, float)) else [_short(w, depth + 1) for w in v]
+    return v if not isinstance(v, str) or len(v) <= 120 else v[:117] + "..."
+
+
+def short_line(out: dict) -> str:
+    """The record as one line of at most LINE_LIMIT characters (but for what the
+    contract's keys take): the other keys shortened, then the last ones left out."""
+    kept = {k: v for k, v in out.items() if k in CONTRACT}
+    rest = {}
+    for k, v in out.items():
+        if k not in kept:
+            v = _short(v)
+            if v is not None and v != {}:
+                rest[k] = v
+    if "workloads" in rest:
+        rest["workloads"] = {k: {f: w[f] for f in ("value", "time_to_tol_ms_mixed", "ms_per_step", "p99_latency_s",
+                                                   "error") if f in w} for k, w in rest["workloads"].items()}
+    while rest and len(json.dumps({**kept, **rest})) > LINE_LIMIT:
+        rest.popitem()
+    return json.dumps({**kept, **rest})
+
+
+def emit(out: dict, record: str = ""):
+    if record:
+        with open(record, "w") as f:
+            json.dump(out, f)
+    print(short_line(out))
+
+
 def run_ours(args):
     import numpy as np
     import torch
@@ -653,12 +710,9 @@ def run_ours(args):
         "time_to_tol_ms_fp64": res["time_to_tol_ms_fp64"],
         "dof_iters_per_s_fp64": ws * n * sum(it64) / t64,   # replicas: identical per rank
         "setup_s": res["setup_s"],
-        "phase_ms": res["phase_ms"],
         "e2e": {"value": ws * n * sum(it_e2e) / te, "unit": "DOF-iters/s",
                 "h2d_bytes_per_step": 8 * n, "d2h_bytes_per_step": 8 * n},
         "roofline": res["roofline"],
-        "rooflines": res["rooflines"],
-        "tiles": res["tiles"],
         "fp64_peak_tflops_measured": probe["tflops"],
         "gpu_launches": launches,
         "clocks": res["clocks"],
@@ -702,8 +756,9 @@ def run_ours(args):
         leg("batched", lambda: run_batched_leg(B, ctx, 2, 1))
         leg("serving", lambda: run_serving_leg(B, 8, 160, 200.0, 8))
         out["workloads"] = extras
+    out.update({"phase_ms": res["phase_ms"], "rooflines": res["rooflines"], "tiles": res["tiles"]})
     if rank == 0:
-        print(json.dumps(out))
+        emit(out, args.record)
     if dist:
         dist.barrier()
         dist.destroy_process_group()
@@ -719,7 +774,7 @@ def run_serving(args):
            "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
            "dtype": "f64 (outer PCG, operator) + f32 (preconditioner)", "data": "synthetic",
            "config": {"workload": leg.pop("workload")}, **{k: v for k, v in leg.items() if k != "value"}}
-    print(json.dumps(out))
+    emit(out, args.record)
 
 
 def run_batched(args):
@@ -738,7 +793,7 @@ def run_batched(args):
                       "l2": leg["l2"]},
            "iters_min_median_max": leg["iters_min_median_max"], "setup_s": leg["setup_s"], "tiles": leg["tiles"],
            "clocks": leg["clocks"]}
-    print(json.dumps(out))
+    emit(out, args.record)
 
 
 def amr_leg(B, torch, which: str, n_steps: int) -> dict:
@@ -785,7 +840,7 @@ def run_amr(args):
            "vs_baseline": None, "dtype": "f64 (outer PCG, operator) + f32 (preconditioner)", "data": "synthetic",
            "config": {"workload": leg["workload"]}, "wall_s_with_setup": leg["wall_s_with_setup"],
            "table": leg["table"], "clocks": leg["clocks"]}
-    print(json.dumps(out))
+    emit(out, args.record)
 
 
 def run_reference_amr(args):
@@ -897,6 +952,7 @@ def main():
                     help="single-mesh workloads: let dg_mesh_create tune the operator's tiles")
     ap.add_argument("--base3", type=int, default=16,
                     help="cube workload: base grid per axis (16 is the workload; smaller for profiling captures)")
+    ap.add_argument("--record", default="", help="write the whole record to this file")
     ap.add_argument("--amr-steps", type=int, default=20, help="amr workloads: refinement steps")
     ap.add_argument("--oracle-leg", action="store_true", help=argparse.SUPPRESS)
     ap.add_argument("--oracle-out", default="", help=argparse.SUPPRESS)
