@@ -404,8 +404,9 @@ def measure_single(B, ctx, mesh, rh, form, steps, warmup, peaks, peak_tf, tkey, 
     if keep_x:
         out["_x"] = (x32.cpu().numpy(), x64.cpu().numpy())
     # operator, the preconditioner's kernels (the x / r update rides its final
-    # kernel), the p update with the side traces
-    out["kernels_per_iteration"] = 1 + int(pc32.stats.kernels_per_apply) + 1
+    # kernel), the p update with the side traces (cubes and mapped squares: and the
+    # kernel of the hanging pairs or of the sub-face weights)
+    out["kernels_per_iteration"] = 1 + int(pc32.stats.kernels_per_apply) + (2 if three or mapped else 1)
     for h in (pc32, pc64, M):
         h.close()
     return out
@@ -414,6 +415,7 @@ def measure_single(B, ctx, mesh, rh, form, steps, warmup, peaks, peak_tf, tkey, 
 def run_batched_leg(B, ctx, steps, warmup, n_problems=256, n_rhs=4, fp64=False, tune=True):
     """Batched workload: many uneven problems x several right-hand sides in
     one graph launch (every instance keeps its own PCG scalars)."""
+    import numpy as np
     torch = ctx.torch
     from paper_2009_01287_gb300 import inputs
     meshes = [inputs.config3_problem(k)[0] for k in range(n_problems)]
@@ -423,8 +425,9 @@ def run_batched_leg(B, ctx, steps, warmup, n_problems=256, n_rhs=4, fp64=False, 
                   stream=ctx.stream)
     setup_s = time.perf_counter() - t0
     st = bat.stats
+    modes = B.modal2_pays(sum(np.bincount(m.p, minlength=9) for m in meshes) * n_rhs, 0)
     tiles = {"tuned": bool(st.tiles_tuned), "elements_per_tile_by_degree": list(st.tile_elems)[1:],
-             "fixed_rule": [min(16, 256 // (p + 1) ** 2) for p in range(1, 9)],
+             "fixed_rule": [32 // (p + 1) if modes else min(16, 256 // (p + 1) ** 2) for p in range(1, 9)],
              "apply_ms_fixed": st.apply_ms_fixed if st.tiles_tuned else None,
              "apply_ms_tuned": st.apply_ms_tuned if st.tiles_tuned else None}
     b = torch.empty(bat.n_dofs, dtype=torch.float64, device=ctx.dev)
