@@ -173,7 +173,10 @@ typedef struct {
   int64_t n_dofs;
   int64_t n_subfaces;     /* sub-faces counted once per side (interior ones twice) */
   int64_t max_level_gap;  /* largest log2 size ratio across a sub-face            */
-  double apply_flops;     /* FP64 flops of one dg_apply as formulated (FMA = 2)  */
+  double apply_flops;     /* FP64 flops of one dg_apply as formulated: a
+                             multiply-add counts 2; of the operator in Legendre
+                             modes (cubes, large square meshes) a lone product or
+                             sum too, which takes as long                      */
   double apply_bytes;     /* algorithmic bytes of one dg_apply: x read, y write,
                              per-element and per-sub-face records read once     */
   int64_t device_bytes;   /* device memory held by the mesh handle              */

@@ -22,12 +22,13 @@
 // 25 us on 98k unknowns, one warp working through all of a tile's sub-faces.)
 // Records, items and tables are fetched before the wait for the preceding
 // kernel: no kernel writes them.  Tiles come heaviest first.
-// For large meshes (modal2_pays); on smaller ones the chain of phases before
-// the traces costs more than the operations that the modes save.  Measured
-// (GB300), whole apply, nodal kernels / these: SIPG, degrees up to 8, 599k
-// unknowns 94.4 / 67.6 us, 289k 52.8 / 42.4, 150k 32.9 / 29.4; degrees up to 6,
-// 98k 23.5 / 23.2 (inside PCG, where the nodal traces ride on the p update, 55.9
-// / 62.7 us per iteration); degrees up to 3, 164k 32.1 / 25.5.
+// For large meshes (modal2_pays, which has both sides of its line); on smaller
+// ones the chain of phases before the traces costs more than the operations that
+// the modes save.  Measured (GB300), whole apply and mixed PCG iteration, nodal
+// kernels / these: SIPG, degrees up to 8, 648k unknowns 102.8 / 72.7 and 285 /
+// 255 us, 297k 53.1 / 43.8 and 162 / 153; degrees up to 6, 150k 29.5 / 24.6 and
+// 89.9 / 89.8, 104k (nodal by the rule) 24.6 / 24.2; degrees up to 3, 176k 35.1 /
+// 26.7 and 74.5 / 69.8; BR2, degrees up to 8, 648k 122.1 / 102.7 and 306 / 291.
 // Every sub-face is evaluated from both of its sides and every sum has a fixed
 // order: applies are bit-reproducible.
 #pragma once
@@ -186,8 +187,10 @@ __device__ __forceinline__ void side2_fetch(const ApplyArgs& A, const ApplyTile&
 // r = cz (u- - u+) + cf F, the two traces multiplied one after the other: with
 // the jump formed first the operator's rounding errors are antisymmetric
 // between the two sides, and CG's counts drift from those of the assembled
-// matrix where they depend on rounding (thousands of iterations at eta = 10^4
-// without the block solves: 8.9% fewer, 1.2% this way).
+// matrix where they depend on rounding (4,990 unknowns, eta = 10^4 without the
+// block solves, forced into modes: 4,385 iterations against 4,648 nodal, 4,601
+// this way).  The terms that need J itself - BR2's liftings - and the cubes' form
+// it first: there the counts stay within 2.5% of the nodal operator's.
 __device__ __forceinline__ double side_residual(double cz, double cf, double o, double n, double F) {
   return fma(-cz, n, fma(cz, o, cf * F));
 }

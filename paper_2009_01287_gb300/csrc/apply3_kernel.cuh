@@ -34,8 +34,8 @@
 // Measured (GB300), apply of the 16^3 hp-random workload (1.7M unknowns, BR2):
 // 689 us in nodal form with face-mass products, 350 in modes with the hanging
 // sub-faces inside the tiles, 272 with their own kernel; 79k unknowns, SIPG,
-// 62.8 / 48.6 / 33.0 us.  The FP64 operations alone are 0.218 ms on the large
-// one at the measured 1.06 TFLOP/s.
+// 62.8 / 48.6 / 33.0 us.  The FP64 operations alone (216.1 Mflop) are 0.204 ms
+// on the large one at the measured 1.06 TFLOP/s.
 // Every sum has a fixed order and there are no atomics on data: applies are
 // bit-reproducible.
 #pragma once

@@ -505,10 +505,10 @@ void launch_modal_update(const dg_mesh& M, double* p, const double* z, double* s
 
 // ============================================================== tile tuner
 // Time of one operator kernel (side traces in place) as a solve runs it:
-// kReps launches captured into a CUDA graph (graph kernel nodes carry no
-// programmatic-launch overlap, as in the PCG graph), the graph launched once
-// to warm up and then timed with CUDA events, best of kRuns, on a private
-// stream ordered after the work already queued on s.
+// kReps launches captured into a CUDA graph (programmatic edges between them, as
+// in the PCG graph), the graph launched once to warm up and then timed with CUDA
+// events, best of kRuns, on a private stream ordered after the work already
+// queued on s.
 static double time_apply_ms(const dg_mesh& M, const double* x, double* y, cudaStream_t s) {
   constexpr int kReps = 20, kRuns = 3;
   cudaStream_t ts = nullptr;
