@@ -23,10 +23,14 @@ struct DevArena {
     return (T*)p;
   }
   template <typename T>
-  T* upload(const std::vector<T>& v, cudaStream_t s) {
-    T* d = alloc<T>(v.size());
-    if (!v.empty()) DG_CUDA(cudaMemcpyAsync(d, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, s));
+  T* upload(const T* v, size_t n, cudaStream_t s) {
+    T* d = alloc<T>(n);
+    if (n > 0) DG_CUDA(cudaMemcpyAsync(d, v, n * sizeof(T), cudaMemcpyHostToDevice, s));
     return d;
+  }
+  template <typename T>
+  T* upload(const std::vector<T>& v, cudaStream_t s) {
+    return upload(v.data(), v.size(), s);
   }
   void release() {
     for (void* p : ptrs) cudaFree(p);

@@ -102,13 +102,9 @@ int dginspect_slices(int64_t rows, const int64_t* ptr, int64_t* sizes, int32_t* 
     sizes[2] = (int64_t)S.row.size();
     sizes[3] = S.entries;
     if (!hdr) return 0;
-    std::vector<int32_t> i;
-    std::vector<double> v;
-    fill_slices(C, S, i, v);
+    fill_slices(C, S, idx, val);
     std::copy(S.hdr.begin(), S.hdr.end(), hdr);
     std::copy(S.row.begin(), S.row.end(), row);
-    std::copy(i.begin(), i.end(), idx);
-    std::copy(v.begin(), v.end(), val);
     return 0;
   } catch (const std::exception& e) {
     g_err = e.what();

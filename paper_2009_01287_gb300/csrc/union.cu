@@ -12,6 +12,7 @@
 // preconditioner it would have alone.
 #include <algorithm>
 #include <cstring>
+#include <memory>
 
 #include "kernels.cuh"
 #include "precond_setup.h"
@@ -37,17 +38,17 @@ template <typename T>
 void upload_slices(DevArena& a, const Csr& C, DevSlices& D, cudaStream_t s) {
   DG_REQUIRE(C.nnz() < (1LL << 31), "matrix too large for 32-bit indices");
   const SlicePlan S = plan_slices(C);
-  std::vector<int32_t> idx;
-  std::vector<T> val;
-  fill_slices(C, S, idx, val);
+  const std::unique_ptr<int32_t[]> idx(new int32_t[S.entries]);   // all written: not cleared first
+  const std::unique_ptr<T[]> val(new T[S.entries]);
+  fill_slices(C, S, idx.get(), val.get());
   D.rows = C.rows;
   D.nnz = C.nnz();
   D.n_cta = S.n_cta;
   D.n_warp = S.n_warp;
   D.hdr = a.upload(S.hdr, s);
   D.row = a.upload(S.row, s);
-  D.idx = a.upload(idx, s);
-  D.val = a.upload(val, s);
+  D.idx = a.upload(idx.get(), S.entries, s);
+  D.val = a.upload(val.get(), S.entries, s);
 }
 
 // [A | B] row by row, B's columns shifted by `shift`

@@ -78,6 +78,15 @@ def test_rows_at_every_threshold(built_lib, rounds):
     assert narrow[narrow[:, 2] == 1, 1].max() == rounds
 
 
+def test_filled_on_several_threads(built_lib):
+    """Large enough for the entries to be written in parts, long rows among them."""
+    rng = np.random.default_rng(3)
+    lens = np.concatenate([rng.integers(0, 60, 20000), rng.integers(1025, 9000, 12)])
+    rng.shuffle(lens)
+    plan = _check(built_lib, lens.tolist())
+    assert len(plan[3]) >= 4 << 17
+
+
 @pytest.mark.parametrize("seed", [0, 1])
 def test_random_rows(built_lib, seed):
     rng = np.random.default_rng(seed)
