@@ -35,8 +35,8 @@
 // Measured (GB300): apply of the 98k-unknown hp mesh on a quadrilateral 58.9 us
 // with every tile evaluating its sub-faces itself (24 of 32 lanes active), 43.9
 // with the weights formed once (22.6 of 27.3 MFLOP; the tiles' kernel 58 -> 36
-// us, the weights' 6); PCG on 24k curved unknowns 70.3 -> 55.3 us per iteration
-// (with the other changes measured beside it).
+// us, the weights' 6) and 42.4 without spills; PCG on 24k curved unknowns 70.3 ->
+// 52.8 us per iteration (with the other changes measured beside it).
 #pragma once
 
 #include "apply_kernel.cuh"
